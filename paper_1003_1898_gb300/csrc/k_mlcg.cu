@@ -125,8 +125,9 @@ __device__ __forceinline__ void lj_stream(const LjConst<G>& K, const FillDesc& d
   uint32_t base[NC];
 #pragma unroll
   for (int c = 0; c < NC; c++) base[c] = d.state[c * d.n_rows + row];
-  uint64_t nv = d.n_per;
-  if (d.limit - row * d.pitch < nv) nv = d.limit - row * d.pitch;
+  uint64_t nv = d.n_per;   // elements of this row that are written: none past the limit
+  const uint64_t left = d.limit > row * d.pitch ? d.limit - row * d.pitch : 0;
+  if (left < nv) nv = left;
   uint32_t* out = static_cast<uint32_t*>(d.out);
   const bool vec = ((d.pitch & 3) == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
   lj_row<G, OM>(K, base, lane, out + row * d.pitch, nv, vec, d, row * d.pitch);

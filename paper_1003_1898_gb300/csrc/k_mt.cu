@@ -286,9 +286,10 @@ __device__ __forceinline__ void mt_stream(const FillDesc& d, uint64_t row, uint3
   uint32_t* orow = store ? out + row * d.pitch : nullptr;
   const uint64_t n = d.n_per;
   // Draws of this row that are written (all n unless the element limit cuts
-  // the row); the stream still advances by n.
+  // the row, none when the row lies past it); the stream still advances by n.
   uint64_t nv = n;
-  if (store && d.limit - row * d.pitch < nv) nv = d.limit - row * d.pitch;
+  const uint64_t left = d.limit > row * d.pitch ? d.limit - row * d.pitch : 0;
+  if (store && left < nv) nv = left;
   uint64_t j = 0;
   const uint32_t mti = d.pos;
   if (mti < 624 && n > 0) {  // rest of the current table
