@@ -13,6 +13,7 @@
 #include "../../include/prng.h"
 #include "common.cuh"
 #include "handle.cuh"
+#include "ranlux_tc.cuh"
 
 using namespace prng;
 
@@ -20,6 +21,12 @@ namespace {
 
 constexpr uint32_t kBlobMagic = 0x50524E47u;  // "PRNG"
 constexpr uint32_t kBlobVersion = 1u;
+
+// The launch tile of a plain fill: the caller's, or by the fill's shape.
+Tile fill_tile(const prng_state* st, const FillDesc& d) {
+  if (!tile_chosen(st->gen, st->p) && st->gen == RANLUX) return ranlux_auto_tile(d);
+  return default_tile(st->gen, st->p);
+}
 
 // n_per outputs per stream in output mode `mode`; doubles take two draws
 // each, so their fill runs the draw pipeline over 2 n_per draws.
@@ -47,7 +54,7 @@ int fill_impl(prng_state* st, void* d_out, uint64_t n_per, int mode, cudaStream_
   d.p = st->p;
   d.mode = mode;
   d.jump = 0;
-  const Tile t = default_tile(st->gen, st->p);
+  const Tile t = fill_tile(st, d);
   cudaError_t e;
   switch (st->gen) {
     case RANMAR: e = launch_fill_ranmar(d, t, s); break;
@@ -136,6 +143,8 @@ bool tile_supported(int gen, Tile t, int p = 0) {
   // RANLUX at p >= 97: also a 96-column staging tile (four delivered blocks
   // per flush), compiled for those levels only.
   if (gen == RANLUX && p >= 97 && t.threads == 64 && t.cols == 96 && t.stages == 1) return true;
+  // ... and the tensor-core form, one luxury cycle (24 delivered words) per product.
+  if (gen == RANLUX && p >= kLuxTcMinP && t.threads == 128 && t.cols == 24 && t.stages == 1) return true;
   static const Tile simple[] = {{128, 32, 1}, {128, 32, 2}, {128, 64, 1}, {256, 32, 1}};
   static const Tile mlcg[] = {{128, 128, 1}, {256, 128, 1}};
   static const Tile lux[] = {{64, 48, 1}, {128, 48, 1}, {256, 48, 1},
@@ -168,6 +177,8 @@ int lux_index(int p) {
 Tile g_tiles[13] = {{128, 128, 1}, {128, 32, 1}, {128, 128, 1}, {256, 128, 1}, {128, 48, 1},
                     {128, 624, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1},
                     {128, 48, 1}, {128, 48, 1}, {128, 48, 1}};
+// Slots whose tile the caller chose; the others' plain fills choose by shape.
+bool g_tile_chosen[13] = {};
 
 int tile_slot(int gen, int p) {
   if (gen != RANLUX) return gen;
@@ -180,6 +191,8 @@ int tile_slot(int gen, int p) {
 namespace prng {
 
 Tile default_tile(int gen, int p) { return g_tiles[tile_slot(gen, p)]; }
+
+bool tile_chosen(int gen, int p) { return g_tile_chosen[tile_slot(gen, p)]; }
 
 }  // namespace prng
 
@@ -197,6 +210,10 @@ int prng_create(prng_state** out, prng_gen_t gen, uint64_t seed, uint32_t n_stre
     if (p < 0) return PRNG_ELUXURY;
   }
   if (n_streams == 0) return PRNG_ESIZE;
+  if (g == RANLUX && lux_tables_init() != cudaSuccess) {
+    cudaGetLastError();
+    return PRNG_ECUDA;
+  }
   prng_state* st = new (std::nothrow) prng_state;
   if (st == nullptr) return PRNG_EALLOC;
   st->gen = g;
@@ -284,7 +301,7 @@ int prng_ising_fused(prng_state* st, int8_t* d_spins, uint32_t L, uint32_t colou
   q.t4 = t4;
   q.t8 = t8;
   q.vec4 = (L % 8 == 0 && (reinterpret_cast<uintptr_t>(d_spins) & 7) == 0) ? 1u : 0u;
-  const Tile t = default_tile(st->gen, st->p);
+  const Tile t = fill_tile(st, d);
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   switch (st->gen) {
@@ -356,6 +373,7 @@ int prng_get_state(prng_state* st, void* h_buf, size_t* bytes) {
     return PRNG_ESIZE;
   }
   std::vector<uint32_t> dev((size_t)n * W);
+  if (st->gen == RANLUX && lux_tc_stuck()) return PRNG_ECUDA;
   if (cudaDeviceSynchronize() != cudaSuccess ||
       cudaMemcpy(dev.data(), st->d_state, dev.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
     return PRNG_ECUDA;
@@ -432,6 +450,7 @@ int prng_set_tile(prng_gen_t gen, uint32_t luxury, uint32_t threads, uint32_t co
   const Tile t{(int)threads, (int)cols, (int)stages};
   if (!tile_supported(g, t, p)) return PRNG_EUNSUPPORTED;
   g_tiles[tile_slot(g, p)] = t;
+  g_tile_chosen[tile_slot(g, p)] = true;
   return PRNG_OK;
 }
 

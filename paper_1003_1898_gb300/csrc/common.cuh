@@ -95,6 +95,7 @@ cudaError_t launch_skip_mlcg(int gen, uint32_t* state, uint64_t n, uint64_t k,
                              cudaStream_t s);
 
 Tile default_tile(int gen, int p);
+bool tile_chosen(int gen, int p);   // by prng_set_tile
 
 // SplitMix64 (Steele, Lea, Flood 2014): gamma increment, then mix64.
 __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {

@@ -1,7 +1,10 @@
 // k_ranlux.cu -- RANLUX entry points (Section 3.6; Appendix A, "RANLUX"):
 // dispatch on the luxury p to the launchers compiled per level (the standard
 // p = 24, 48, 97, 223, 389 and the planar scheme's p = 120, 240, 408).
+#include <algorithm>
+
 #include "ranlux.cuh"
+#include "ranlux_tc.cuh"
 
 namespace prng {
 
@@ -14,8 +17,36 @@ PRNG_RANLUX_DECLARE(120)
 PRNG_RANLUX_DECLARE(240)
 PRNG_RANLUX_DECLARE(408)
 
+// The tensor-core form costs the same per block at every p, the borrow chain p
+// steps.  Cycles per block of each on a busy SM, from fills of 256 to 131,072
+// streams: the chain's latency (4.9 per step and about 590 for the block's
+// output) while its warps have a scheduler each, 4.25 per step and 280 per warp
+// of the busiest scheduler beyond; the product's round trip (1,250 and 365 per
+// tile of 128 streams on the SM, four tiles at a time).  Setting the product up
+// costs about 6,500 cycles more than starting a chain.  65,536 x 4,096 u32 (us,
+// chain / product): p = 97 230 / 234, 120 258 / 233, 223 405 / 234, 389 640 /
+// 233; 4,096 x 4,096: p = 223 138 / 133, 389 202 / 133; 4,096 x 32: 13 / 16.
+// Fused half-sweeps go through the ring form of the product, whose short rows
+// pay off later (4096^2 over 65,536 streams, 128 draws each, p = 223: 50 / 55;
+// over 4,096, 2,048 draws each, p = 389: 550 / 470).
+Tile ranlux_auto_tile(const FillDesc& d) {
+  const uint64_t nb = d.n_per / 24, sched = 4 * (uint64_t)sm_count();
+  const uint64_t p = (uint64_t)d.p;
+  if (d.p >= kLuxTcMinP) {
+    const uint64_t warps = ((d.n_rows + 31) / 32 + sched - 1) / sched;
+    const uint64_t tiles = ((d.n_rows + 127) / 128 + sched / 4 - 1) / (sched / 4);
+    const uint64_t chain = std::max<uint64_t>((49 * p + 5900) / 10, warps * ((17 * p + 1120) / 4));
+    const uint64_t tc = (tiles <= 4 ? 1250 + 365 * tiles : 675 * tiles) * 106 / 100;
+    const uint64_t setup = d.mode == OUT_ISING ? 40000 : 6500;
+    if (chain > tc && nb * (chain - tc) > setup) return Tile{128, 24, 1};
+  }
+  if (ranlux_ring_ok(d) || d.p < 97) return Tile{64, 56, 1};
+  return Tile{64, 96, 1};
+}
+
 cudaError_t launch_fill_ranlux(const FillDesc& d, Tile t, cudaStream_t s) {
   if (d.n_rows == 0 || d.n_per == 0) return cudaSuccess;
+  if (t.cols == 24 && d.p >= kLuxTcMinP) return launch_fill_ranlux_tc(d, s);
   switch (d.p) {
     case 24: return ranlux_fill_p<24>(d, t, s);
     case 48: return ranlux_fill_p<48>(d, t, s);
