@@ -198,8 +198,11 @@ typedef struct prng_batch prng_batch;
 
 /* Plan a batch.  Copies the request list (handles must stay alive and must
  * not be destroyed before the batch); allocates the work items, two
- * descriptor buffers and the work counters.  PRNG_EBLOB if a handle appears
- * twice. */
+ * descriptor buffers and the work counters.  RANLUX fills at p >= 97 are cut
+ * into items of 32 streams and, when they are long, of part of their draws,
+ * whose start states the plan holds too (76 bytes per stream and part; without
+ * room for them these fills take the serial form).  PRNG_EBLOB if a handle
+ * appears twice. */
 int prng_batch_create(prng_batch **out, const prng_fill_req *reqs, uint32_t n_reqs);
 
 /* Run the batch once on `stream` (asynchronous).  Every handle's position
@@ -219,7 +222,9 @@ void prng_batch_destroy(prng_batch *b);
 /* A batched-fill engine for request sets that change from launch to launch
  * (a serving loop's ticks).  It owns a ring of staging slots, each sized for
  * max_requests requests and max_items work items (work items as for
- * prng_batch_create).  prng_batcher_launch plans the given requests into
+ * prng_batch_create; RANLUX streams are cut into parts only where the slot has
+ * room for the items, and the parts' start states come from the library's
+ * stream-ordered pool).  prng_batcher_launch plans the given requests into
  * the next slot, copies them to the device and launches the same family
  * kernels as a batch, on `stream`, asynchronously; a slot is reused once the
  * launch that last used it has completed (the call waits for that on the
@@ -344,7 +349,10 @@ int prng_calib_swb(uint32_t chains, uint32_t warps_per_sm, uint32_t iters, uint3
  * (RANMAR: 97, MT19937: 624) and staging buffers (1 or 2; for MT19937 the
  * streams per warp: 1, or 2 on half a warp each).  Set by the
  * autotuner; only the combinations compiled into the library are accepted
- * (PRNG_EUNSUPPORTED otherwise).  Not thread-safe against concurrent fills. */
+ * (PRNG_EUNSUPPORTED otherwise).  RANLUX at p >= 97 also takes 128, 24, 1 (the
+ * tensor-core form) and 128, 24, 2 (the same, long streams cut into parts, whose
+ * start states come from the library's stream-ordered pool); until a tile is
+ * set, RANLUX fills choose theirs by shape.  Not thread-safe against concurrent fills. */
 int prng_set_tile(prng_gen_t gen, uint32_t luxury, uint32_t threads, uint32_t cols,
                   uint32_t stages);
 int prng_get_tile(prng_gen_t gen, uint32_t luxury, uint32_t *threads, uint32_t *cols,

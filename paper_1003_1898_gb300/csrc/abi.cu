@@ -143,8 +143,10 @@ bool tile_supported(int gen, Tile t, int p = 0) {
   // RANLUX at p >= 97: also a 96-column staging tile (four delivered blocks
   // per flush), compiled for those levels only.
   if (gen == RANLUX && p >= 97 && t.threads == 64 && t.cols == 96 && t.stages == 1) return true;
-  // ... and the tensor-core form, one luxury cycle (24 delivered words) per product.
-  if (gen == RANLUX && p >= kLuxTcMinP && t.threads == 128 && t.cols == 24 && t.stages == 1) return true;
+  // ... and the tensor-core form, one luxury cycle (24 delivered words) per
+  // product; with stages = 2 long streams may be cut into segments.
+  if (gen == RANLUX && p >= kLuxTcMinP && t.threads == 128 && t.cols == 24 &&
+      (t.stages == 1 || t.stages == 2)) return true;
   static const Tile simple[] = {{128, 32, 1}, {128, 32, 2}, {128, 64, 1}, {256, 32, 1}};
   static const Tile mlcg[] = {{128, 128, 1}, {256, 128, 1}};
   static const Tile lux[] = {{64, 48, 1}, {128, 48, 1}, {256, 48, 1},

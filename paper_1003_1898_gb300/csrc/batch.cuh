@@ -18,6 +18,8 @@ struct BatchReq {
   FillDesc d;
   uint64_t seed;       // re-seed base (if reseed)
   int32_t gen, reseed;
+  uint32_t tiles;      // RANLUX on the tensor cores: the output has a tensor map
+  uint32_t pad;
 };
 
 // Rows [row0, row0 + rows) of request req.

@@ -15,8 +15,7 @@
 #include <vector>
 
 #include "../../include/prng.h"
-#include "batch.cuh"
-#include "handle.cuh"
+#include "plan.cuh"
 
 using namespace prng;
 
@@ -38,7 +37,10 @@ struct prng_batch {
   BatchItem* d_items = nullptr;
   uint32_t fam_off[FAM_COUNT] = {};
   uint32_t fam_n[FAM_COUNT] = {};
-  Tile fam_tile[FAM_COUNT] = {};
+  ItemPlan plan;
+  CUtensorMap* d_maps = nullptr;              // outputs of the tensor-core RANLUX requests
+  std::vector<uint8_t> tiles;                 //   and which of the requests have one
+  uint32_t* d_starts[FAM_COUNT] = {};         // their segment starts
   Buffers buf[2];
   int next = 0;
   cudaStream_t cap = nullptr;
@@ -60,7 +62,9 @@ void destroy_batch(prng_batch* b) {
     if (u.d_counters) cudaFree(u.d_counters);
   }
   if (b->d_items) cudaFree(b->d_items);
+  if (b->d_maps) cudaFree(b->d_maps);
   for (int f = 0; f < FAM_COUNT; f++) {
+    if (b->d_starts[f]) cudaFree(b->d_starts[f]);
     if (b->branch[f]) cudaStreamDestroy(b->branch[f]);
     if (b->join[f]) cudaEventDestroy(b->join[f]);
   }
@@ -88,16 +92,7 @@ cudaError_t capture(prng_batch* b, Buffers& u) {
     if (b->fam_n[f] == 0) continue;
     cudaStream_t s = b->branch[f];
     cudaStreamWaitEvent(s, b->fork, 0);
-    const BatchQueue q = queue(f);
-    const Tile t = b->fam_tile[f];
-    const bool f32 = is_f32_family(f);
-    switch (kind_of(f)) {
-      case FAM_MLCG: launch_batch_mlcg(q, t, s); break;
-      case FAM_XOR128: launch_batch_xor128(q, t, f32, s); break;
-      case FAM_RANMAR: launch_batch_ranmar(q, t, f32, s); break;
-      case FAM_MT: launch_batch_mt(q, t, f32, s); break;
-      default: launch_batch_ranlux(q, lux_p_of(f), t, f32, s); break;
-    }
+    launch_family(f, queue(f), b->plan, b->d_maps, b->d_starts[f], s);
     cudaEventRecord(b->join[f], s);
     used[nused++] = f;
   }
@@ -141,41 +136,66 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
   b->reqs.assign(reqs, reqs + n_reqs);
   cudaGetDevice(&b->device);
 
-  // Work items per family, longest rows first.
-  std::vector<std::vector<BatchItem>> items(FAM_COUNT);
-  std::vector<std::vector<uint64_t>> cost(FAM_COUNT);
-  for (int f = 0; f < FAM_COUNT; f++) {
-    b->fam_tile[f] = tile_of(f);
-  }
-  for (uint32_t i = 0; i < n_reqs; i++) {
-    const prng_fill_req& r = reqs[i];
-    const prng_state* st = r.st;
-    if (r.reseed) {
-      for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 256) {
-        const uint32_t rows = (uint32_t)std::min<uint64_t>(256, st->n_streams - r0);
-        items[FAM_SEED].push_back(BatchItem{i, rows, r0});
-        cost[FAM_SEED].push_back(0);
+  std::vector<CUtensorMap> maps;
+  std::vector<BatchItem> all;
+  // Work items per family, longest rows first; RANLUX on the tensor cores when
+  // there is room for its segments' starts.
+  auto plan_items = [&]() {
+    std::vector<std::vector<BatchItem>> items(FAM_COUNT);
+    std::vector<std::vector<uint64_t>> cost(FAM_COUNT);
+    b->plan.choose(reqs, n_reqs, true);
+    b->tiles.assign(n_reqs, 0);
+    maps.clear();
+    all.clear();
+    for (uint32_t i = 0; i < n_reqs; i++) {
+      const prng_fill_req& r = reqs[i];
+      const prng_state* st = r.st;
+      if (r.reseed) {
+        for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 256) {
+          const uint32_t rows = (uint32_t)std::min<uint64_t>(256, st->n_streams - r0);
+          items[FAM_SEED].push_back(BatchItem{i, rows, r0});
+          cost[FAM_SEED].push_back(0);
+        }
+      }
+      if (r.n_per_stream == 0) continue;
+      const int kind = family_of(st->gen, st->p);
+      const int f = (r.f32 && kind != FAM_MLCG) ? kind + FAM_F32 : kind;  // MLCG mixes dtypes
+      b->plan.items(f, i, st, r.n_per_stream, [&](const BatchItem& it) {
+        items[f].push_back(it);
+        cost[f].push_back(b->plan.cost(f, r.n_per_stream) * (kind == FAM_MLCG || kind == FAM_MT ? it.rows : 1));
+      });
+      if (b->plan.is_lux_tc(f)) {
+        if (maps.empty()) maps.resize(n_reqs);
+        b->tiles[i] = request_map(r, &maps[i]) ? 1 : 0;
       }
     }
-    if (r.n_per_stream == 0) continue;
-    const int kind = family_of(st->gen, st->p);
-    const int f = (r.f32 && kind != FAM_MLCG) ? kind + FAM_F32 : kind;  // MLCG mixes dtypes
-    const uint32_t per = rows_per_item(f, b->fam_tile[f]);
-    for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per) {
-      const uint32_t rows = (uint32_t)std::min<uint64_t>(per, st->n_streams - r0);
-      items[f].push_back(BatchItem{i, rows, r0});
-      cost[f].push_back(r.n_per_stream * (kind == FAM_MLCG || kind == FAM_MT ? rows : 1));
+    for (int f = 0; f < FAM_COUNT; f++) {
+      std::vector<size_t> order(items[f].size());
+      for (size_t k = 0; k < order.size(); k++) order[k] = k;
+      std::stable_sort(order.begin(), order.end(),
+                       [&](size_t a, size_t c) { return cost[f][a] > cost[f][c]; });
+      b->fam_off[f] = (uint32_t)all.size();
+      b->fam_n[f] = (uint32_t)order.size();
+      for (size_t k : order) all.push_back(items[f][k]);
     }
-  }
-  std::vector<BatchItem> all;
-  for (int f = 0; f < FAM_COUNT; f++) {
-    std::vector<size_t> order(items[f].size());
-    for (size_t k = 0; k < order.size(); k++) order[k] = k;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](size_t a, size_t c) { return cost[f][a] > cost[f][c]; });
-    b->fam_off[f] = (uint32_t)all.size();
-    b->fam_n[f] = (uint32_t)order.size();
-    for (size_t k : order) all.push_back(items[f][k]);
+  };
+  auto alloc_starts = [&]() {
+    for (int f = 0; f < FAM_COUNT; f++)
+      if (b->plan.is_lux_tc(f) && b->fam_n[f] > 0 &&
+          cudaMalloc(&b->d_starts[f], lux_start_bytes(b->fam_n[f])) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+      }
+    return true;
+  };
+  plan_items();
+  if (!alloc_starts()) {
+    for (auto& p : b->d_starts) {
+      if (p) cudaFree(p);
+      p = nullptr;
+    }
+    b->plan.tensor = false;
+    plan_items();
   }
 
   int rc = PRNG_OK;
@@ -185,6 +205,11 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
       cudaMemcpy(b->d_items, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice) !=
           cudaSuccess)
     rc = PRNG_ECUDA;
+  if (rc == PRNG_OK && !maps.empty()) {
+    if (cudaMalloc(&b->d_maps, n_reqs * sizeof(CUtensorMap)) != cudaSuccess) rc = PRNG_EALLOC;
+    else if (cudaMemcpy(b->d_maps, maps.data(), n_reqs * sizeof(CUtensorMap), cudaMemcpyHostToDevice) != cudaSuccess)
+      rc = PRNG_ECUDA;
+  }
   for (auto& u : b->buf) {
     if (rc != PRNG_OK) break;
     if (cudaMallocHost(&u.h_reqs, n_reqs * sizeof(BatchReq)) != cudaSuccess ||
@@ -238,6 +263,7 @@ int prng_batch_launch(prng_batch* b, void* stream) {
     q.seed = r.seed;
     q.gen = st->gen;
     q.reseed = r.reseed ? 1 : 0;
+    q.tiles = b->tiles[i];
     st->pos = advance_pos(st->gen, q.d.pos, r.n_per_stream);
   }
   if (u.exec == nullptr) {

@@ -15,8 +15,8 @@
 #include <vector>
 
 #include "../../include/prng.h"
-#include "batch.cuh"
-#include "handle.cuh"
+#include "plan.cuh"
+#include "scratch.cuh"
 
 using namespace prng;
 
@@ -27,8 +27,10 @@ constexpr int kSlots = 4;
 struct Slot {
   BatchReq* h_reqs = nullptr;     // pinned
   BatchItem* h_items = nullptr;   // pinned
+  CUtensorMap* h_maps = nullptr;  // pinned; outputs of the tensor-core RANLUX requests
   BatchReq* d_reqs = nullptr;
   BatchItem* d_items = nullptr;
+  CUtensorMap* d_maps = nullptr;
   uint32_t* d_counters = nullptr;
   cudaEvent_t done = nullptr;
   bool pending = false;
@@ -43,6 +45,7 @@ struct prng_batcher {
   Slot slot[kSlots];
   int next = 0;
   std::vector<const prng_state*> handles;   // duplicate check, sized once
+  std::vector<uint32_t> order;              // requests, longest rows first
 };
 
 namespace {
@@ -54,6 +57,8 @@ void destroy_batcher(prng_batcher* b) {
     if (u.done) cudaEventDestroy(u.done);
     if (u.h_reqs) cudaFreeHost(u.h_reqs);
     if (u.h_items) cudaFreeHost(u.h_items);
+    if (u.h_maps) cudaFreeHost(u.h_maps);
+    if (u.d_maps) cudaFree(u.d_maps);
     if (u.d_reqs) cudaFree(u.d_reqs);
     if (u.d_items) cudaFree(u.d_items);
     if (u.d_counters) cudaFree(u.d_counters);
@@ -75,6 +80,7 @@ int prng_batcher_create(prng_batcher** out, uint32_t max_requests, uint64_t max_
   b->max_items = max_items;
   try {
     b->handles.reserve(max_requests);
+    b->order.reserve(max_requests);
   } catch (...) {
     delete b;
     return PRNG_EALLOC;
@@ -82,6 +88,8 @@ int prng_batcher_create(prng_batcher** out, uint32_t max_requests, uint64_t max_
   for (auto& u : b->slot) {
     if (cudaMallocHost(&u.h_reqs, max_requests * sizeof(BatchReq)) != cudaSuccess ||
         cudaMallocHost(&u.h_items, max_items * sizeof(BatchItem)) != cudaSuccess ||
+        cudaMallocHost(&u.h_maps, max_requests * sizeof(CUtensorMap)) != cudaSuccess ||
+        cudaMalloc(&u.d_maps, max_requests * sizeof(CUtensorMap)) != cudaSuccess ||
         cudaMalloc(&u.d_reqs, max_requests * sizeof(BatchReq)) != cudaSuccess ||
         cudaMalloc(&u.d_items, max_items * sizeof(BatchItem)) != cudaSuccess ||
         cudaMalloc(&u.d_counters, FAM_COUNT * sizeof(uint32_t)) != cudaSuccess) {
@@ -103,26 +111,36 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
   if (n_reqs == 0) return PRNG_OK;
   if (reqs == nullptr) return PRNG_ENULL;
   if (n_reqs > b->max_requests) return PRNG_ESIZE;
-  uint64_t fam_n[FAM_COUNT] = {};
   for (uint32_t i = 0; i < n_reqs; i++) {
     const prng_fill_req& r = reqs[i];
     if (r.st == nullptr) return PRNG_ENULL;
     if (r.n_per_stream > 0 && r.d_out == nullptr) return PRNG_ENULL;
     if ((reinterpret_cast<uintptr_t>(r.d_out) & 3) != 0) return PRNG_ESIZE;
     if (r.n_per_stream > 0 && r.st->n_streams > UINT64_MAX / r.n_per_stream) return PRNG_ESIZE;
-    if (r.reseed) fam_n[FAM_SEED] += (r.st->n_streams + 255) / 256;
-    if (r.n_per_stream > 0) {
-      const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
-      const uint32_t per = rows_per_item(f, tile_of(f));
-      fam_n[f] += (r.st->n_streams + per - 1) / per;
-    }
   }
-  uint64_t total = 0;
+  // Items per family: RANLUX streams cut into segments where the slot has room
+  // for them, whole otherwise.
+  ItemPlan plan;
+  uint64_t fam_n[FAM_COUNT], total = 0;
   uint32_t fam_off[FAM_COUNT];
-  for (int f = 0; f < FAM_COUNT; f++) {
-    fam_off[f] = (uint32_t)std::min<uint64_t>(total, b->max_items);
-    total += fam_n[f];
-  }
+  auto count = [&](bool cut) {
+    plan.choose(reqs, n_reqs, cut);
+    std::fill(fam_n, fam_n + FAM_COUNT, 0);
+    for (uint32_t i = 0; i < n_reqs; i++) {
+      const prng_fill_req& r = reqs[i];
+      if (r.reseed) fam_n[FAM_SEED] += (r.st->n_streams + 255) / 256;
+      if (r.n_per_stream == 0) continue;
+      const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
+      fam_n[f] += plan.count(f, r.st, r.n_per_stream);
+    }
+    total = 0;
+    for (int f = 0; f < FAM_COUNT; f++) {
+      fam_off[f] = (uint32_t)std::min<uint64_t>(total, b->max_items);
+      total += fam_n[f];
+    }
+    return total <= b->max_items;
+  };
+  if (!count(true)) count(false);
   if (total > b->max_items) return PRNG_ESIZE;
   // A handle may appear once per launch (its streams advance once): sorted
   // copy of the handles, adjacent equal ones rejected.
@@ -136,6 +154,19 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
     if (cudaEventSynchronize(u.done) != cudaSuccess) return PRNG_ECUDA;
     u.pending = false;
   }
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  uint32_t* starts = nullptr;   // of the RANLUX segments, for this launch
+  uint64_t lux_items = 0;
+  for (int f = 0; f < FAM_COUNT; f++)
+    if (plan.is_lux_tc(f)) lux_items += fam_n[f];
+  if (lux_items > 0 &&
+      scratch_alloc(reinterpret_cast<void**>(&starts), lux_start_bytes(lux_items), s) != cudaSuccess) {
+    cudaGetLastError();
+    starts = nullptr;
+    plan.tensor = false;        // no room: the borrow chain, with no more items than uncut streams
+    count(false);
+  }
+  bool maps = false;
   uint32_t at[FAM_COUNT];
   std::memcpy(at, fam_off, sizeof(at));
   for (uint32_t i = 0; i < n_reqs; i++) {
@@ -163,46 +194,55 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
             BatchItem{i, (uint32_t)std::min<uint64_t>(256, st->n_streams - r0), r0};
     if (r.n_per_stream > 0) {
       const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
-      const uint32_t per = rows_per_item(f, tile_of(f));
-      for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per)
-        u.h_items[at[f]++] = BatchItem{i, (uint32_t)std::min<uint64_t>(per, st->n_streams - r0), r0};
+      if (plan.is_lux_tc(f)) {
+        q.tiles = request_map(r, &u.h_maps[i]) ? 1 : 0;
+        maps = true;
+      }
     }
   }
-  for (int f = FAM_MLCG; f < FAM_COUNT; f++) {  // longest rows first within a family
-    const bool per_row = kind_of(f) == FAM_MLCG || kind_of(f) == FAM_MT;
-    std::sort(u.h_items + fam_off[f], u.h_items + fam_off[f] + fam_n[f],
-              [&](const BatchItem& a, const BatchItem& c) {
-                const uint64_t ca = u.h_reqs[a.req].d.n_per * (per_row ? a.rows : 1);
-                const uint64_t cc = u.h_reqs[c.req].d.n_per * (per_row ? c.rows : 1);
-                return ca > cc;
-              });
+  // Items, the requests with the longest rows first (a request's items all cost
+  // the same but for the last, so ordering the requests orders the items).
+  b->order.clear();
+  for (uint32_t i = 0; i < n_reqs; i++)
+    if (reqs[i].n_per_stream > 0) b->order.push_back(i);
+  std::sort(b->order.begin(), b->order.end(), [&](uint32_t x, uint32_t y) {
+    return reqs[x].n_per_stream != reqs[y].n_per_stream ? reqs[x].n_per_stream > reqs[y].n_per_stream : x < y;
+  });
+  for (uint32_t i : b->order) {
+    const prng_fill_req& r = reqs[i];
+    const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
+    plan.items(f, i, r.st, r.n_per_stream, [&](const BatchItem& it) { u.h_items[at[f]++] = it; });
   }
-  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  auto fail = [&](int rc) {
+    cudaGetLastError();
+    if (starts != nullptr) scratch_free(starts, s);
+    return rc;
+  };
   if (cudaMemcpyAsync(u.d_reqs, u.h_reqs, n_reqs * sizeof(BatchReq), cudaMemcpyHostToDevice, s) !=
           cudaSuccess ||
       (total > 0 && cudaMemcpyAsync(u.d_items, u.h_items, total * sizeof(BatchItem),
                                     cudaMemcpyHostToDevice, s) != cudaSuccess) ||
-      cudaMemsetAsync(u.d_counters, 0, FAM_COUNT * sizeof(uint32_t), s) != cudaSuccess) {
-    cudaGetLastError();
-    return PRNG_ECUDA;
-  }
+      (maps && cudaMemcpyAsync(u.d_maps, u.h_maps, n_reqs * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s) !=
+                   cudaSuccess) ||
+      cudaMemsetAsync(u.d_counters, 0, FAM_COUNT * sizeof(uint32_t), s) != cudaSuccess)
+    return fail(PRNG_ECUDA);
   auto queue = [&](int f) {
     return BatchQueue{u.d_reqs, u.d_items + fam_off[f], (uint32_t)fam_n[f], u.d_counters + f};
   };
   cudaError_t e = launch_batch_seed(queue(FAM_SEED), s);
+  uint64_t lux_at = 0;
   for (int f = FAM_MLCG; f < FAM_COUNT && e == cudaSuccess; f++) {
     if (fam_n[f] == 0) continue;
-    const BatchQueue q = queue(f);
-    const bool f32 = f >= FAM_KINDS;
-    switch (kind_of(f)) {
-      case FAM_MLCG: e = launch_batch_mlcg(q, tile_of(f), s); break;
-      case FAM_XOR128: e = launch_batch_xor128(q, tile_of(f), f32, s); break;
-      case FAM_RANMAR: e = launch_batch_ranmar(q, tile_of(f), f32, s); break;
-      case FAM_MT: e = launch_batch_mt(q, tile_of(f), f32, s); break;
-      default: e = launch_batch_ranlux(q, lux_p_of(f), tile_of(f), f32, s); break;
+    uint32_t* st = nullptr;
+    if (plan.is_lux_tc(f)) {
+      st = starts + lux_start_bytes(lux_at) / sizeof(uint32_t);
+      lux_at += fam_n[f];
     }
+    e = launch_family(f, queue(f), plan, u.d_maps, st, s);
   }
-  if (e != cudaSuccess || cudaEventRecord(u.done, s) != cudaSuccess) return PRNG_ECUDA;
+  if (e != cudaSuccess) return fail(PRNG_ECUDA);
+  if (starts != nullptr && scratch_free(starts, s) != cudaSuccess) return PRNG_ECUDA;
+  if (cudaEventRecord(u.done, s) != cudaSuccess) return PRNG_ECUDA;
   u.pending = true;
   b->next = (b->next + 1) % kSlots;
   return PRNG_OK;

@@ -23,30 +23,48 @@ PRNG_RANLUX_DECLARE(408)
 // output) while its warps have a scheduler each, 4.25 per step and 280 per warp
 // of the busiest scheduler beyond; the product's round trip (1,250 and 365 per
 // tile of 128 streams on the SM, four tiles at a time).  Setting the product up
-// costs about 6,500 cycles more than starting a chain.  65,536 x 4,096 u32 (us,
-// chain / product): p = 97 230 / 234, 120 258 / 233, 223 405 / 234, 389 640 /
-// 233; 4,096 x 4,096: p = 223 138 / 133, 389 202 / 133; 4,096 x 32: 13 / 16.
-// Fused half-sweeps go through the ring form of the product, whose short rows
-// pay off later (4096^2 over 65,536 streams, 128 draws each, p = 223: 50 / 55;
-// over 4,096, 2,048 draws each, p = 389: 550 / 470).
+// costs about 6,500 cycles more than starting a chain, cutting streams into
+// segments 30,000 (a second kernel, the segments' starts) plus a product per
+// segment up to 16 and about four per segment filled.  Measured in us, chain /
+// product / segments: 65,536 x 4,096 u32 at p = 97 230 / 234 / -, p = 120 258 /
+// 233, 223 405 / 234, 389 640 / 233; 4,096 x 4,096 at p = 223 139 / 133 / 52;
+// 16,384 x 4,096 143 / 136 / 99; 256 x 8,192 265 / 249 / 43; 16,384 x 1,024 47 /
+// 46 / 48; 32,768 x 1,024 68 / 53 / 65; 1,024 x 1,024 45 / 45 / 37; 4,096 x 248
+// 20 / 22 / 35.  Fused half-sweeps go through the ring form of the product,
+// whose short rows pay off later (4096^2 over 65,536 streams, 128 draws each, p =
+// 223: 50 / 55; over 4,096, 2,048 draws each, p = 389: 550 / 470).
 Tile ranlux_auto_tile(const FillDesc& d) {
-  const uint64_t nb = d.n_per / 24, sched = 4 * (uint64_t)sm_count();
-  const uint64_t p = (uint64_t)d.p;
-  if (d.p >= kLuxTcMinP) {
-    const uint64_t warps = ((d.n_rows + 31) / 32 + sched - 1) / sched;
-    const uint64_t tiles = ((d.n_rows + 127) / 128 + sched / 4 - 1) / (sched / 4);
-    const uint64_t chain = std::max<uint64_t>((49 * p + 5900) / 10, warps * ((17 * p + 1120) / 4));
-    const uint64_t tc = (tiles <= 4 ? 1250 + 365 * tiles : 675 * tiles) * 106 / 100;
-    const uint64_t setup = d.mode == OUT_ISING ? 40000 : 6500;
-    if (chain > tc && nb * (chain - tc) > setup) return Tile{128, 24, 1};
+  Tile t = ranlux_ring_ok(d) || d.p < 97 ? Tile{64, 56, 1} : Tile{64, 96, 1};
+  if (d.p < kLuxTcMinP || d.n_per < 24) return t;
+  const uint64_t nb = d.n_per / 24, p = (uint64_t)d.p, sms = (uint64_t)sm_count();
+  auto product = [&](uint64_t tiles) {   // cycles of a product with `tiles` tiles to run
+    const uint64_t c = (tiles + sms - 1) / sms;
+    return (c <= 4 ? 1250 + 365 * c : 675 * c) * 106 / 100;
+  };
+  const uint64_t warps = (d.n_rows + 31) / 32, tiles = (d.n_rows + 127) / 128;
+  const uint64_t per_sched = (warps + 4 * sms - 1) / (4 * sms);
+  uint64_t best = nb * std::max<uint64_t>((49 * p + 5900) / 10, per_sched * ((17 * p + 1120) / 4));
+  auto offer = [&](uint64_t cycles, Tile tile) {
+    if (cycles < best) {
+      best = cycles;
+      t = tile;
+    }
+  };
+  offer((d.mode == OUT_ISING ? 40000 : 6500) + nb * product(tiles), Tile{128, 24, 1});
+  const LuxSplit sp = lux_split(warps * nb, nb);
+  if (sp.cut && d.mode != OUT_ISING && nb < 1ull << 40) {
+    const uint64_t B = 1ull << sp.lgb, segs = (nb + B - 1) / B, slots = 16 * sms;
+    const uint64_t rounds = (warps * segs + slots - 1) / slots;
+    offer(30000 + std::min<uint64_t>(segs, 16) * product(std::min<uint64_t>(tiles, 4 * sms)) +
+              rounds * (B + 4) * product(std::min<uint64_t>((warps * segs + 3) / 4, 4 * sms)),
+          Tile{128, 24, 2});
   }
-  if (ranlux_ring_ok(d) || d.p < 97) return Tile{64, 56, 1};
-  return Tile{64, 96, 1};
+  return t;
 }
 
 cudaError_t launch_fill_ranlux(const FillDesc& d, Tile t, cudaStream_t s) {
   if (d.n_rows == 0 || d.n_per == 0) return cudaSuccess;
-  if (t.cols == 24 && d.p >= kLuxTcMinP) return launch_fill_ranlux_tc(d, s);
+  if (t.cols == 24 && d.p >= kLuxTcMinP) return launch_fill_ranlux_tc(d, t.stages == 2, s);
   switch (d.p) {
     case 24: return ranlux_fill_p<24>(d, t, s);
     case 48: return ranlux_fill_p<48>(d, t, s);

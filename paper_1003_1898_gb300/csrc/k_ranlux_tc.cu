@@ -32,17 +32,19 @@
 #include <utility>
 #include <vector>
 
-#include <cuda.h>
-
 #include "ranlux_tc.cuh"
+#include "scratch.cuh"
 #include "tc.cuh"
 
 namespace prng {
 
 namespace {
 
-constexpr int kLevels = 8;
-constexpr int kLevelP[kLevels] = {24, 48, 97, 223, 389, 120, 240, 408};
+constexpr int kLevels = 6;   // p >= kLuxTcMinP
+constexpr int kLevelP[kLevels] = {97, 223, 389, 120, 240, 408};
+// Operands per level: 2^i luxury cycles, i < kPowers (0: the fill's own; the
+// others move a segment's start along its stream).
+constexpr int kPowers = 24;
 
 constexpr int kNK = 80;                       // K and N of the product: 72 bytes, constants, padding
 constexpr int kTabBytes = kNK * kNK * 2;      // the f16 operand, in core-matrix order
@@ -52,8 +54,8 @@ constexpr uint32_t kMagic = 0x3F000000u;      // pattern of 2^23 x 2^-24
 
 constexpr int kTmemCols = 128, kColD = 0, kColA = 80;
 
-// One operand per luxury level (filled on a device's first RANLUX handle).
-__device__ uint4 g_tab[kLevels][kTabBytes / 16];
+// Filled on a device's first RANLUX handle (1.8 MB).
+__device__ uint4 g_tab[kLevels][kPowers][kTabBytes / 16];
 // Set when a kernel gave up waiting for the tensor core (never seen).
 __device__ uint32_t g_stuck;
 
@@ -209,14 +211,17 @@ cudaError_t lux_tables_init() {
       c >>= 32;
     }
     const Big binv = mod_m(v);
-    host.resize((size_t)kLevels * kTabBytes / 2);
+    host.resize((size_t)kLevels * kPowers * kTabBytes / 2);
     for (int l = 0; l < kLevels; l++) {
       Big a = one, s = binv;
       for (int k = kLevelP[l]; k; k >>= 1) {
         if (k & 1) a = mul_m(a, s);
         s = mul_m(s, s);
       }
-      build_tab(a, host.data() + (size_t)l * kTabBytes / 2);
+      for (int i = 0; i < kPowers; i++) {
+        build_tab(a, host.data() + (size_t)(l * kPowers + i) * kTabBytes / 2);
+        a = mul_m(a, a);
+      }
     }
   }
   e = cudaMemcpyToSymbol(g_tab, host.data(), host.size() * 2);
@@ -475,31 +480,38 @@ struct TcTable {
   uint32_t tmem;
 };
 
-// The digits of N as this thread's A operand, then one product for the CTA's
-// 128 rows; `bad` (any thread's) ends it.  Returns false when the CTA gives up.
-__device__ __forceinline__ bool lux_issue(TcTable& sh, uint32_t tm, const uint32_t (&N)[18], bool bad) {
+// The digits of N as this thread's A operand (before the CTA barrier that
+// precedes the product).
+__device__ __forceinline__ void lux_digits(uint32_t tm, const uint32_t (&N)[18]) {
   uint32_t A[36];
 #pragma unroll
   for (int i = 0; i < 18; i++) {
     A[2 * i] = __byte_perm(N[i], 0, 0x4140);
     A[2 * i + 1] = __byte_perm(N[i], 0, 0x4342);
   }
-  const uint32_t wl = (threadIdx.x >> 5) << 21;      // this warp's TMEM lanes
-  tc::st36(tm + wl + kColA, A);
+  tc::st36(tm + ((threadIdx.x >> 5) << 21) + kColA, A);   // this warp's TMEM lanes
   tc::fence_before_sync();
-  if (__syncthreads_or(bad)) return false;
-  if (threadIdx.x < 32) {
-    if (tc::elect_one()) {
-      tc::fence_after_sync();
-      const uint32_t b = tc::smem_addr(sh.tab);
+}
+
+// Warp 0, after that barrier: the product of the CTA's 128 rows.
+__device__ __forceinline__ void lux_product(TcTable& sh, uint32_t tm) {
+  if (tc::elect_one()) {
+    tc::fence_after_sync();
+    const uint32_t b = tc::smem_addr(sh.tab);
 #pragma unroll
-      for (int s = 0; s < kNK / 16; s++)
-        tc::mma_f16_ts(tm + kColD, tm + kColA + 8 * s, tc::smem_desc(b + 2 * s * kKStep, kKStep, kRStep),
-                       tc::idesc_f16_f32(128, kNK), s > 0);
-      tc::mma_commit(&sh.bar);
-    }
-    __syncwarp();
+    for (int s = 0; s < kNK / 16; s++)
+      tc::mma_f16_ts(tm + kColD, tm + kColA + 8 * s, tc::smem_desc(b + 2 * s * kKStep, kKStep, kRStep),
+                     tc::idesc_f16_f32(128, kNK), s > 0);
+    tc::mma_commit(&sh.bar);
   }
+  __syncwarp();
+}
+
+// Both, when no thread is `bad`; false when the CTA gives up.
+__device__ __forceinline__ bool lux_issue(TcTable& sh, uint32_t tm, const uint32_t (&N)[18], bool bad) {
+  lux_digits(tm, N);
+  if (__syncthreads_or(bad)) return false;
+  if (threadIdx.x < 32) lux_product(sh, tm);
   return true;
 }
 
@@ -586,12 +598,26 @@ __device__ __forceinline__ void lux_store(const FillDesc& d, uint64_t row, bool 
   d.state[24 * d.n_rows + row] = c;
 }
 
-// TMEM, barrier and operand of the CTA (visible after the next CTA barrier).
-__device__ __forceinline__ void lux_setup(TcTable& sh, int level) {
+// Operand `power` of the level into shared memory (visible to the tensor core
+// after the next CTA barrier).
+__device__ __forceinline__ void lux_operand(TcTable& sh, int level, int power) {
+  for (int i = threadIdx.x; i < kTabBytes / 16; i += 128) sh.tab[i] = g_tab[level][power][i];
+  tc::fence_smem_to_async();
+}
+
+// TMEM and barrier of the CTA (visible after the next CTA barrier).
+__device__ __forceinline__ void lux_setup(TcTable& sh) {
   if (threadIdx.x < 32) tc::tmem_alloc(&sh.tmem, kTmemCols);
   if (threadIdx.x == 0) tc::mbar_init(&sh.bar, 1);
-  for (int i = threadIdx.x; i < kTabBytes / 16; i += 128) sh.tab[i] = g_tab[level][i];
-  tc::fence_smem_to_async();
+}
+// All threads: release the TMEM after every product has been taken.
+__device__ __forceinline__ void lux_teardown(uint32_t tm) {
+  tc::fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    tc::fence_after_sync();
+    tc::tmem_free(tm, kTmemCols);
+  }
 }
 
 // h steps on the state, through 24 words of shared scratch.
@@ -664,7 +690,8 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tiles(const FillDesc d, 
 
   uint32_t V[24], c;
   lux_state(d, row, active, V, c);
-  lux_setup(sh, level);
+  lux_setup(sh);
+  lux_operand(sh, level, 0);
 
   const LuxPlan plan(d);
   TileOut<OM> to{boxes[wi], (uint32_t)(lane * 128 + ((lane & 7) << 4)), &map, (uint32_t)wrow0, wrow0 < nr, 0};
@@ -741,12 +768,7 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tiles(const FillDesc d, 
     to.release((uint32_t)((d.n_per + kBox - 1) / kBox));
   }
   if (lane == 0) tc::tile_store_wait_read();
-  tc::fence_before_sync();
-  __syncthreads();
-  if (wi == 0) {
-    tc::fence_after_sync();
-    tc::tmem_free(tm, kTmemCols);
-  }
+  lux_teardown(tm);
 }
 
 // The same for any output (unaligned rows, the fused half-sweep, host memory)
@@ -767,7 +789,8 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int
 
   uint32_t V[24], c;
   lux_state(d, row, active, V, c);
-  lux_setup(sh, level);
+  lux_setup(sh);
+  lux_operand(sh, level, 0);
 
   const LuxPlan plan(d);
   uint64_t fpos = 0;   // draws of the row written out
@@ -890,12 +913,328 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int
     lux_finish(d, row, active, N, R, plan.m, reinterpret_cast<uint32_t*>(sh.tab) + 25 * tid,
                    [&](uint64_t k, uint32_t prev, uint32_t x) { emit(fpos + k, prev, x); });
   }
+  lux_teardown(tm);
+}
+
+// ------------------------------------------------- segments and batched fills
+//
+// A stream whose blocks one thread would walk for long is cut into segments of B
+// = 2^lgb blocks, each a row of its own: k_lux_starts walks the segments' starts
+// along their streams, B cycles per product, and k_lux_items fills the segments.
+// The first kernel alone reads the streams' states and the second's last segments
+// alone write them, so no row waits for another.  A work item is the 32 streams
+// of one warp in one segment; the four warps of a CTA work on different items, of
+// one request or several, and share each product.  A request's items lie segment
+// after segment, all its streams in each.
+//
+// k_lux_starts takes the segments in groups of 16, each group's first start by
+// products with 2^i x 16 B cycles for the bits of its number (a row keeps a
+// product when its bit is set), the others one after the other: every segment's
+// start by its own bits, with a state load, a head and an operand load per
+// segment, took longer than it saved above 4,096 streams (65,536 x 256: 55 us
+// against 31 uncut).
+
+// Starts of an item: words N[18] and the zero flag, 32 streams side by side.
+constexpr uint32_t kStartWords = 19 * 32;
+
+struct LuxItem {
+  uint32_t seg;
+  uint64_t row0;
+  const CUtensorMap* map;   // of its output, or nullptr
+};
+
+constexpr int kLgGroup = 4, kGroup = 1 << kLgGroup;
+
+__device__ __forceinline__ uint32_t lux_segment(const LuxJob& job, uint32_t it) {
+  return job.reqs != nullptr ? job.items[it].rows : it / job.warps;
+}
+
+// Item `it` and its fill (into `sd`, this warp's copy).
+__device__ __forceinline__ LuxItem lux_item(const LuxJob& job, uint32_t it, FillDesc* sd) {
+  const int lane = threadIdx.x & 31;
+  LuxItem I;
+  __syncwarp();
+  if (job.reqs != nullptr) {
+    const BatchItem b = job.items[it];
+    I.seg = b.rows;
+    I.row0 = b.row0;
+    I.map = job.reqs[b.req].tiles ? job.maps + b.req : nullptr;
+    load_desc(sd, job.reqs[b.req].d, lane, 32);
+  } else {
+    I.seg = it / job.warps;
+    I.row0 = 32ull * (it - I.seg * job.warps);
+    I.map = job.tiles ? &job.map : nullptr;
+    load_desc(sd, job.one, lane, 32);
+  }
+  __syncwarp();
+  return I;
+}
+
+__global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ LuxJob job, int level) {
+  __shared__ __align__(128) TcTable sh;
+  __shared__ uint32_t scratch[128 * 25];
+  __shared__ FillDesc descs[4];
+  const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+  const uint32_t it = blockIdx.x * 4 + wi;
+  const uint32_t seg = it < job.n_items ? lux_segment(job, it) : 1u;
+  const bool have = seg % kGroup == 0;
+  if (!__syncthreads_or(have)) return;
+  lux_setup(sh);
+
+  uint32_t N[18];
+  uint32_t cnt = 0, warps = 0;   // segments of this group; items from one to the next
+  bool zero = false;
+  if (have) {
+    const FillDesc& d = descs[wi];
+    const LuxItem I = lux_item(job, it, &descs[wi]);
+    const uint64_t row = I.row0 + lane;
+    const bool active = row < d.n_rows;
+    const LuxPlan plan(d);
+    const uint64_t segs = job.max_seg > 0 ? ((d.n_per / 24 + (1ull << job.lgb) - 1) >> job.lgb) : 1;
+    cnt = segs > seg + kGroup ? kGroup : segs > seg ? (uint32_t)(segs - seg) : 1u;
+    warps = (uint32_t)((d.n_rows + 31) / 32);
+    uint32_t V[24], c;
+    lux_state(d, row, active, V, c);
+    uint32_t* out = static_cast<uint32_t*>(d.out);
+    lux_head(V, c, plan.h, scratch + 25 * tid, [&](uint64_t k, uint32_t prev, uint32_t x) {
+      const uint64_t e = row * d.pitch + k;
+      if (seg != 0 || !active || e >= d.limit) return;   // the first group writes the head
+      if (d.mode == OUT_F64) {
+        if (k & 1) st_pair<24>(out + e - 1, prev, x);
+      } else {
+        st_out(out + e, d.mode == OUT_F32 ? tc_conv<OUT_F32>(x) : x);
+      }
+    });
+    if (plan.nb == 0 && plan.m == 0) lux_store(d, row, active, V, c);   // ends inside the open block
+    lux_load(V, c, N, zero);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 18; i++) N[i] = d_word(i);
+  }
   tc::fence_before_sync();
   __syncthreads();
-  if (wi == 0) {
-    tc::fence_after_sync();
-    tc::tmem_free(tm, kTmemCols);
+  tc::fence_after_sync();
+  const uint32_t tm = sh.tmem;
+  lux_constants(tm);
+  bool ok = true;
+  uint32_t products = 0;
+  // To the group's first segment, by the bits of its number.
+  const uint32_t group = have ? seg / kGroup : 0;
+  for (int i = 0; __syncthreads_or((group >> i) != 0); i++) {
+    const bool take = (group >> i) & 1u;
+    if (!__syncthreads_or(take)) continue;          // also: the operand is not in use any more
+    lux_operand(sh, level, job.lgb + kLgGroup + i);
+    if (!lux_issue(sh, tm, N, !ok)) break;
+    uint32_t T[18];
+    ok = lux_take(sh, tm, products & 1u, T) && ok;
+    products++;
+    if (take) {
+#pragma unroll
+      for (int k = 0; k < 18; k++) N[k] = T[k];
+    }
   }
+  // Segment after segment.
+  if (__syncthreads_or(cnt > 1)) lux_operand(sh, level, job.lgb);
+  for (uint32_t j = 0;; j++) {
+    if (j < cnt) {
+      uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords + lane;
+#pragma unroll
+      for (int k = 0; k < 18; k++) st[32 * k] = N[k];
+      st[32 * 18] = zero ? 1u : 0u;
+    }
+    if (!__syncthreads_or(j + 1 < cnt) || !lux_issue(sh, tm, N, !ok)) break;
+    ok = lux_take(sh, tm, products & 1u, N) && ok;
+    products++;
+  }
+  if (!ok) atomicExch(&g_stuck, 1u);
+  lux_teardown(tm);
+}
+
+// A warp's 32 rows of one segment: staging tiles as TileOut's, but any range of
+// a tile can leave on its own, word by word, when it is cut by the segment's
+// ends or the request's limit, or when the rows are not 16-byte aligned.
+struct SegOut {
+  uint8_t* box;
+  const CUtensorMap* map;   // of the limit's whole rows; nullptr: word by word
+  uint32_t rowb;
+  uint32_t off;             // element of the row at tile 0, word 0
+  uint32_t lo;              // first word of the segment in its first tile
+  uint64_t whole;           // rows before the one that the request's limit cuts
+  uint64_t done, pos;       // tiles left behind / words staged, counted from `off`
+
+  __device__ __forceinline__ uint32_t at(uint32_t chunk) const {
+    return rowb ^ ((chunk & 7u) << 4) ^ ((chunk & 8u) << 9);
+  }
+  __device__ __forceinline__ void put4(uint32_t q, uint4 v) const {
+    *reinterpret_cast<uint4*>(box + at((uint32_t)(pos >> 2) + q)) = v;
+  }
+  __device__ __forceinline__ void acquire() const {
+    if ((threadIdx.x & 31) == 0) tc::tile_store_wait_read();
+    __syncwarp();
+  }
+  // Words [from, to) of tile `done` of the rows [r0, r1) of the warp.
+  __device__ __forceinline__ void words(const FillDesc& d, uint64_t row0, int r0, int r1, uint32_t from,
+                                        uint32_t to) const {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint8_t* b = box + (done & 1) * 4096 + (lane & 3) * 4;
+    uint32_t* out = static_cast<uint32_t*>(d.out);
+    if (lane < from || lane >= to) return;
+    for (int r = r0; r < r1; r++) {
+      const uint64_t e = (row0 + r) * d.pitch + 32 * done + off + lane;
+      if (e < d.limit)
+        st_out(out + e, *reinterpret_cast<const uint32_t*>(b + r * 128 + (((lane >> 2) ^ (r & 7)) << 4)));
+    }
+  }
+  // Tile `done`, words up to `to`, leaves.
+  __device__ __forceinline__ void leave(const FillDesc& d, uint64_t row0, uint32_t to) {
+    const uint64_t left = d.n_rows - row0;
+    const int rows = left < 32 ? (int)left : 32;
+    if (map != nullptr && lo == 0 && to == kBox) {
+      tc::fence_smem_to_async();
+      __syncwarp();
+      if ((threadIdx.x & 31) == 0 && row0 < whole)
+        tc::tile_store(map, tc::smem_addr(box) + (uint32_t)(done & 1) * 4096u, (uint32_t)done * kBox, (uint32_t)row0);
+      if (whole >= row0 && whole < row0 + rows)
+        words(d, row0, (int)(whole - row0), (int)(whole - row0) + 1, 0, kBox);
+    } else {
+      __syncwarp();
+      words(d, row0, 0, rows, lo, to);
+    }
+    lo = 0;
+    done++;
+  }
+};
+
+// Segments of one luxury level's fills.
+//
+// Per warp and product as k_fill_ranlux_tiles; a CTA's four warps are at
+// different places of different items and meet only at the products.
+template <int OM>
+__global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ LuxJob job, int level) {
+  __shared__ __align__(1024) uint8_t boxes[4][2 * 4096];
+  __shared__ __align__(128) TcTable sh;
+  __shared__ FillDesc descs[4];
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+  lux_setup(sh);
+  lux_operand(sh, level, 0);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tm = sh.tmem;
+  lux_constants(tm);
+
+  const FillDesc& d = descs[wi];
+  SegOut so{};
+  so.box = boxes[wi];
+  so.rowb = (uint32_t)(lane * 128 + ((lane & 7) << 4));
+  uint32_t next = blockIdx.x * 4 + wi;     // item of a single fill's warps, in turn
+  bool have = false, dry = false, due = false, zero = false, last = false, ok = true;
+  uint64_t row0 = 0, left = 0;
+  int m = 0;
+  uint32_t N[18], R[18];
+#pragma unroll
+  for (int i = 0; i < 18; i++) N[i] = d_word(i);
+
+  auto words = [&]() {
+    lux_words(N, R);
+    if (zero) {
+#pragma unroll
+      for (int i = 0; i < 18; i++) R[i] = 0;
+    }
+  };
+  auto deliver = [&]() {
+    words();
+    so.acquire();
+    so.put4(0, lux_chunk<OM, 0>(R));
+    so.put4(1, lux_chunk<OM, 1>(R));
+    so.put4(2, lux_chunk<OM, 2>(R));
+    so.put4(3, lux_chunk<OM, 3>(R));
+    so.put4(4, lux_chunk<OM, 4>(R));
+    so.put4(5, lux_chunk<OM, 5>(R));
+    so.pos += 24;
+    if ((so.pos >> 5) > so.done) so.leave(d, row0, kBox);
+  };
+
+  for (uint32_t it = 0;; it++) {
+    while (!have && !dry && ok) {         // this warp's next item that needs a product
+      uint32_t i;
+      if (job.counter != nullptr) {
+        i = pop_warp(job.counter);
+      } else {
+        i = next;
+        next += gridDim.x * 4;
+      }
+      dry = i >= job.n_items;
+      if (dry) break;
+      const LuxItem I = lux_item(job, i, &descs[wi]);
+      const LuxPlan plan(d);
+      const uint64_t b0 = (uint64_t)I.seg << job.lgb;
+      if (b0 > 0 && plan.nb <= b0) continue;
+      uint64_t nb = plan.nb - b0;
+      last = true;
+      if (job.max_seg > 0 && nb > 1ull << job.lgb) {
+        nb = 1ull << job.lgb;
+        last = false;
+      }
+      m = last ? plan.m : 0;
+      left = nb + (m > 0 ? 1 : 0);
+      if (left == 0) continue;            // all of it in the block that was open
+      row0 = I.row0;
+      const uint64_t e0 = plan.h + 24 * b0;
+      const uint32_t* st = job.starts + (uint64_t)i * kStartWords + lane;
+#pragma unroll
+      for (int k = 0; k < 18; k++) N[k] = st[32 * k];
+      zero = st[32 * 18] != 0;
+      so.off = (uint32_t)(e0 & 3);
+      so.pos = e0 - so.off;
+      so.done = so.pos >> 5;
+      so.lo = (uint32_t)(so.pos & 31);
+      so.map = so.off == 0 ? I.map : nullptr;
+      so.whole = d.limit / d.pitch;
+      have = true;
+    }
+    lux_digits(tm, N);
+    if (!__syncthreads_or(have)) break;
+    if (wi == 0) lux_product(sh, tm);
+    if (due) deliver();                   // the previous block, while the product runs
+    due = false;
+    // A warp whose wait gives up drops its item and takes no other.
+    ok = __all_sync(0xFFFFFFFFu, lux_take(sh, tm, it & 1u, N)) && ok;
+    have = have && ok;
+    if (!have) continue;
+    if (--left > 0) {
+      due = true;
+      continue;
+    }
+    if (m == 0) {
+      deliver();
+    } else {
+      lux_back24(N);                      // the state at the start of the open block
+      words();
+    }
+    if (so.pos & 31) so.leave(d, row0, (uint32_t)(so.pos & 31));
+    so.acquire();                         // the tiles are free
+    if (last) {
+      const uint64_t row = row0 + lane;
+      const bool active = row < d.n_rows;
+      uint32_t* out = static_cast<uint32_t*>(d.out);
+      lux_finish(d, row, active, N, R, m, reinterpret_cast<uint32_t*>(so.box) + 25 * lane,
+                 [&](uint64_t k, uint32_t prev, uint32_t x) {
+                   const uint64_t e = row * d.pitch + d.n_per - m + k;
+                   if (!active || e >= d.limit) return;
+                   if constexpr (OM == OUT_F64) {
+                     if (k & 1) st_pair<24>(out + e - 1, prev, x);
+                   } else {
+                     st_out(out + e, tc_conv<OM>(x));
+                   }
+                 });
+      __syncwarp();
+    }
+    have = false;
+  }
+  if (!ok && lane == 0) atomicExch(&g_stuck, 1u);
+  if (lane == 0) tc::tile_store_wait_read();
+  lux_teardown(tm);
 }
 
 int level_of(int p) {
@@ -906,10 +1245,7 @@ int level_of(int p) {
 
 }  // namespace
 
-// The tensor map of a fill's output as an n_rows x pitch array of words, tiles of
-// 32 x 32; false when it has none (memory that is not this device's, sizes past
-// the map's limits).
-static bool out_map(const FillDesc& d, CUtensorMap* map) {
+bool lux_out_map(void* out, uint64_t pitch, uint64_t rows, CUtensorMap* map) {
   using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -921,30 +1257,92 @@ static bool out_map(const FillDesc& d, CUtensorMap* map) {
       f = nullptr;
     return reinterpret_cast<Encode>(f);
   }();
-  if (encode == nullptr || d.pitch >= 1ull << 32 || d.n_rows >= 1ull << 32) return false;
+  if (encode == nullptr || out == nullptr || (reinterpret_cast<uintptr_t>(out) & 15) != 0 || (pitch & 3) != 0 ||
+      pitch == 0 || rows == 0 || pitch >= 1ull << 32 || rows >= 1ull << 32)
+    return false;
   cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, d.out) != cudaSuccess) {
+  if (cudaPointerGetAttributes(&at, out) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   int dev = -1;
   cudaGetDevice(&dev);
   if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
-  const cuuint64_t dim[2] = {d.pitch, d.n_rows}, stride[1] = {4 * d.pitch};
+  const cuuint64_t dim[2] = {pitch, rows}, stride[1] = {4 * pitch};
   const cuuint32_t box[2] = {(cuuint32_t)kBox, (cuuint32_t)kBox}, step[2] = {1, 1};
-  return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, d.out, dim, stride, box, step,
+  return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, out, dim, stride, box, step,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_fill_ranlux_tc(const FillDesc& d, cudaStream_t s) {
+uint64_t lux_start_bytes(uint64_t items) { return items * kStartWords * sizeof(uint32_t); }
+
+LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest) {
+  // Four CTAs per SM of four warps each.  Few blocks: a segment for each of those
+  // warps, of 8 blocks at least (a segment's start costs about three).  Many: three
+  // or four segments per warp, which even out the last wave.
+  const uint64_t slots = 16 * (uint64_t)sm_count(), share = warp_blocks / slots;
+  const uint64_t want = share < 24 ? std::max<uint64_t>(8, share + 1) : share / 3;
+  LuxSplit sp;
+  while (sp.lgb < 40 && (1ull << sp.lgb) < want) sp.lgb++;
+  if (share >= 24 && sp.lgb > 4) sp.lgb--;
+  // Group g starts by powers lgb + 4 .. lgb + 4 + log2(g).
+  while ((longest >> sp.lgb >> kLgGroup >> std::max(0, kPowers - kLgGroup - sp.lgb)) != 0) sp.lgb++;
+  sp.cut = longest > 1ull << sp.lgb;
+  return sp;
+}
+
+cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s) {
+  if (job.n_items == 0) return cudaSuccess;
+  const int level = level_of(p);
+  if (level < 0) return cudaErrorInvalidValue;
+  const uint32_t ctas = (job.n_items + 3) / 4, cap = 4 * (uint32_t)sm_count();
+  k_lux_starts<<<ctas, 128, 0, s>>>(job, level);
+  const uint32_t grid = ctas < cap ? ctas : cap;
+  switch (mode) {
+    case OUT_U32: k_lux_items<OUT_U32><<<grid, 128, 0, s>>>(job, level); break;
+    case OUT_F32: k_lux_items<OUT_F32><<<grid, 128, 0, s>>>(job, level); break;
+    case OUT_F64: k_lux_items<OUT_F64><<<grid, 128, 0, s>>>(job, level); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+// A plain fill cut into segments (scratch for their starts from the retained pool).
+static cudaError_t launch_segments(const FillDesc& d, const LuxSplit& sp, cudaStream_t s) {
+  LuxJob job{};
+  const uint64_t nb = (d.n_per - std::min<uint64_t>(d.n_per, d.pos < 24 ? 24 - d.pos : 0)) / 24;
+  const uint64_t warps = (d.n_rows + 31) / 32, segs = std::max<uint64_t>(1, (nb + (1ull << sp.lgb) - 1) >> sp.lgb);
+  if (warps * segs > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+  job.one = d;
+  job.warps = (uint32_t)warps;
+  job.n_items = (uint32_t)(warps * segs);
+  job.lgb = sp.lgb;
+  job.max_seg = (uint32_t)segs - 1;
+  job.tiles = lux_out_map(d.out, d.pitch, d.n_rows, &job.map) ? 1 : 0;
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&job.starts), lux_start_bytes(job.n_items), s);
+  if (e != cudaSuccess) return e;
+  e = launch_lux_job(job, d.p, d.mode, s);
+  const cudaError_t ef = scratch_free(job.starts, s);
+  return e != cudaSuccess ? e : ef;
+}
+
+cudaError_t launch_fill_ranlux_tc(const FillDesc& d, bool segments, cudaStream_t s) {
   const int level = level_of(d.p);
   if (level < 0) return cudaErrorInvalidValue;
+  if (segments && d.out != nullptr && d.mode != OUT_ISING) {
+    const LuxSplit sp = lux_split((d.n_rows + 31) / 32 * (d.n_per / 24), d.n_per / 24);
+    if (sp.cut) {
+      const cudaError_t e = launch_segments(d, sp, s);
+      if (e != cudaErrorMemoryAllocation) return e;
+      cudaGetLastError();
+    }
+  }
   const bool vec = (d.pos >= 24 || (d.pos & 3) == 0) && (d.pitch & 3) == 0 &&
                    (d.mode == OUT_ISING || (reinterpret_cast<uintptr_t>(d.out) & 15) == 0);
   const uint64_t grid = (d.n_rows + 127) / 128;
   CUtensorMap map;
-  const bool tiles = vec && d.mode != OUT_ISING && d.out != nullptr && out_map(d, &map);
+  const bool tiles = vec && d.mode != OUT_ISING && lux_out_map(d.out, d.pitch, d.n_rows, &map);
   return with_mode(d.mode, [&](auto mode) {
     constexpr int OM = decltype(mode)::value;
     if constexpr (OM != OUT_ISING) {

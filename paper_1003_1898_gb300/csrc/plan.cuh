@@ -1,0 +1,111 @@
+// plan.cuh -- how the fills of a batch are cut into work items (host side, shared
+// by prng_batch_* and prng_batcher_*).
+#pragma once
+
+#include <algorithm>
+
+#include "../../include/prng.h"
+#include "batch.cuh"
+#include "handle.cuh"
+#include "ranlux_tc.cuh"
+
+namespace prng {
+
+struct ItemPlan {
+  bool tensor = true;            // false: RANLUX on the borrow chain (no room for the segments' starts)
+  Tile tile[FAM_COUNT];
+  LuxSplit split[FAM_COUNT];     // tensor-core families
+  uint32_t max_seg[FAM_COUNT] = {};
+
+  ItemPlan() {
+    for (int f = 0; f < FAM_COUNT; f++) tile[f] = tile_of(f);
+  }
+  // RANLUX families whose fills run on the tensor cores.
+  bool is_lux_tc(int f) const {
+    return tensor && kind_of(f) >= FAM_LUX24 && kind_of(f) < FAM_KINDS && lux_p_of(f) >= kLuxTcMinP;
+  }
+  // The segment length of every tensor-core family, from all its requests;
+  // without `cut` each stream is one segment.
+  void choose(const prng_fill_req* reqs, uint32_t n, bool cut) {
+    uint64_t wb[FAM_COUNT] = {}, longest[FAM_COUNT] = {};
+    for (uint32_t i = 0; i < n; i++) {
+      if (reqs[i].n_per_stream == 0) continue;
+      const int f = fill_family(reqs[i].st->gen, reqs[i].st->p, reqs[i].f32 != 0);
+      if (!is_lux_tc(f)) continue;
+      const uint64_t nb = reqs[i].n_per_stream / 24;
+      wb[f] += (reqs[i].st->n_streams + 31) / 32 * (nb + 1);
+      longest[f] = std::max(longest[f], nb);
+    }
+    for (int f = 0; f < FAM_COUNT; f++) {
+      split[f] = LuxSplit{};
+      max_seg[f] = 0;
+      if (cut && longest[f] > 0) split[f] = lux_split(wb[f], longest[f]);
+      if (split[f].cut) max_seg[f] = (uint32_t)(segments(f, 24 * longest[f]) - 1);
+    }
+  }
+  // Segments of a request of n draws per stream.  (A start inside a block can
+  // leave one block fewer than n / 24; a segment past the last block is skipped.)
+  uint64_t segments(int f, uint64_t n) const {
+    if (!split[f].cut) return 1;
+    const uint64_t B = 1ull << split[f].lgb;
+    return std::max<uint64_t>(1, (n / 24 + B - 1) / B);
+  }
+  uint64_t count(int f, const prng_state* st, uint64_t n) const {
+    if (is_lux_tc(f)) return (st->n_streams + 31) / 32 * segments(f, n);
+    const uint32_t per = rows_per_item(f, tile[f]);
+    return (st->n_streams + per - 1) / per;
+  }
+  // Work of the request's longest item, in draws or blocks of one thread.
+  uint64_t cost(int f, uint64_t n) const {
+    if (is_lux_tc(f)) return split[f].cut ? std::min<uint64_t>(n / 24, 1ull << split[f].lgb) : n / 24;
+    return n;
+  }
+  // The request's items, in order.
+  template <class Push>
+  void items(int f, uint32_t req, const prng_state* st, uint64_t n, Push push) const {
+    if (is_lux_tc(f)) {
+      const uint64_t segs = segments(f, n);
+      for (uint64_t s = 0; s < segs; s++)
+        for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 32) push(BatchItem{req, (uint32_t)s, r0});
+      return;
+    }
+    const uint32_t per = rows_per_item(f, tile[f]);
+    for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per)
+      push(BatchItem{req, (uint32_t)std::min<uint64_t>(per, st->n_streams - r0), r0});
+  }
+};
+
+// Tensor map of a request's output, up to its limit's last whole row.
+inline bool request_map(const prng_fill_req& r, CUtensorMap* map) {
+  const uint64_t full = r.st->n_streams * r.n_per_stream;
+  const uint64_t limit = (r.n_valid == 0 || r.n_valid > full) ? full : r.n_valid;
+  return r.n_per_stream > 0 && lux_out_map(r.d_out, r.n_per_stream, limit / r.n_per_stream, map);
+}
+
+// The kernel of family f (not the seeding) on stream s; starts: the family's
+// segment starts, lux_start_bytes(q.n_items), for a tensor-core family.
+inline cudaError_t launch_family(int f, const BatchQueue& q, const ItemPlan& plan, const CUtensorMap* maps,
+                                 uint32_t* starts, cudaStream_t s) {
+  const bool f32 = is_f32_family(f);
+  const Tile t = plan.tile[f];
+  switch (kind_of(f)) {
+    case FAM_MLCG: return launch_batch_mlcg(q, t, s);
+    case FAM_XOR128: return launch_batch_xor128(q, t, f32, s);
+    case FAM_RANMAR: return launch_batch_ranmar(q, t, f32, s);
+    case FAM_MT: return launch_batch_mt(q, t, f32, s);
+    default: break;
+  }
+  if (!plan.is_lux_tc(f)) return launch_batch_ranlux(q, lux_p_of(f), t, f32, s);
+  LuxJob job{};
+  job.reqs = q.reqs;
+  job.items = q.items;
+  job.maps = maps;
+  job.counter = q.counter;
+  job.starts = starts;
+  job.n_items = q.n_items;
+  job.max_seg = plan.max_seg[f];
+  job.lgb = plan.split[f].lgb;
+  return launch_lux_job(job, lux_p_of(f), f32 ? OUT_F32 : OUT_U32, s);
+}
+
+}  // namespace prng

@@ -1,5 +1,7 @@
-// ranlux_tc.cuh -- entry points of the tensor-core RANLUX fill (k_ranlux_tc.cu).
+// ranlux_tc.cuh -- entry points of the tensor-core RANLUX fills (k_ranlux_tc.cu).
 #pragma once
+
+#include <cuda.h>
 
 #include "ranlux.cuh"
 
@@ -21,6 +23,36 @@ bool lux_tc_stuck();
 // The launch tile of a plain fill that leaves it to the library.
 Tile ranlux_auto_tile(const FillDesc& d);
 
-cudaError_t launch_fill_ranlux_tc(const FillDesc& d, cudaStream_t s);
+// A plain fill; with `segments` a few long streams may be cut into segments.
+cudaError_t launch_fill_ranlux_tc(const FillDesc& d, bool segments, cudaStream_t s);
+
+// Fills of one luxury level and output type as work items of 32 streams and one
+// segment (BatchItem: req, row0, and the segment in `rows`).
+struct LuxJob {
+  CUtensorMap map;          // single fill: its output's, if tiles
+  FillDesc one;             // single fill (reqs == nullptr): item = segment x warps + warp of 32 streams
+  const BatchReq* reqs;
+  const BatchItem* items;
+  const CUtensorMap* maps;  // by request, valid where BatchReq::tiles
+  uint32_t* counter;        // items are popped from it, or taken in turn when it is nullptr
+  uint32_t* starts;         // lux_start_bytes(n_items)
+  uint32_t n_items, warps, max_seg, tiles;
+  int lgb;                  // segments of 2^lgb blocks; all of a stream when max_seg = 0
+};
+cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s);
+uint64_t lux_start_bytes(uint64_t items);
+
+// How long the segments are of fills that have warp_blocks blocks in all (per 32
+// streams) and `longest` blocks in the longest stream; cut: whether any stream is.
+struct LuxSplit {
+  int lgb = 0;
+  bool cut = false;
+};
+LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest);
+
+// The tensor map of an output as a rows x pitch array of words in tiles of 32 x
+// 32; false when it has none (unaligned, not this device's memory, past the
+// map's limits).
+bool lux_out_map(void* out, uint64_t pitch, uint64_t rows, CUtensorMap* map);
 
 }  // namespace prng

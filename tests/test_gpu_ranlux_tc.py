@@ -1,5 +1,5 @@
-"""The tensor-core RANLUX fill (tile 128 x 24) against the oracle: heads, tails
-and copy-outs of every length class, every output mode, aligned and unaligned
+"""The tensor-core RANLUX fills (tile 128 x 24: streams whole, or long ones cut
+into segments) against the oracle: heads, tails and copy-outs of every length class, every output mode, aligned and unaligned
 rows, and the states at which its modular arithmetic could go wrong."""
 import numpy as np
 import pytest
@@ -23,11 +23,11 @@ def _built():
     P.lib()
 
 
-@pytest.fixture(autouse=True)
-def _tile():
+@pytest.fixture(autouse=True, params=[1, 2], ids=["whole", "segments"])
+def _tile(request):
     saved = {p: P.prng_get_tile("ranlux", p) for p in LEVELS}
     for p in LEVELS:
-        P.prng_set_tile("ranlux", p, 128, 24, 1)
+        P.prng_set_tile("ranlux", p, 128, 24, request.param)
     yield
     for p, t in saved.items():
         P.prng_set_tile("ranlux", p, *t)
@@ -147,3 +147,34 @@ def test_bulk_equals_borrow_chain():
         P.prng_destroy(h)
     assert torch.equal(outs[0], outs[1])
     assert blobs[0] == blobs[1]
+
+
+@pytest.mark.parametrize("lux", [97, 223, 408])
+def test_batches_of_segments(lux):
+    # Requests of several shapes in one launch, streams long enough to be cut,
+    # a limit inside a row, unaligned rows, continued over three launches.
+    specs = [(70, 24 * 100 + 7, 0), (1, 4100, 0), (129, 2400, 129 * 2400 - 3000), (33, 2404, 2404 * 32 + 17),
+             (5, 30, 0), (40, 20, 0)]
+    for batcher in (False, True):
+        hs, outs, reqs, refs = [], [], [], []
+        for i, (ns, per, valid) in enumerate(specs):
+            hs.append(P.prng_create("ranlux", 500 + i, ns, lux))
+            outs.append(torch.full((ns * per,), -7, dtype=torch.int32, device="cuda"))
+            reqs.append({"st": hs[-1], "d_out": outs[-1], "n_per_stream": per, "n_valid": valid, "f32": i % 2 == 1})
+            refs.append(oracle.fill("ranlux", 500 + i, ns, 3 * per, luxury=lux))
+        b = P.prng_batcher_create(len(specs), 4096) if batcher else P.prng_batch_create(reqs)
+        for k in range(3):
+            for o in outs:
+                o.fill_(-7)
+            P.prng_batcher_launch(b, reqs) if batcher else P.prng_batch_launch(b)
+            for i, ((ns, per, valid), o, ref) in enumerate(zip(specs, outs, refs)):
+                want = ref[:, k * per:(k + 1) * per].reshape(-1)[:valid or None]
+                if i % 2 == 1:
+                    want = oracle.to_f32("ranlux", want).view(np.uint32)
+                got = o.cpu().numpy()
+                np.testing.assert_array_equal(got[:want.size].view(np.uint32), want, err_msg=f"{specs[i]} launch {k}")
+                assert np.all(got[want.size:] == -7), f"{specs[i]} wrote past n_valid"
+        torch.cuda.synchronize()
+        (P.prng_batcher_destroy if batcher else P.prng_batch_destroy)(b)
+        for h in hs:
+            P.prng_destroy(h)
