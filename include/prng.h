@@ -268,7 +268,8 @@ typedef struct prng_ising_req {
  * The descriptors are passed by value to the kernels (no allocation).
  * Lattices with L a multiple of 16, d_spins and d_draws 16-byte aligned and
  * (pitch = 0 or per a multiple of 8 and pitch of 4) run a thread per 16
- * sites with 16-byte row and draw accesses; the others a thread per site.
+ * sites of four rows with 16-byte row and draw accesses; the others a thread
+ * per four sites.
  * The result is the same. */
 int prng_ising_half_sweep(const prng_ising_req *reqs, uint32_t n, void *stream);
 

@@ -16,9 +16,9 @@
 // Lattices whose rows split into 16-byte chunks (L a multiple of 16, both
 // buffers 16-byte aligned, and a draw layout that keeps 8 consecutive
 // ranks in one row) take the vector form: a thread owns 16 consecutive
-// sites of a row, 8 of them of the colour, and moves them as one 16-byte
-// load and store per row (its own row and the rows above and below) and two
-// 16-byte draw loads.  The others take the scalar form, a thread per site.
+// sites of four rows, 8 of them of the colour in each, and moves them as one
+// 16-byte load and store per row (the rows above and below read too) and two
+// 16-byte draw loads per row.  The others take the scalar form, a thread per site.
 #include <cmath>
 
 #include "../../include/prng.h"
@@ -72,10 +72,26 @@ __global__ void __launch_bounds__(kIsingThreads) k_ising_half_sweep(const __grid
   }
 }
 
-// Vector form.  The 16-byte store also rewrites the 8 sites of the other
-// colour with the values it read: nothing changes them during the
-// half-sweep, so readers of those neighbours see the same bytes.
+// Vector form: a thread owns kIsingRows rows of 16 consecutive sites and updates
+// the 8 sites of the colour in each, four at a time as the bytes of a word.
+//
+// A spin byte is 0x01 or 0xFF, so two spins' XOR is 0x00 (aligned) or 0xFE, and
+// with the four neighbours' XORs e the site's class is bit logic on whole words:
+// two or more e set: dE <= 0, flip; exactly one: dE = 4; none: dE = 8.  The draw
+// decides the last two by d < t << shift, which is (d >> shift) < t without the
+// shift (always, when t << shift passes 32 bits).  A flip is XOR 0xFE.  The
+// 16-byte store also rewrites the 8 sites of the other colour with the values it
+// read: nothing changes them during the half-sweep, so readers of those
+// neighbours see the same bytes.
+//
+// What bounds it is DRAM: per site updated 2 bytes of spins read and 2 written
+// (both colours' bytes) and 4 of draws.  The site-by-site form it replaces
+// (compare, multiply and select per site on bytes, one row per thread) ran 340
+// instructions per 8 updates and was bound by their issue: 11 lattices of 4096^2
+// 179 -> 135 us, 4 of them 58 -> 37, 16 of 1024^2 15 -> 11; smaller launches cost
+// what a launch costs in both.
 constexpr int kIsingVecThreads = 256;
+constexpr int kIsingRows = 4;
 
 __device__ __forceinline__ uint32_t ising_lattice_of(const IsingLaunch& b) {
   uint32_t lo = 0, hi = b.n;
@@ -87,50 +103,102 @@ __device__ __forceinline__ uint32_t ising_lattice_of(const IsingLaunch& b) {
   return lo;
 }
 
+// q = a / b, by a shift when b is a power of two.
+__device__ __forceinline__ uint32_t div_pow2(uint32_t a, uint32_t b) {
+  return (b & (b - 1)) == 0 ? a >> (31 - __clz(b)) : a / b;
+}
+
+// m |= bit when d < t.
+__device__ __forceinline__ void or_if_below(uint32_t& m, uint32_t d, uint32_t t, uint32_t bit) {
+  asm("{\n\t"
+      ".reg .pred p;\n\t"
+      "setp.lt.u32 p, %1, %2;\n\t"
+      "@p or.b32 %0, %0, %3;\n\t"
+      "}"
+      : "+r"(m)
+      : "r"(d), "r"(t), "r"(bit));
+}
+
+// 0xFE in the bytes of the four sites c that flip, given their neighbours above
+// (u), below (n) and on either side (l, r) and their draws.
+__device__ __forceinline__ uint32_t ising_flips4(uint32_t c, uint32_t u, uint32_t n, uint32_t l, uint32_t r,
+                                                 uint4 d, uint32_t t4, uint32_t t8, uint32_t always4,
+                                                 uint32_t always8) {
+  uint32_t m4 = always4, m8 = always8;
+  or_if_below(m4, d.x, t4, 0x000000FEu);
+  or_if_below(m4, d.y, t4, 0x0000FE00u);
+  or_if_below(m4, d.z, t4, 0x00FE0000u);
+  or_if_below(m4, d.w, t4, 0xFE000000u);
+  or_if_below(m8, d.x, t8, 0x000000FEu);
+  or_if_below(m8, d.y, t8, 0x0000FE00u);
+  or_if_below(m8, d.z, t8, 0x00FE0000u);
+  or_if_below(m8, d.w, t8, 0xFE000000u);
+  const uint32_t any_v = (u ^ c) | (n ^ c), both_v = (u ^ c) & (n ^ c);
+  const uint32_t any_h = (l ^ c) | (r ^ c), both_h = (l ^ c) & (r ^ c);
+  const uint32_t any = any_v | any_h;
+  return both_v | both_h | (any_v & any_h) | (any & m4) | (~any & m8);
+}
+
 __global__ void __launch_bounds__(kIsingVecThreads) k_ising_half_sweep_v(const __grid_constant__ IsingLaunch b) {
   const uint32_t lo = ising_lattice_of(b);
   const prng_ising_req& q = b.r[lo];
   const uint32_t L = q.L, cpr = L >> 4;                      // 16-site chunks per row
-  const uint32_t chunk = (blockIdx.x - b.block0[lo]) * kIsingVecThreads + threadIdx.x;
-  if (chunk >= L * cpr) return;                              // L <= 65534: L * L / 16 < 2^28
-  const uint32_t y = chunk / cpr, x0 = (chunk - y * cpr) << 4;
-  const uint32_t yu = y == 0 ? L - 1 : y - 1, yd = y + 1 == L ? 0 : y + 1;
-  int8_t* row = q.d_spins + (uint64_t)y * L;
-  union V { uint4 v; int8_t c[16]; };
-  V C, U, D;
-  C.v = *reinterpret_cast<const uint4*>(row + x0);
-  U.v = *reinterpret_cast<const uint4*>(q.d_spins + (uint64_t)yu * L + x0);
-  D.v = *reinterpret_cast<const uint4*>(q.d_spins + (uint64_t)yd * L + x0);
-  const int lft = row[x0 == 0 ? L - 1 : x0 - 1];
-  const int rgt = row[x0 + 16 == L ? 0 : x0 + 16];
-  const uint32_t par = (y + q.colour) & 1u;                 // x parity of the colour in row y
-  const uint32_t k0 = y * (L >> 1) + (x0 >> 1);              // colour rank of the first site
-  uint64_t di = k0;
-  if (q.pitch != 0) {   // 8 ranks never straddle a row of `per` (per % 8 == 0)
-    const uint32_t per = q.per;
-    const uint32_t pr = (per & (per - 1)) == 0 ? k0 >> (__ffs(per) - 1) : k0 / per;
-    di = (uint64_t)pr * q.pitch + (k0 - pr * per);
+  const uint32_t unit = (blockIdx.x - b.block0[lo]) * kIsingVecThreads + threadIdx.x;
+  if (unit >= L / kIsingRows * cpr) return;                  // L <= 65520: L * L / 64 < 2^26
+  const uint32_t strip = div_pow2(unit, cpr);
+  const uint32_t y0 = strip * kIsingRows, x0 = (unit - strip * cpr) << 4;
+  const uint64_t w4 = (uint64_t)q.t4 << q.shift, w8 = (uint64_t)q.t8 << q.shift;
+  const uint32_t t4 = (uint32_t)w4, t8 = (uint32_t)w8;
+  const uint32_t always4 = w4 >> 32 ? 0xFEFEFEFEu : 0u, always8 = w8 >> 32 ? 0xFEFEFEFEu : 0u;
+  int8_t* const col = q.d_spins + x0;
+
+  uint4 row[kIsingRows + 2];   // rows y0 - 1 .. y0 + kIsingRows
+#pragma unroll
+  for (int i = 0; i < kIsingRows + 2; i++) {
+    uint32_t y = y0 + i - 1;
+    if (i == 0 && y0 == 0) y = L - 1;
+    if (i == kIsingRows + 1 && y == L) y = 0;
+    row[i] = *reinterpret_cast<const uint4*>(col + (uint64_t)y * L);
   }
-  const uint4 d0 = *reinterpret_cast<const uint4*>(q.d_draws + di);
-  const uint4 d1 = *reinterpret_cast<const uint4*>(q.d_draws + di + 4);
-  const uint32_t dr[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-  V O = C;
+  uint4 d[kIsingRows][2];
+  uint32_t side[kIsingRows];   // the neighbour beside the chunk: before it, or behind it
 #pragma unroll
-  for (int i = 0; i < 8; i++) {
-#pragma unroll
-    for (int p = 0; p < 2; p++) {     // compile-time byte index for each parity
-      if ((uint32_t)p != par) continue;
-      const int bi = 2 * i + p;
-      const int s = C.c[bi];
-      const int l = bi == 0 ? lft : C.c[bi - 1];
-      const int r = bi == 15 ? rgt : C.c[bi + 1];
-      const int dE = 2 * s * (U.c[bi] + D.c[bi] + l + r);
-      const uint32_t v = dr[i] >> q.shift;
-      const bool accept = dE <= 0 || (dE == 4 ? v < q.t4 : v < q.t8);
-      if (accept) O.c[bi] = (int8_t)(-s);
+  for (int i = 0; i < kIsingRows; i++) {
+    const uint32_t y = y0 + i, par = (y + q.colour) & 1u;     // x parity of the colour in row y
+    const uint32_t k0 = y * (L >> 1) + (x0 >> 1);              // colour rank of the first site
+    uint64_t di = k0;
+    if (q.pitch != 0) {   // 8 ranks never straddle a row of `per` (per % 8 == 0)
+      const uint32_t pr = div_pow2(k0, q.per);
+      di = (uint64_t)pr * q.pitch + (k0 - pr * q.per);
     }
+    d[i][0] = __ldcs(reinterpret_cast<const uint4*>(q.d_draws + di));
+    d[i][1] = __ldcs(reinterpret_cast<const uint4*>(q.d_draws + di + 4));
+    const uint32_t xs = par ? (x0 + 16 == L ? 0 : x0 + 16) : (x0 == 0 ? L - 1 : x0 - 1);
+    side[i] = (uint8_t)q.d_spins[(uint64_t)y * L + xs];
   }
-  *reinterpret_cast<uint4*>(row + x0) = O.v;
+#pragma unroll
+  for (int i = 0; i < kIsingRows; i++) {
+    const bool odd = ((y0 + i + q.colour) & 1u) != 0;
+    const uint4 C = row[i + 1], U = row[i], D = row[i + 2];
+    // Bytes of the colour (and, in the row itself, of the other one), in order.
+    const uint32_t mine = odd ? 0x7531u : 0x6420u, other = odd ? 0x6420u : 0x7531u;
+    const uint32_t c0 = __byte_perm(C.x, C.y, mine), c1 = __byte_perm(C.z, C.w, mine);
+    const uint32_t o0 = __byte_perm(C.x, C.y, other), o1 = __byte_perm(C.z, C.w, other);
+    // The other neighbour in the row: one place before (even sites) or behind (odd ones).
+    const uint32_t s0 = __byte_perm(o0, odd ? o1 : side[i], odd ? 0x4321u : 0x2104u);
+    const uint32_t s1 = __byte_perm(o1, odd ? side[i] : o0, odd ? 0x4321u : 0x2107u);
+    const uint32_t f0 = ising_flips4(c0, __byte_perm(U.x, U.y, mine), __byte_perm(D.x, D.y, mine), o0, s0, d[i][0],
+                                     t4, t8, always4, always8);
+    const uint32_t f1 = ising_flips4(c1, __byte_perm(U.z, U.w, mine), __byte_perm(D.z, D.w, mine), o1, s1, d[i][1],
+                                     t4, t8, always4, always8);
+    const uint32_t lo2 = odd ? 0x1404u : 0x4140u, hi2 = odd ? 0x3424u : 0x4342u;
+    uint4 O;
+    O.x = C.x ^ __byte_perm(f0, 0, lo2);
+    O.y = C.y ^ __byte_perm(f0, 0, hi2);
+    O.z = C.z ^ __byte_perm(f1, 0, lo2);
+    O.w = C.w ^ __byte_perm(f1, 0, hi2);
+    *reinterpret_cast<uint4*>(col + (uint64_t)(y0 + i) * L) = O;
+  }
 }
 
 // Whether a lattice can take the vector form.
@@ -156,9 +224,9 @@ extern "C" int prng_ising_half_sweep(const prng_ising_req* reqs, uint32_t n, voi
   }
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   // Each group of up to kIsingPerLaunch lattices: the vector-form ones in one
-  // launch, the rest in another (a thread per 16 sites / per 4 sites).
+  // launch, the rest in another (a thread per 4 x 16 sites / per 4 sites).
   for (int vec = 1; vec >= 0; vec--) {
-    const uint64_t per_block = vec ? (uint64_t)kIsingVecThreads * 16
+    const uint64_t per_block = vec ? (uint64_t)kIsingVecThreads * 16 * kIsingRows
                                    : (uint64_t)kIsingThreads * kIsingSitesPerThread * 2;
     IsingLaunch b;
     b.n = 0;
