@@ -21,24 +21,79 @@
 namespace prng {
 
 // RMARIN (James 1988, cited by Section 3.5): 97 entries of 24 bits, most
-// significant bit first, from the lagged product generator mod 179 and the
-// LCG (53 l + 1) mod 169.  Written in canonical order V[k] = U[97 - k].
-__device__ void rmarin_to_state(uint32_t ij, uint32_t kl, uint32_t* st, uint64_t n, uint64_t row) {
-  uint32_t i = (ij / 177) % 177 + 2, j = ij % 177 + 2;
-  uint32_t k = (kl / 169) % 178 + 1, l = kl % 169;
-  for (int ii = 1; ii <= 97; ii++) {
+// significant bit first, from the lagged product generator m <- i j k mod 179
+// and the LCG l <- (53 l + 1) mod 169.  Written in canonical order V[k] = U[97 -
+// k].
+//
+// Both sequences jump, so the entries need not wait for one another: 179 is
+// prime and no term is 0, so with logarithms to the base 2 (a primitive root of
+// 179) a term is i^A j^B k^C, the exponents a tribonacci sequence mod 178; and n
+// LCG steps are l -> 53^n l + c mod 169.  kRmarin holds them for the start of
+// every entry (24 steps each).  A thread takes `cnt` entries from entry e0 on:
+// one thread for all of them (2,328 serial steps) took 76 us to re-seed up to 4,096
+// streams and 328 for 131,072; now 7, 12 (4,096 streams) and 206, integer-bound.
+struct Rmarin {
+  uint8_t log[179], exp[178];
+  uint8_t e[97][3][3];   // exponents of (i, j, k) for the three terms before entry e
+  uint8_t a[97], c[97];  // LCG: l -> a l + c mod 169
+};
+constexpr Rmarin make_rmarin() {
+  Rmarin t{};
+  uint32_t x = 1;
+  for (int n = 0; n < 178; n++) {
+    t.exp[n] = (uint8_t)x;
+    t.log[x] = (uint8_t)n;
+    x = 2 * x % 179;
+  }
+  uint32_t w[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}}, a = 1, c = 0;
+  for (int e = 0; e < 97; e++) {
+    for (int r = 0; r < 3; r++)
+      for (int v = 0; v < 3; v++) t.e[e][r][v] = (uint8_t)w[r][v];
+    t.a[e] = (uint8_t)a;
+    t.c[e] = (uint8_t)c;
+    for (int k = 0; k < 24; k++) {
+      for (int v = 0; v < 3; v++) {
+        const uint32_t m = (w[0][v] + w[1][v] + w[2][v]) % 178;
+        w[0][v] = w[1][v];
+        w[1][v] = w[2][v];
+        w[2][v] = m;
+      }
+      a = 53 * a % 169;
+      c = (53 * c + 1) % 169;
+    }
+  }
+  return t;
+}
+__device__ constexpr Rmarin kRmarin = make_rmarin();
+
+__device__ void rmarin_entries(uint32_t ij, uint32_t kl, uint32_t* st, uint64_t n, uint64_t row, int e0, int cnt) {
+  const uint32_t li = kRmarin.log[(ij / 177) % 177 + 2], lj = kRmarin.log[ij % 177 + 2],
+                 lk = kRmarin.log[(kl / 169) % 178 + 1];
+  uint32_t v[3];
+#pragma unroll
+  for (int r = 0; r < 3; r++)
+    v[r] = kRmarin.exp[(kRmarin.e[e0][r][0] * li + kRmarin.e[e0][r][1] * lj + kRmarin.e[e0][r][2] * lk) % 178];
+  uint32_t i = v[0], j = v[1], k = v[2], l = (kRmarin.a[e0] * (kl % 169) + kRmarin.c[e0]) % 169;
+  for (int e = e0; e < e0 + cnt; e++) {
     uint32_t acc = 0;
-    for (int b = 23; b >= 0; b--) {
-      const uint32_t m = ((i * j) % 179 * k) % 179;
+#pragma unroll 8
+    for (int b = 0; b < 24; b++) {
+      const uint32_t m = i * j * k % 179;   // below 179^3: one reduction does
       i = j;
       j = k;
       k = m;
       l = (53 * l + 1) % 169;
-      acc |= ((l * m) % 64 >= 32 ? 1u : 0u) << b;
+      acc = 2 * acc + ((l * m >> 5) & 1u);
     }
-    st[(uint64_t)(97 - ii) * n + row] = acc;
+    st[(uint64_t)(96 - e) * n + row] = acc;
   }
-  st[97 * n + row] = 362436u;  // C_0 = 362436 / 2^24
+  if (e0 == 0) st[97 * n + row] = 362436u;  // C_0 = 362436 / 2^24
+}
+
+// Stream `row` of a RANMAR handle: its entries e0 .. e0 + cnt - 1.
+__device__ void seed_ranmar(uint64_t seed, uint64_t n, uint32_t* st, uint64_t row, int e0, int cnt) {
+  const uint64_t s = splitmix64(seed + row);
+  rmarin_entries((uint32_t)s % 31329u, (uint32_t)(s >> 32) % 30082u, st, n, row, e0, cnt);
 }
 
 // Seed stream `row` of a handle of n streams (state layout in common.cuh).
@@ -64,7 +119,7 @@ __device__ void seed_stream(int gen, uint64_t seed, uint64_t n, uint32_t* st, ui
       st[n + row] = 1 + hi % 2147483398u;
       break;
     case RANMAR:
-      rmarin_to_state(lo % 31329u, hi % 30082u, st, n, row);
+      rmarin_entries(lo % 31329u, hi % 30082u, st, n, row, 0, 97);
       break;
     case RANLUX: {
       uint32_t x = (uint32_t)(s % 2147483563ull);
@@ -79,12 +134,15 @@ __device__ void seed_stream(int gen, uint64_t seed, uint64_t n, uint32_t* st, ui
       break;
     }
     case MT19937: {
-      uint32_t* mt = st + row * 624;
-      uint32_t v = lo;
-      mt[0] = v;
-      for (uint32_t k = 1; k < 624; k++) {
-        v = 1812433253u * (v ^ (v >> 30)) + k;
-        mt[k] = v;
+      uint4* mt = reinterpret_cast<uint4*>(st + row * 624);   // 16-byte stores: four words a step
+      uint4 q;
+      q.w = lo;
+      for (uint32_t k = 0; k < 624; k += 4) {
+        q.x = k == 0 ? lo : 1812433253u * (q.w ^ (q.w >> 30)) + k;
+        q.y = 1812433253u * (q.x ^ (q.x >> 30)) + k + 1;
+        q.z = 1812433253u * (q.y ^ (q.y >> 30)) + k + 2;
+        q.w = 1812433253u * (q.z ^ (q.z >> 30)) + k + 3;
+        mt[k / 4] = q;
       }
       break;
     }
@@ -96,6 +154,13 @@ __global__ void k_seed(int gen, uint64_t seed, uint64_t n, uint32_t* st) {
   if (row < n) seed_stream(gen, seed, n, st, row);
 }
 
+// RANMAR handles: a thread per stream and G entries (blockIdx.y counts them).
+__global__ void __launch_bounds__(128) k_seed_ranmar(uint64_t seed, uint64_t n, uint32_t* st, int G) {
+  const uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int e0 = blockIdx.y * G;
+  if (row < n) seed_ranmar(seed, n, st, row, e0, e0 + G < 97 ? G : 97 - e0);
+}
+
 // Persistent seeding of every re-seeded request of a batch: an item is up
 // to 256 consecutive streams of one request.
 __global__ void __launch_bounds__(256) k_batch_seed(const BatchQueue q) {
@@ -105,7 +170,16 @@ __global__ void __launch_bounds__(256) k_batch_seed(const BatchQueue q) {
     if (it >= q.n_items) break;
     const BatchItem I = q.items[it];
     const BatchReq& r = q.reqs[I.req];
-    if (threadIdx.x < I.rows) seed_stream(r.gen, r.seed, r.d.n_rows, r.d.state, I.row0 + threadIdx.x);
+    if (r.gen == RANMAR) {   // the fewer streams, the fewer entries per thread
+      const uint32_t G = I.rows < 16 ? 1 : I.rows / 8, groups = (97 + G - 1) / G;
+      for (uint32_t u = threadIdx.x; u < I.rows * groups; u += 256) {
+        const uint32_t g = u / I.rows, e0 = g * G;
+        seed_ranmar(r.seed, r.d.n_rows, r.d.state, I.row0 + (u - g * I.rows), (int)e0,
+                    (int)(e0 + G < 97 ? G : 97 - e0));
+      }
+    } else if (threadIdx.x < I.rows) {
+      seed_stream(r.gen, r.seed, r.d.n_rows, r.d.state, I.row0 + threadIdx.x);
+    }
   }
 }
 
@@ -165,7 +239,15 @@ cudaError_t launch_batch_seed(const BatchQueue& q, cudaStream_t s) {
 cudaError_t launch_seed(int gen, int p, uint64_t seed, uint64_t n, uint32_t* state, cudaStream_t s) {
   (void)p;
   if (n == 0) return cudaSuccess;
-  const int T = (gen == RANMAR || gen == MT19937) ? 64 : 256;
+  if (gen == RANMAR) {
+    // Enough threads to fill the GPU; the jump to an entry costs about one entry.
+    const uint64_t want = (uint64_t)sm_count() * 2048;
+    int G = 97;
+    while (G > 1 && n * ((97 + G - 1) / G) < want) G = (G + 1) / 2;
+    k_seed_ranmar<<<dim3((unsigned)((n + 127) / 128), (unsigned)((97 + G - 1) / G)), 128, 0, s>>>(seed, n, state, G);
+    return cudaGetLastError();
+  }
+  const int T = gen == MT19937 ? 64 : 256;
   k_seed<<<(unsigned)((n + T - 1) / T), T, 0, s>>>(gen, seed, n, state);
   return cudaGetLastError();
 }
