@@ -40,7 +40,9 @@ struct prng_batch {
   ItemPlan plan;
   CUtensorMap* d_maps = nullptr;              // outputs of the tensor-core RANLUX requests
   std::vector<uint8_t> tiles;                 //   and which of the requests have one
-  uint32_t* d_starts[FAM_COUNT] = {};         // their segment starts
+  uint32_t* d_starts[FAM_COUNT] = {};         // their segments' starts,
+  uint32_t* d_firsts[FAM_COUNT] = {};         //   the items that begin a group of segments
+  uint32_t n_groups[FAM_COUNT] = {};          //   and how many
   Buffers buf[2];
   int next = 0;
   cudaStream_t cap = nullptr;
@@ -92,7 +94,7 @@ cudaError_t capture(prng_batch* b, Buffers& u) {
     if (b->fam_n[f] == 0) continue;
     cudaStream_t s = b->branch[f];
     cudaStreamWaitEvent(s, b->fork, 0);
-    launch_family(f, queue(f), b->plan, b->d_maps, b->d_starts[f], s);
+    launch_family(f, queue(f), b->plan, b->d_maps, b->d_starts[f], b->d_firsts[f], b->n_groups[f], s);
     cudaEventRecord(b->join[f], s);
     used[nused++] = f;
   }
@@ -151,8 +153,9 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
       const prng_fill_req& r = reqs[i];
       const prng_state* st = r.st;
       if (r.reseed) {
-        for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 256) {
-          const uint32_t rows = (uint32_t)std::min<uint64_t>(256, st->n_streams - r0);
+        const uint32_t per = b->plan.seed_rows(st);
+        for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per) {
+          const uint32_t rows = (uint32_t)std::min<uint64_t>(per, st->n_streams - r0);
           items[FAM_SEED].push_back(BatchItem{i, rows, r0});
           cost[FAM_SEED].push_back(0);
         }
@@ -180,12 +183,22 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
     }
   };
   auto alloc_starts = [&]() {
-    for (int f = 0; f < FAM_COUNT; f++)
-      if (b->plan.is_lux_tc(f) && b->fam_n[f] > 0 &&
-          cudaMalloc(&b->d_starts[f], lux_start_bytes(b->fam_n[f])) != cudaSuccess) {
+    for (int f = 0; f < FAM_COUNT; f++) {
+      if (!b->plan.is_lux_tc(f) || b->fam_n[f] == 0) continue;
+      std::vector<uint32_t> firsts;
+      for (uint32_t k = 0; k < b->fam_n[f]; k++)
+        if (b->plan.first(all[b->fam_off[f] + k])) firsts.push_back(k);
+      b->n_groups[f] = (uint32_t)firsts.size();
+      const size_t bytes = lux_start_bytes(b->fam_n[f]);   // one allocation for both
+      if (cudaMalloc(&b->d_starts[f], bytes + firsts.size() * sizeof(uint32_t)) != cudaSuccess) {
         cudaGetLastError();
         return false;
       }
+      b->d_firsts[f] = b->d_starts[f] + bytes / sizeof(uint32_t);
+      if (cudaMemcpy(b->d_firsts[f], firsts.data(), firsts.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) !=
+          cudaSuccess)
+        return false;
+    }
     return true;
   };
   plan_items();

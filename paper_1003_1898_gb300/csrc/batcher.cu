@@ -27,6 +27,8 @@ constexpr int kSlots = 4;
 struct Slot {
   BatchReq* h_reqs = nullptr;     // pinned
   BatchItem* h_items = nullptr;   // pinned
+  uint32_t* h_firsts = nullptr;   // pinned; items that begin a group of RANLUX segments
+  uint32_t* d_firsts = nullptr;
   CUtensorMap* h_maps = nullptr;  // pinned; outputs of the tensor-core RANLUX requests
   BatchReq* d_reqs = nullptr;
   BatchItem* d_items = nullptr;
@@ -57,6 +59,8 @@ void destroy_batcher(prng_batcher* b) {
     if (u.done) cudaEventDestroy(u.done);
     if (u.h_reqs) cudaFreeHost(u.h_reqs);
     if (u.h_items) cudaFreeHost(u.h_items);
+    if (u.h_firsts) cudaFreeHost(u.h_firsts);
+    if (u.d_firsts) cudaFree(u.d_firsts);
     if (u.h_maps) cudaFreeHost(u.h_maps);
     if (u.d_maps) cudaFree(u.d_maps);
     if (u.d_reqs) cudaFree(u.d_reqs);
@@ -88,6 +92,8 @@ int prng_batcher_create(prng_batcher** out, uint32_t max_requests, uint64_t max_
   for (auto& u : b->slot) {
     if (cudaMallocHost(&u.h_reqs, max_requests * sizeof(BatchReq)) != cudaSuccess ||
         cudaMallocHost(&u.h_items, max_items * sizeof(BatchItem)) != cudaSuccess ||
+        cudaMallocHost(&u.h_firsts, max_items * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMalloc(&u.d_firsts, max_items * sizeof(uint32_t)) != cudaSuccess ||
         cudaMallocHost(&u.h_maps, max_requests * sizeof(CUtensorMap)) != cudaSuccess ||
         cudaMalloc(&u.d_maps, max_requests * sizeof(CUtensorMap)) != cudaSuccess ||
         cudaMalloc(&u.d_reqs, max_requests * sizeof(BatchReq)) != cudaSuccess ||
@@ -128,7 +134,7 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
     std::fill(fam_n, fam_n + FAM_COUNT, 0);
     for (uint32_t i = 0; i < n_reqs; i++) {
       const prng_fill_req& r = reqs[i];
-      if (r.reseed) fam_n[FAM_SEED] += (r.st->n_streams + 255) / 256;
+      if (r.reseed) fam_n[FAM_SEED] += (r.st->n_streams + plan.seed_rows(r.st) - 1) / plan.seed_rows(r.st);
       if (r.n_per_stream == 0) continue;
       const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
       fam_n[f] += plan.count(f, r.st, r.n_per_stream);
@@ -188,10 +194,11 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
     q.gen = st->gen;
     q.reseed = r.reseed ? 1 : 0;
     st->pos = advance_pos(st->gen, q.d.pos, r.n_per_stream);
-    if (r.reseed)
-      for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 256)
-        u.h_items[at[FAM_SEED]++] =
-            BatchItem{i, (uint32_t)std::min<uint64_t>(256, st->n_streams - r0), r0};
+    if (r.reseed) {
+      const uint32_t per = plan.seed_rows(st);
+      for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per)
+        u.h_items[at[FAM_SEED]++] = BatchItem{i, (uint32_t)std::min<uint64_t>(per, st->n_streams - r0), r0};
+    }
     if (r.n_per_stream > 0) {
       const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
       if (plan.is_lux_tc(f)) {
@@ -213,6 +220,14 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
     const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
     plan.items(f, i, r.st, r.n_per_stream, [&](const BatchItem& it) { u.h_items[at[f]++] = it; });
   }
+  uint32_t groups[FAM_COUNT] = {}, group0[FAM_COUNT] = {}, n_firsts = 0;
+  for (int f = 0; f < FAM_COUNT; f++) {
+    if (!plan.is_lux_tc(f) || plan.max_seg[f] == 0) continue;
+    group0[f] = n_firsts;
+    for (uint32_t k = 0; k < fam_n[f]; k++)
+      if (plan.first(u.h_items[fam_off[f] + k])) u.h_firsts[n_firsts++] = k;
+    groups[f] = n_firsts - group0[f];
+  }
   auto fail = [&](int rc) {
     cudaGetLastError();
     if (starts != nullptr) scratch_free(starts, s);
@@ -222,6 +237,8 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
           cudaSuccess ||
       (total > 0 && cudaMemcpyAsync(u.d_items, u.h_items, total * sizeof(BatchItem),
                                     cudaMemcpyHostToDevice, s) != cudaSuccess) ||
+      (n_firsts > 0 && cudaMemcpyAsync(u.d_firsts, u.h_firsts, n_firsts * sizeof(uint32_t), cudaMemcpyHostToDevice,
+                                       s) != cudaSuccess) ||
       (maps && cudaMemcpyAsync(u.d_maps, u.h_maps, n_reqs * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s) !=
                    cudaSuccess) ||
       cudaMemsetAsync(u.d_counters, 0, FAM_COUNT * sizeof(uint32_t), s) != cudaSuccess)
@@ -238,7 +255,7 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
       st = starts + lux_start_bytes(lux_at) / sizeof(uint32_t);
       lux_at += fam_n[f];
     }
-    e = launch_family(f, queue(f), plan, u.d_maps, st, s);
+    e = launch_family(f, queue(f), plan, u.d_maps, st, u.d_firsts + group0[f], groups[f], s);
   }
   if (e != cudaSuccess) return fail(PRNG_ECUDA);
   if (starts != nullptr && scratch_free(starts, s) != cudaSuccess) return PRNG_ECUDA;

@@ -934,61 +934,70 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int
 // segment, took longer than it saved above 4,096 streams (65,536 x 256: 55 us
 // against 31 uncut).
 
-// Starts of an item: words N[18] and the zero flag, 32 streams side by side.
-constexpr uint32_t kStartWords = 19 * 32;
+// What the second kernel needs of an item, in one place: the fill and where the
+// item lies in it, then the words N[18] and the zero flag of its 32 streams side
+// by side.
+struct LuxHead {
+  FillDesc d;
+  uint64_t row0;
+  const CUtensorMap* map;   // of a batched fill's output, or nullptr
+  uint32_t seg, pad;
+};
+constexpr uint32_t kHeadWords = sizeof(LuxHead) / 4, kHeadPitch = 64;
+static_assert(sizeof(LuxHead) % 4 == 0 && kHeadWords <= kHeadPitch, "copied as words by two lanes' turns");
+constexpr uint32_t kStartWords = kHeadPitch + 19 * 32;
 
-struct LuxItem {
+constexpr int kLgGroup = 4, kGroup = (int)kLuxGroup;
+static_assert(kGroup == 1 << kLgGroup, "");
+
+// Head of item `it`, by its warp.
+__device__ __forceinline__ void lux_head_of(const LuxJob& job, uint32_t it, LuxHead* h) {
+  const int lane = threadIdx.x & 31;
   uint32_t seg;
   uint64_t row0;
-  const CUtensorMap* map;   // of its output, or nullptr
-};
-
-constexpr int kLgGroup = 4, kGroup = 1 << kLgGroup;
-
-__device__ __forceinline__ uint32_t lux_segment(const LuxJob& job, uint32_t it) {
-  return job.reqs != nullptr ? job.items[it].rows : it / job.warps;
-}
-
-// Item `it` and its fill (into `sd`, this warp's copy).
-__device__ __forceinline__ LuxItem lux_item(const LuxJob& job, uint32_t it, FillDesc* sd) {
-  const int lane = threadIdx.x & 31;
-  LuxItem I;
-  __syncwarp();
+  const CUtensorMap* map;
   if (job.reqs != nullptr) {
     const BatchItem b = job.items[it];
-    I.seg = b.rows;
-    I.row0 = b.row0;
-    I.map = job.reqs[b.req].tiles ? job.maps + b.req : nullptr;
-    load_desc(sd, job.reqs[b.req].d, lane, 32);
+    seg = b.rows;
+    row0 = b.row0;
+    map = job.reqs[b.req].tiles ? job.maps + b.req : nullptr;
+    load_desc(&h->d, job.reqs[b.req].d, lane, 32);
   } else {
-    I.seg = it / job.warps;
-    I.row0 = 32ull * (it - I.seg * job.warps);
-    I.map = job.tiles ? &job.map : nullptr;
-    load_desc(sd, job.one, lane, 32);
+    seg = it / job.warps;
+    row0 = 32ull * (it - seg * job.warps);
+    map = nullptr;   // the job's own
+    load_desc(&h->d, job.one, lane, 32);
+  }
+  if (lane == 0) {
+    h->row0 = row0;
+    h->map = map;
+    h->seg = seg;
   }
   __syncwarp();
-  return I;
 }
 
 __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ LuxJob job, int level) {
   __shared__ __align__(128) TcTable sh;
   __shared__ uint32_t scratch[128 * 25];
-  __shared__ FillDesc descs[4];
+  __shared__ LuxHead heads[4];
   const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
-  const uint32_t it = blockIdx.x * 4 + wi;
-  const uint32_t seg = it < job.n_items ? lux_segment(job, it) : 1u;
-  const bool have = seg % kGroup == 0;
-  if (!__syncthreads_or(have)) return;
+  const uint32_t g = blockIdx.x * 4 + wi;     // the groups' first items
+  const bool have = g < job.n_groups;
+  const uint32_t it = !have                 ? 0
+                      : job.firsts != nullptr ? job.firsts[g]
+                      : job.reqs != nullptr   ? g
+                                              : g / job.warps * kGroup * job.warps + g % job.warps;
   lux_setup(sh);
 
   uint32_t N[18];
-  uint32_t cnt = 0, warps = 0;   // segments of this group; items from one to the next
+  uint32_t seg = 0, cnt = 0, warps = 0;   // first segment and segments of this group; items from one to the next
   bool zero = false;
   if (have) {
-    const FillDesc& d = descs[wi];
-    const LuxItem I = lux_item(job, it, &descs[wi]);
-    const uint64_t row = I.row0 + lane;
+    lux_head_of(job, it, &heads[wi]);
+    const FillDesc& d = heads[wi].d;
+    const uint64_t row = heads[wi].row0 + lane;
     const bool active = row < d.n_rows;
+    seg = heads[wi].seg;
     const LuxPlan plan(d);
     const uint64_t segs = job.max_seg > 0 ? ((d.n_per / 24 + (1ull << job.lgb) - 1) >> job.lgb) : 1;
     cnt = segs > seg + kGroup ? kGroup : segs > seg ? (uint32_t)(segs - seg) : 1u;
@@ -1037,7 +1046,12 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
   if (__syncthreads_or(cnt > 1)) lux_operand(sh, level, job.lgb);
   for (uint32_t j = 0;; j++) {
     if (j < cnt) {
-      uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords + lane;
+      uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords;
+      if (lane == 0) heads[wi].seg = seg + j;
+      __syncwarp();
+      const uint32_t* h = reinterpret_cast<const uint32_t*>(&heads[wi]);
+      for (uint32_t k = lane; k < kHeadWords; k += 32) st[k] = h[k];
+      st += kHeadPitch + lane;
 #pragma unroll
       for (int k = 0; k < 18; k++) st[32 * k] = N[k];
       st[32 * 18] = zero ? 1u : 0u;
@@ -1079,10 +1093,28 @@ struct SegOut {
     const uint8_t* b = box + (done & 1) * 4096 + (lane & 3) * 4;
     uint32_t* out = static_cast<uint32_t*>(d.out);
     if (lane < from || lane >= to) return;
+    const uint64_t e0 = row0 * d.pitch + 32 * done + off + lane;
+    auto at_row = [&](int r) {
+      return *reinterpret_cast<const uint32_t*>(b + r * 128 + (((lane >> 2) ^ (r & 7)) << 4));
+    };
+    if (r1 - r0 == 32 && e0 + 31 * d.pitch < d.limit) {   // the usual case: eight rows in flight
+      uint32_t* p = out + e0;
+      const uint64_t pitch = d.pitch;
+      for (int r = 0; r < 32; r += 8) {
+        uint32_t v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) v[k] = at_row(r + k);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+          st_out(p, v[k]);
+          p += pitch;
+        }
+      }
+      return;
+    }
     for (int r = r0; r < r1; r++) {
-      const uint64_t e = (row0 + r) * d.pitch + 32 * done + off + lane;
-      if (e < d.limit)
-        st_out(out + e, *reinterpret_cast<const uint32_t*>(b + r * 128 + (((lane >> 2) ^ (r & 7)) << 4)));
+      const uint64_t e = e0 + r * d.pitch;
+      if (e < d.limit) st_out(out + e, at_row(r));
     }
   }
   // Tile `done`, words up to `to`, leaves.
@@ -1113,7 +1145,7 @@ template <int OM>
 __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ LuxJob job, int level) {
   __shared__ __align__(1024) uint8_t boxes[4][2 * 4096];
   __shared__ __align__(128) TcTable sh;
-  __shared__ FillDesc descs[4];
+  __shared__ LuxHead heads[4];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   lux_setup(sh);
   lux_operand(sh, level, 0);
@@ -1123,11 +1155,14 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
   const uint32_t tm = sh.tmem;
   lux_constants(tm);
 
-  const FillDesc& d = descs[wi];
+  const FillDesc& d = heads[wi].d;
   SegOut so{};
   so.box = boxes[wi];
   so.rowb = (uint32_t)(lane * 128 + ((lane & 7) << 4));
-  uint32_t next = blockIdx.x * 4 + wi;     // item of a single fill's warps, in turn
+  // The next item, in lane 0: popped when the one before it starts, so that it is
+  // there when it is wanted; the warps of a single fill take theirs in turn.
+  uint32_t next = blockIdx.x * 4 + wi;
+  if (job.counter != nullptr && lane == 0) next = atomicAdd(job.counter, 1u);
   bool have = false, dry = false, due = false, zero = false, last = false, ok = true;
   uint64_t row0 = 0, left = 0;
   int m = 0;
@@ -1157,18 +1192,22 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
 
   for (uint32_t it = 0;; it++) {
     while (!have && !dry && ok) {         // this warp's next item that needs a product
-      uint32_t i;
-      if (job.counter != nullptr) {
-        i = pop_warp(job.counter);
-      } else {
-        i = next;
-        next += gridDim.x * 4;
-      }
+      const uint32_t i = __shfl_sync(0xFFFFFFFFu, next, 0);
       dry = i >= job.n_items;
       if (dry) break;
-      const LuxItem I = lux_item(job, i, &descs[wi]);
+      if (job.counter == nullptr) next += gridDim.x * 4;
+      else if (lane == 0) next = atomicAdd(job.counter, 1u);
+      const uint32_t* st = job.starts + (uint64_t)i * kStartWords;
+      uint32_t* h = reinterpret_cast<uint32_t*>(&heads[wi]);
+      __syncwarp();
+      for (uint32_t k = lane; k < kHeadWords; k += 32) h[k] = st[k];
+      st += kHeadPitch + lane;
+#pragma unroll
+      for (int k = 0; k < 18; k++) N[k] = st[32 * k];
+      zero = st[32 * 18] != 0;
+      __syncwarp();
       const LuxPlan plan(d);
-      const uint64_t b0 = (uint64_t)I.seg << job.lgb;
+      const uint64_t b0 = (uint64_t)heads[wi].seg << job.lgb;
       if (b0 > 0 && plan.nb <= b0) continue;
       uint64_t nb = plan.nb - b0;
       last = true;
@@ -1179,17 +1218,13 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
       m = last ? plan.m : 0;
       left = nb + (m > 0 ? 1 : 0);
       if (left == 0) continue;            // all of it in the block that was open
-      row0 = I.row0;
+      row0 = heads[wi].row0;
       const uint64_t e0 = plan.h + 24 * b0;
-      const uint32_t* st = job.starts + (uint64_t)i * kStartWords + lane;
-#pragma unroll
-      for (int k = 0; k < 18; k++) N[k] = st[32 * k];
-      zero = st[32 * 18] != 0;
       so.off = (uint32_t)(e0 & 3);
       so.pos = e0 - so.off;
       so.done = so.pos >> 5;
       so.lo = (uint32_t)(so.pos & 31);
-      so.map = so.off == 0 ? I.map : nullptr;
+      so.map = so.off != 0 ? nullptr : job.reqs != nullptr ? heads[wi].map : job.tiles ? &job.map : nullptr;
       so.whole = d.limit / d.pitch;
       have = true;
     }
@@ -1282,10 +1317,9 @@ LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest) {
   // warps, of 8 blocks at least (a segment's start costs about three).  Many: three
   // or four segments per warp, which even out the last wave.
   const uint64_t slots = 16 * (uint64_t)sm_count(), share = warp_blocks / slots;
-  const uint64_t want = share < 24 ? std::max<uint64_t>(8, share + 1) : share / 3;
+  const uint64_t want = share < 24 ? std::max<uint64_t>(8, share + 1) : std::max<uint64_t>(16, share / 4);
   LuxSplit sp;
   while (sp.lgb < 40 && (1ull << sp.lgb) < want) sp.lgb++;
-  if (share >= 24 && sp.lgb > 4) sp.lgb--;
   // Group g starts by powers lgb + 4 .. lgb + 4 + log2(g).
   while ((longest >> sp.lgb >> kLgGroup >> std::max(0, kPowers - kLgGroup - sp.lgb)) != 0) sp.lgb++;
   sp.cut = longest > 1ull << sp.lgb;
@@ -1297,7 +1331,7 @@ cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s) {
   const int level = level_of(p);
   if (level < 0) return cudaErrorInvalidValue;
   const uint32_t ctas = (job.n_items + 3) / 4, cap = 4 * (uint32_t)sm_count();
-  k_lux_starts<<<ctas, 128, 0, s>>>(job, level);
+  k_lux_starts<<<(job.n_groups + 3) / 4, 128, 0, s>>>(job, level);
   const uint32_t grid = ctas < cap ? ctas : cap;
   switch (mode) {
     case OUT_U32: k_lux_items<OUT_U32><<<grid, 128, 0, s>>>(job, level); break;
@@ -1319,6 +1353,7 @@ static cudaError_t launch_segments(const FillDesc& d, const LuxSplit& sp, cudaSt
   job.n_items = (uint32_t)(warps * segs);
   job.lgb = sp.lgb;
   job.max_seg = (uint32_t)segs - 1;
+  job.n_groups = (uint32_t)(warps * ((segs + kGroup - 1) / kGroup));
   job.tiles = lux_out_map(d.out, d.pitch, d.n_rows, &job.map) ? 1 : 0;
   cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&job.starts), lux_start_bytes(job.n_items), s);
   if (e != cudaSuccess) return e;

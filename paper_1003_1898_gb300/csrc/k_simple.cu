@@ -138,6 +138,7 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
   const uint64_t left = d.n_rows > row0 + cr0 ? d.n_rows - (row0 + cr0) : 0;
   const int crows = left >= (uint64_t)RS * (CH - 1) + 1 ? CH : (int)((left + RS - 1) / RS);
   const uint64_t last_row = (row0 + T < d.n_rows ? row0 + T : d.n_rows) - 1;
+  const bool cut = OM != OUT_ISING && last_row * d.pitch + d.n_per > d.limit;   // some of these rows are
   const int sw = tid & 7;
 
   const uint64_t n = d.n_per;
@@ -160,27 +161,43 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
       for (int c = 0; c < w; c++) my[4 * ((c >> 2) ^ sw) + (c & 3)] = conv<G, OM>(g.next());
     }
     __syncthreads();
-    if (w == K && (vec_ok || OM == OUT_ISING) && last_row * d.pitch + c0 + K <= d.limit) {
+    if ((w & 3) == 0 && (vec_ok || OM == OUT_ISING)) {
       const uint32_t* src = t + cr0 * K + 4 * cslot;
       uint32_t* dst = cg + c0;
       const uint64_t edst = (row0 + cr0) * d.pitch + 4 * cch + c0;
+      if (4 * cch < w) {
+        if (!cut) {
 #pragma unroll
-      for (int k = 0; k < CH; k++)
-        if (k < crows) {
-          if constexpr (OM == OUT_ISING)
-            put4<OM, G::WB>(d, nullptr, edst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
-          else
-            st_chunk<OM, G::WB>(dst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
+          for (int k = 0; k < CH; k++)
+            if (k < crows) {
+              if constexpr (OM == OUT_ISING)
+                put4<OM, G::WB>(d, nullptr, edst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
+              else
+                st_chunk<OM, G::WB>(dst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
+            }
+        } else {   // a batched request's or a jump fill's last rows: up to the limit
+          for (int k = 0; k < crows; k++) {
+            const uint64_t e = edst + k * cstep;
+            const uint4 v = *reinterpret_cast<const uint4*>(src + k * RS * K);
+            if (e + 4 <= d.limit) {
+              st_chunk<OM, G::WB>(dst + k * cstep, v);
+            } else if constexpr (OM != OUT_F64) {   // doubles have no limit
+              if (e < d.limit) st_out(dst + k * cstep, v.x);
+              if (e + 1 < d.limit) st_out(dst + k * cstep + 1, v.y);
+              if (e + 2 < d.limit) st_out(dst + k * cstep + 2, v.z);
+            }
+          }
         }
+      }
     } else {
-      // Partial tile, unaligned output or a jump fill's last chunk: scalar
+      // Columns that are no whole 16-byte chunks, or unaligned output: scalar
       // stores, warp per row, lanes on consecutive columns.
       constexpr int NW = T / 32;
       const int lane = tid & 31, wi = tid >> 5;
-      for (int r = wi; r < T; r += NW) {
-        const uint64_t rr = row0 + r;
-        if (rr >= d.n_rows) break;
-        const uint64_t base = rr * d.pitch + c0;
+      const int rows = d.n_rows - row0 < (uint64_t)T ? (int)(d.n_rows - row0) : T;
+#pragma unroll 4
+      for (int r = wi; r < rows; r += NW) {
+        const uint64_t base = (row0 + r) * d.pitch + c0;
         if constexpr (OM == OUT_F64) {   // w, base and the limit are even
           for (int c = 2 * lane; c < w; c += 64)
             if (base + c < d.limit)

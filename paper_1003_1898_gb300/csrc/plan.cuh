@@ -16,6 +16,8 @@ struct ItemPlan {
   Tile tile[FAM_COUNT];
   LuxSplit split[FAM_COUNT];     // tensor-core families
   uint32_t max_seg[FAM_COUNT] = {};
+  uint32_t mt_rows = 2;          // MT19937 streams per item, one after the other
+  uint32_t ranmar_seed_rows = 256;
 
   ItemPlan() {
     for (int f = 0; f < FAM_COUNT; f++) tile[f] = tile_of(f);
@@ -25,8 +27,12 @@ struct ItemPlan {
     return tensor && kind_of(f) >= FAM_LUX24 && kind_of(f) < FAM_KINDS && lux_p_of(f) >= kLuxTcMinP;
   }
   // The segment length of every tensor-core family, from all its requests;
-  // without `cut` each stream is one segment.
+  // without `cut` each stream is one segment and MT19937 items are coarser.
   void choose(const prng_fill_req* reqs, uint32_t n, bool cut) {
+    mt_rows = cut ? 1 : 2;
+    const bool fine = cut && !tile_chosen(XOR128, 0);
+    tile[FAM_XOR128] = tile[FAM_XOR128 + FAM_F32] = fine ? Tile{64, 32, 1} : tile_of(FAM_XOR128);
+    ranmar_seed_rows = cut ? 16 : 256;
     uint64_t wb[FAM_COUNT] = {}, longest[FAM_COUNT] = {};
     for (uint32_t i = 0; i < n; i++) {
       if (reqs[i].n_per_stream == 0) continue;
@@ -50,11 +56,16 @@ struct ItemPlan {
     const uint64_t B = 1ull << split[f].lgb;
     return std::max<uint64_t>(1, (n / 24 + B - 1) / B);
   }
+  // Streams per re-seeding item.
+  uint32_t seed_rows(const prng_state* st) const { return st->gen == RANMAR ? ranmar_seed_rows : 256u; }
+  uint32_t rows(int f) const { return kind_of(f) == FAM_MT ? mt_rows : rows_per_item(f, tile[f]); }
   uint64_t count(int f, const prng_state* st, uint64_t n) const {
     if (is_lux_tc(f)) return (st->n_streams + 31) / 32 * segments(f, n);
-    const uint32_t per = rows_per_item(f, tile[f]);
+    const uint32_t per = rows(f);
     return (st->n_streams + per - 1) / per;
   }
+  // Of a tensor-core family's items, those that start a group of segments.
+  bool first(const BatchItem& it) const { return it.rows % kLuxGroup == 0; }
   // Work of the request's longest item, in draws or blocks of one thread.
   uint64_t cost(int f, uint64_t n) const {
     if (is_lux_tc(f)) return split[f].cut ? std::min<uint64_t>(n / 24, 1ull << split[f].lgb) : n / 24;
@@ -69,7 +80,7 @@ struct ItemPlan {
         for (uint64_t r0 = 0; r0 < st->n_streams; r0 += 32) push(BatchItem{req, (uint32_t)s, r0});
       return;
     }
-    const uint32_t per = rows_per_item(f, tile[f]);
+    const uint32_t per = rows(f);
     for (uint64_t r0 = 0; r0 < st->n_streams; r0 += per)
       push(BatchItem{req, (uint32_t)std::min<uint64_t>(per, st->n_streams - r0), r0});
   }
@@ -83,9 +94,10 @@ inline bool request_map(const prng_fill_req& r, CUtensorMap* map) {
 }
 
 // The kernel of family f (not the seeding) on stream s; starts: the family's
-// segment starts, lux_start_bytes(q.n_items), for a tensor-core family.
+// segment starts, lux_start_bytes(q.n_items), and the n_groups items that start
+// a group of segments, for a tensor-core family.
 inline cudaError_t launch_family(int f, const BatchQueue& q, const ItemPlan& plan, const CUtensorMap* maps,
-                                 uint32_t* starts, cudaStream_t s) {
+                                 uint32_t* starts, const uint32_t* firsts, uint32_t n_groups, cudaStream_t s) {
   const bool f32 = is_f32_family(f);
   const Tile t = plan.tile[f];
   switch (kind_of(f)) {
@@ -102,6 +114,8 @@ inline cudaError_t launch_family(int f, const BatchQueue& q, const ItemPlan& pla
   job.maps = maps;
   job.counter = q.counter;
   job.starts = starts;
+  job.firsts = plan.max_seg[f] > 0 ? firsts : nullptr;
+  job.n_groups = plan.max_seg[f] > 0 ? n_groups : q.n_items;
   job.n_items = q.n_items;
   job.max_seg = plan.max_seg[f];
   job.lgb = plan.split[f].lgb;

@@ -36,9 +36,13 @@ struct LuxJob {
   const CUtensorMap* maps;  // by request, valid where BatchReq::tiles
   uint32_t* counter;        // items are popped from it, or taken in turn when it is nullptr
   uint32_t* starts;         // lux_start_bytes(n_items)
-  uint32_t n_items, warps, max_seg, tiles;
+  const uint32_t* firsts;   // batch: items whose segment is a multiple of kLuxGroup (nullptr: all are)
+  uint32_t n_items, n_groups, warps, max_seg, tiles;
   int lgb;                  // segments of 2^lgb blocks; all of a stream when max_seg = 0
 };
+// Segments whose starts one row walks after one another.
+constexpr uint32_t kLuxGroup = 16;
+
 cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s);
 uint64_t lux_start_bytes(uint64_t items);
 
