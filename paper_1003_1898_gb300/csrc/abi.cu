@@ -52,6 +52,7 @@ int fill_impl(prng_state* st, void* d_out, uint64_t n_per, int mode, cudaStream_
   d.limit = UINT64_MAX;
   d.pos = st->pos;
   d.p = st->p;
+  d.x0 = fill_multiplier(st->gen, n_per);
   d.mode = mode;
   d.jump = 0;
   const Tile t = fill_tile(st, d);
@@ -67,16 +68,6 @@ int fill_impl(prng_state* st, void* d_out, uint64_t n_per, int mode, cudaStream_
   if (e != cudaSuccess) return PRNG_ECUDA;
   st->pos = advance_pos(st->gen, st->pos, n_per);
   return PRNG_OK;
-}
-
-// a^e mod m on the host, for a, m < 2^31 (products stay below 2^62).
-uint64_t host_powmod(uint64_t a, uint64_t e, uint64_t m) {
-  uint64_t r = 1, b = a % m;
-  for (; e; e >>= 1) {
-    if (e & 1) r = r * b % m;
-    b = b * b % m;
-  }
-  return r;
 }
 
 int jump_impl(int gen, uint64_t x0, uint64_t first, uint64_t n, uint32_t n_chunks, void* d_out,
@@ -102,12 +93,12 @@ int jump_impl(int gen, uint64_t x0, uint64_t first, uint64_t n, uint32_t n_chunk
   // The start moved `first` draws on: x_first = a^first x0 (per component).
   if (gen == GGL) {
     if (x0 == 0 || x0 >= 2147483647ull) return PRNG_ESEED;
-    x0 = host_powmod(16807, first, 2147483647ull) * x0 % 2147483647ull;
+    x0 = (uint64_t)const_powmod(16807, first, 2147483647ull) * x0 % 2147483647ull;
   } else {
     uint64_t s1 = x0 & 0xFFFFFFFFull, s2 = x0 >> 32;
     if (s1 == 0 || s1 >= 2147483563ull || s2 == 0 || s2 >= 2147483399ull) return PRNG_ESEED;
-    s1 = host_powmod(40014, first, 2147483563ull) * s1 % 2147483563ull;
-    s2 = host_powmod(40692, first, 2147483399ull) * s2 % 2147483399ull;
+    s1 = (uint64_t)const_powmod(40014, first, 2147483563ull) * s1 % 2147483563ull;
+    s2 = (uint64_t)const_powmod(40692, first, 2147483399ull) * s2 % 2147483399ull;
     x0 = s1 | (s2 << 32);
   }
   // The generator's fill tile decides the kernel.  The lane-parallel one
@@ -288,6 +279,7 @@ int prng_ising_fused(prng_state* st, int8_t* d_spins, uint32_t L, uint32_t colou
   d.limit = sites;
   d.pos = st->pos;
   d.p = st->p;
+  d.x0 = fill_multiplier(st->gen, d.n_per);
   d.mode = OUT_ISING;
   d.jump = 0;
   IsingSink& q = d.ising;

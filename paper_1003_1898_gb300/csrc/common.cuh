@@ -69,7 +69,8 @@ struct FillDesc {
   void* out;           // u32 or f32 output, NULL for a skip
   uint64_t pitch;      // elements between consecutive rows of `out`
   uint64_t limit;      // only elements with linear index < limit are written
-  uint64_t x0;         // jump fills: start value (RANECU: s1 | s2 << 32)
+  uint64_t x0;         // jump fills: start value (RANECU: s1 | s2 << 32); other fills of GGL and
+                       // RANECU: the multiplier a^n_per of the call, component by component likewise
   uint32_t pos;        // RANLUX: draws delivered from the current block; MT: mti
   int32_t p;           // RANLUX luxury p
   int32_t mode;        // OutMode: u32 words, floats, or doubles from pairs
@@ -93,6 +94,24 @@ cudaError_t launch_seed(int gen, int p, uint64_t seed, uint64_t n, uint32_t* sta
                         cudaStream_t s);
 cudaError_t launch_skip_mlcg(int gen, uint32_t* state, uint64_t n, uint64_t k,
                              cudaStream_t s);
+
+// a^e mod m, a constant expression (m < 2^31).
+constexpr uint32_t const_powmod(uint64_t a, uint64_t e, uint64_t m) {
+  uint64_t r = 1;
+  for (; e; e >>= 1) {
+    if (e & 1) r = r * a % m;
+    a = a * a % m;
+  }
+  return (uint32_t)r;
+}
+
+// FillDesc::x0 of a fill of n draws per stream (0 for generators without one).
+inline uint64_t fill_multiplier(int gen, uint64_t n) {
+  if (gen == GGL) return const_powmod(16807, n, 2147483647ull);
+  if (gen == RANECU)
+    return const_powmod(40014, n, 2147483563ull) | (uint64_t)const_powmod(40692, n, 2147483399ull) << 32;
+  return 0;
+}
 
 Tile default_tile(int gen, int p);
 bool tile_chosen(int gen, int p);   // by prng_set_tile
@@ -151,6 +170,17 @@ __device__ __forceinline__ uint32_t mulmod_pm(uint32_t x, uint32_t y) {
   const uint64_t p = (uint64_t)x * y;
   const uint64_t t = (p & 0x7FFFFFFFull) + (p >> 31) * C;
   const uint32_t r = (uint32_t)(t & 0x7FFFFFFFull) + (uint32_t)(t >> 31) * C;
+  return umin32(r, r - M);
+}
+
+// x y mod (2^31 - C) for a fixed y < 2^31 with q = floor(y 2^32 / (2^31 - C)) at
+// hand (Shoup's method): the quotient's estimate from q is at most one too
+// small, so one conditional subtraction ends it -- five instructions where the
+// two folds of mulmod_pm take about twelve.  Any 32-bit x.
+template <uint32_t C>
+__device__ __forceinline__ uint32_t mulmod_fixed(uint32_t x, uint32_t y, uint32_t q) {
+  constexpr uint32_t M = 0x80000000u - C;
+  const uint32_t r = x * y - __umulhi(x, q) * M;   // below 2 M
   return umin32(r, r - M);
 }
 

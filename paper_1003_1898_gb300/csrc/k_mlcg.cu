@@ -11,17 +11,60 @@
 // stream's output row, with no shared-memory staging and no barriers.
 // Rows are taken in a grid-stride loop.  Since every stream of a call
 // advances by the same n, the state left after the call is the stored state
-// times a^n, one multiplication per row with a^n computed once per warp.
+// times a^n, one multiplication per row with a^n from the host.
+//
+// GGL is bound by DRAM, RANECU by the multiply-adds of its two products per
+// draw.  The step from block to block is a product with a constant, whose
+// quotient constant is known too (mulmod_fixed).  131,072 x 8,192 in us, two folds
+// -> this: RANECU u32 845 -> 707, f32 864 -> 746, its jump fill 779 (staged, a
+// thread per chunk) -> 702; GGL 686 (DRAM) as before.
 #include "batch.cuh"
 
 namespace prng {
 
+// One multiplicative generator x <- A x mod (2^31 - C): its step, the steps of 32
+// draws and to the next 128-draw block, and a lane's first multipliers.
+template <uint32_t A, uint32_t C>
+struct Mlcg {
+  static constexpr uint32_t M = 0x80000000u - C;
+  static constexpr uint32_t kBlock = const_powmod(A, 128, M);
+  static constexpr uint32_t kBlockQ = (uint32_t)(((uint64_t)kBlock << 32) / M);
+  static constexpr uint32_t kWarp = const_powmod(A, 32, M);
+  static constexpr uint32_t kWarpQ = (uint32_t)(((uint64_t)kWarp << 32) / M);
+  struct Lanes {
+    uint32_t quad[32], word[32];   // A^(4 lane + 1), A^(lane + 1)
+  };
+  static constexpr Lanes make_lanes() {
+    Lanes t{};
+    for (int l = 0; l < 32; l++) {
+      t.quad[l] = const_powmod(A, 4 * l + 1, M);
+      t.word[l] = const_powmod(A, l + 1, M);
+    }
+    return t;
+  }
+  static __device__ __forceinline__ uint32_t step(uint32_t x) { return mlcg_step<A, C>(x); }
+  static __device__ __forceinline__ uint32_t next_block(uint32_t x) { return mulmod_fixed<C>(x, kBlock, kBlockQ); }
+  static __device__ __forceinline__ uint32_t next_warp(uint32_t x) { return mulmod_fixed<C>(x, kWarp, kWarpQ); }
+  static __device__ __forceinline__ uint32_t mul(uint32_t x, uint32_t y) { return mulmod_pm<C>(x, y); }
+  static __device__ __forceinline__ uint32_t pow(uint64_t e) { return powmod_pm<C>(A, e); }
+};
+using Mlcg0 = Mlcg<16807u, 1u>;
+using Mlcg1 = Mlcg<40014u, 85u>;
+using Mlcg2 = Mlcg<40692u, 249u>;
+__device__ constexpr Mlcg0::Lanes kLanes0 = Mlcg0::make_lanes();
+__device__ constexpr Mlcg1::Lanes kLanes1 = Mlcg1::make_lanes();
+__device__ constexpr Mlcg2::Lanes kLanes2 = Mlcg2::make_lanes();
+
 // GGL: one component, x <- 16807 x mod (2^31 - 1).
 struct GglLJ {
   static constexpr int NC = 1, SH = 7;
-  static __device__ __forceinline__ uint32_t step(int, uint32_t x) { return mlcg_step<16807u, 1u>(x); }
-  static __device__ __forceinline__ uint32_t mul(int, uint32_t x, uint32_t y) { return mulmod_pm<1u>(x, y); }
-  static __device__ __forceinline__ uint32_t pow(int, uint64_t e) { return powmod_pm<1u>(16807u, e); }
+  static __device__ __forceinline__ uint32_t step(int, uint32_t x) { return Mlcg0::step(x); }
+  static __device__ __forceinline__ uint32_t next_block(int, uint32_t x) { return Mlcg0::next_block(x); }
+  static __device__ __forceinline__ uint32_t next_warp(int, uint32_t x) { return Mlcg0::next_warp(x); }
+  static __device__ __forceinline__ uint32_t lane_mul(int, int l) { return kLanes0.quad[l]; }
+  static __device__ __forceinline__ uint32_t word_mul(int, int l) { return kLanes0.word[l]; }
+  static __device__ __forceinline__ uint32_t mul(int, uint32_t x, uint32_t y) { return Mlcg0::mul(x, y); }
+  static __device__ __forceinline__ uint32_t pow(int, uint64_t e) { return Mlcg0::pow(e); }
   static __device__ __forceinline__ uint32_t x0_part(int, uint64_t x0) { return (uint32_t)x0; }
   static __device__ __forceinline__ uint32_t out(const uint32_t (&s)[NC]) { return s[0]; }
 };
@@ -31,14 +74,24 @@ struct GglLJ {
 struct RanecuLJ {
   static constexpr int NC = 2, SH = 7;
   static __device__ __forceinline__ uint32_t step(int c, uint32_t x) {
-    return c == 0 ? mlcg_step<40014u, 85u>(x) : mlcg_step<40692u, 249u>(x);
+    return c == 0 ? Mlcg1::step(x) : Mlcg2::step(x);
+  }
+  static __device__ __forceinline__ uint32_t next_block(int c, uint32_t x) {
+    return c == 0 ? Mlcg1::next_block(x) : Mlcg2::next_block(x);
+  }
+  static __device__ __forceinline__ uint32_t next_warp(int c, uint32_t x) {
+    return c == 0 ? Mlcg1::next_warp(x) : Mlcg2::next_warp(x);
+  }
+  static __device__ __forceinline__ uint32_t lane_mul(int c, int l) {
+    return c == 0 ? kLanes1.quad[l] : kLanes2.quad[l];
+  }
+  static __device__ __forceinline__ uint32_t word_mul(int c, int l) {
+    return c == 0 ? kLanes1.word[l] : kLanes2.word[l];
   }
   static __device__ __forceinline__ uint32_t mul(int c, uint32_t x, uint32_t y) {
-    return c == 0 ? mulmod_pm<85u>(x, y) : mulmod_pm<249u>(x, y);
+    return c == 0 ? Mlcg1::mul(x, y) : Mlcg2::mul(x, y);
   }
-  static __device__ __forceinline__ uint32_t pow(int c, uint64_t e) {
-    return c == 0 ? powmod_pm<85u>(40014u, e) : powmod_pm<249u>(40692u, e);
-  }
+  static __device__ __forceinline__ uint32_t pow(int c, uint64_t e) { return c == 0 ? Mlcg1::pow(e) : Mlcg2::pow(e); }
   static __device__ __forceinline__ uint32_t x0_part(int c, uint64_t x0) {
     return c == 0 ? (uint32_t)(x0 & 0xFFFFFFFFu) : (uint32_t)(x0 >> 32);
   }
@@ -55,17 +108,16 @@ __device__ __forceinline__ uint32_t lj_conv(uint32_t v) {
   else return v;   // u32, or a raw draw paired at the store
 }
 
-// Per-warp constants of one call: multipliers to a lane's first draw, to
-// the next 128-draw block and over the whole call (n draws).
+// Per-warp constants of one call: multipliers to a lane's first draw and over
+// the whole call (handle fills).
 template <class G>
 struct LjConst {
-  uint32_t lane_mul[G::NC], block_mul[G::NC], fin_mul[G::NC];
-  __device__ __forceinline__ void init(int lane, uint64_t n) {
+  uint32_t lane_mul[G::NC], fin_mul[G::NC];
+  __device__ __forceinline__ void init(int lane, uint64_t multiplier) {
 #pragma unroll
     for (int c = 0; c < G::NC; c++) {
-      lane_mul[c] = G::pow(c, 4 * lane + 1);
-      block_mul[c] = G::pow(c, 128);
-      fin_mul[c] = G::pow(c, n);
+      lane_mul[c] = G::lane_mul(c, lane);
+      fin_mul[c] = G::x0_part(c, multiplier);
     }
   }
 };
@@ -113,7 +165,37 @@ __device__ __forceinline__ void lj_row(const LjConst<G>& K, const uint32_t (&bas
         if (c0 + 4 * lane + i < nv) st_out(orow + c0 + i, o[i]);
     }
 #pragma unroll
-    for (int c = 0; c < NC; c++) s[c] = G::mul(c, s[c], K.block_mul[c]);
+    for (int c = 0; c < NC; c++) s[c] = G::next_block(c, s[c]);
+  }
+}
+
+// The same for u32 or float rows that are not 16-byte aligned: lane l takes draws
+// l, l + 32, l + 64 and l + 96 of a block (a product with the constant a^32 costs
+// what a step costs), so every store is one contiguous 128-byte run instead of
+// every fourth word of 512 bytes.  4,096 x 4,095 GGL 27 -> 21 us, 65,536 x
+// 1,001 75 -> 57.
+template <class G, int OM>
+__device__ __forceinline__ void lj_row_words(const uint32_t (&base)[G::NC], int lane, uint32_t* orow, uint64_t nv) {
+  constexpr int NC = G::NC;
+  uint32_t s[NC];
+#pragma unroll
+  for (int c = 0; c < NC; c++) s[c] = G::mul(c, G::word_mul(c, lane), base[c]);
+  for (uint64_t c0 = lane; c0 < nv; c0 += 128) {
+    uint32_t t[NC], o[4];
+#pragma unroll
+    for (int c = 0; c < NC; c++) t[c] = s[c];
+    o[0] = lj_conv<G, OM>(G::out(t));
+#pragma unroll
+    for (int i = 1; i < 4; i++) {
+#pragma unroll
+      for (int c = 0; c < NC; c++) t[c] = G::next_warp(c, t[c]);
+      o[i] = lj_conv<G, OM>(G::out(t));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+      if (c0 + 32 * i < nv) st_out(orow + c0 + 32 * i, o[i]);
+#pragma unroll
+    for (int c = 0; c < NC; c++) s[c] = G::next_block(c, s[c]);
   }
 }
 
@@ -130,7 +212,10 @@ __device__ __forceinline__ void lj_stream(const LjConst<G>& K, const FillDesc& d
   if (left < nv) nv = left;
   uint32_t* out = static_cast<uint32_t*>(d.out);
   const bool vec = ((d.pitch & 3) == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
-  lj_row<G, OM>(K, base, lane, out + row * d.pitch, nv, vec, d, row * d.pitch);
+  if ((OM == OUT_U32 || OM == OUT_F32) && !vec)
+    lj_row_words<G, OM>(base, lane, out + row * d.pitch, nv);
+  else
+    lj_row<G, OM>(K, base, lane, out + row * d.pitch, nv, vec, d, row * d.pitch);
   if (lane == 0) {
 #pragma unroll
     for (int c = 0; c < NC; c++) d.state[c * d.n_rows + row] = G::mul(c, base[c], K.fin_mul[c]);
@@ -144,7 +229,7 @@ __global__ void __launch_bounds__(WPB * 32) k_fill_lj(const FillDesc d) {
   const uint64_t nwarps = (uint64_t)gridDim.x * WPB;
   const uint64_t wrow = (uint64_t)blockIdx.x * WPB + (threadIdx.x >> 5);
   LjConst<G> K;
-  K.init(lane, d.n_per);
+  K.init(lane, d.x0);
   if (!d.jump) {
     for (uint64_t row = wrow; row < d.n_rows; row += nwarps) lj_stream<G, OM>(K, d, row, lane);
     return;
@@ -161,8 +246,10 @@ __global__ void __launch_bounds__(WPB * 32) k_fill_lj(const FillDesc d) {
   for (uint64_t row = wrow; row < d.n_rows; row += nwarps) {
     uint64_t nv = d.n_per;
     if (d.limit - row * d.pitch < nv) nv = d.limit - row * d.pitch;
-    lj_row<G, OM>(K, jrow, lane, out + row * d.pitch, nv, vec_ok && ((row * d.pitch) & 3) == 0, d,
-                  row * d.pitch);
+    if ((OM == OUT_U32 || OM == OUT_F32) && !vec_ok)
+      lj_row_words<G, OM>(jrow, lane, out + row * d.pitch, nv);
+    else
+      lj_row<G, OM>(K, jrow, lane, out + row * d.pitch, nv, vec_ok, d, row * d.pitch);
 #pragma unroll
     for (int c = 0; c < NC; c++) jrow[c] = G::mul(c, jrow[c], jstep[c]);
   }
@@ -185,14 +272,14 @@ __global__ void __launch_bounds__(WPB * 32) k_batch_mlcg(const BatchQueue q) {
     __syncwarp();
     if (r.gen == GGL) {
       LjConst<GglLJ> K;
-      K.init(lane, d.n_per);
+      K.init(lane, d.x0);
       for (uint32_t k = 0; k < I.rows; k++) {
         if (d.mode == OUT_F32) lj_stream<GglLJ, OUT_F32>(K, d, I.row0 + k, lane);
         else lj_stream<GglLJ, OUT_U32>(K, d, I.row0 + k, lane);
       }
     } else {
       LjConst<RanecuLJ> K;
-      K.init(lane, d.n_per);
+      K.init(lane, d.x0);
       for (uint32_t k = 0; k < I.rows; k++) {
         if (d.mode == OUT_F32) lj_stream<RanecuLJ, OUT_F32>(K, d, I.row0 + k, lane);
         else lj_stream<RanecuLJ, OUT_U32>(K, d, I.row0 + k, lane);

@@ -288,8 +288,10 @@ __device__ __forceinline__ void mt_stream(const FillDesc& d, uint64_t row, uint3
   // Draws of this row that are written (all n unless the element limit cuts
   // the row, none when the row lies past it); the stream still advances by n.
   uint64_t nv = n;
-  const uint64_t left = d.limit > row * d.pitch ? d.limit - row * d.pitch : 0;
-  if (store && left < nv) nv = left;
+  if (store && d.limit - row * d.pitch < nv) nv = d.limit - row * d.pitch;
+  if constexpr (!REG) {   // batched fills alone have rows past the limit
+    if (store && row * d.pitch >= d.limit) nv = 0;
+  }
   uint64_t j = 0;
   const uint32_t mti = d.pos;
   if (mti < 624 && n > 0) {  // rest of the current table

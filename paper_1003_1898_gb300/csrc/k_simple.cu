@@ -106,6 +106,73 @@ __device__ __forceinline__ uint32_t conv(uint32_t v) {
 template <int K>
 __device__ __forceinline__ int swz(int row, int ch) { return ch ^ (row & 7); }
 
+// Copy-out of a staged tile that is not plain: columns [c0, c0 + w) of rows
+// [row0, row0 + T), with fewer columns than the tile's, unaligned rows, or rows
+// that a batched request's or a jump fill's limit cuts.  Not inlined: inside the
+// column loop it cost the plain copy-out 11 % (256 x 4,096 f32 70 -> 78 us).
+template <class G, int T, int K, int OM>
+__device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint64_t row0, uint64_t c0, int w) {
+  constexpr int CH = K / 4, RS = T / CH, NW = T / 32;
+  const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+  const uint64_t pitch = d.pitch, limit = d.limit;
+  const int rows = d.n_rows - row0 < (uint64_t)T ? (int)(d.n_rows - row0) : T;
+  uint32_t* out = static_cast<uint32_t*>(d.out);
+  const bool aligned = ((pitch & 3) == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
+  const bool cut = (row0 + rows - 1) * pitch + c0 + w > limit;
+  if (OM != OUT_ISING && (w & 3) == 0 && aligned) {   // whole 16-byte chunks, but for the cut one
+    const int cch = tid % CH;
+    if (4 * cch >= w) return;
+#pragma unroll 4
+    for (int r = tid / CH; r < rows; r += RS) {
+      const uint64_t e = (row0 + r) * pitch + c0 + 4 * cch;
+      const uint4 v = *reinterpret_cast<const uint4*>(t + r * K + 4 * swz<K>(r, cch));
+      if (e + 4 <= limit) {
+        st_chunk<OM, G::WB>(out + e, v);
+      } else if constexpr (OM != OUT_F64) {           // doubles have no limit
+        if (e < limit) st_out(out + e, v.x);
+        if (e + 1 < limit) st_out(out + e + 1, v.y);
+        if (e + 2 < limit) st_out(out + e + 2, v.z);
+      }
+    }
+    return;
+  }
+  // Word by word: a warp per row, lanes on consecutive columns.
+  if (OM != OUT_F64 && OM != OUT_ISING && w == K && rows == T && !cut) {   // eight rows in flight
+    uint32_t* p = out + (row0 + wi) * pitch + c0 + lane;
+    const uint64_t step = NW * pitch;
+    for (int r0 = wi; r0 < T; r0 += 8 * NW) {
+      uint32_t v[8][K / 32];
+#pragma unroll
+      for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < K / 32; j++) {
+          const int r = r0 + i * NW, c = lane + 32 * j;
+          v[i][j] = t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)];
+        }
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+#pragma unroll
+        for (int j = 0; j < K / 32; j++) st_out(p + 32 * j, v[i][j]);
+        p += step;
+      }
+    }
+    return;
+  }
+  for (int r = wi; r < rows; r += NW) {
+    const uint64_t base = (row0 + r) * pitch + c0;
+    if constexpr (OM == OUT_F64) {   // w, base and the limit are even
+      for (int c = 2 * lane; c < w; c += 64)
+        if (base + c < limit)
+          st_pair<G::WB>(out + base + c, t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)],
+                         t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3) + 1]);
+    } else {
+      for (int c = lane; c < w; c += 32)
+        if (base + c < limit)
+          put1<OM>(d, out + base + c, base + c, t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)]);
+    }
+  }
+}
+
 // Streams [row0, row0 + T) of a fill, one per thread; smem holds S tiles of
 // T * K words.
 template <class G, int T, int K, int S, int OM>
@@ -138,7 +205,6 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
   const uint64_t left = d.n_rows > row0 + cr0 ? d.n_rows - (row0 + cr0) : 0;
   const int crows = left >= (uint64_t)RS * (CH - 1) + 1 ? CH : (int)((left + RS - 1) / RS);
   const uint64_t last_row = (row0 + T < d.n_rows ? row0 + T : d.n_rows) - 1;
-  const bool cut = OM != OUT_ISING && last_row * d.pitch + d.n_per > d.limit;   // some of these rows are
   const int sw = tid & 7;
 
   const uint64_t n = d.n_per;
@@ -161,54 +227,20 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
       for (int c = 0; c < w; c++) my[4 * ((c >> 2) ^ sw) + (c & 3)] = conv<G, OM>(g.next());
     }
     __syncthreads();
-    if ((w & 3) == 0 && (vec_ok || OM == OUT_ISING)) {
+    if (w == K && (vec_ok || OM == OUT_ISING) && last_row * d.pitch + c0 + K <= d.limit) {
       const uint32_t* src = t + cr0 * K + 4 * cslot;
       uint32_t* dst = cg + c0;
       const uint64_t edst = (row0 + cr0) * d.pitch + 4 * cch + c0;
-      if (4 * cch < w) {
-        if (!cut) {
 #pragma unroll
-          for (int k = 0; k < CH; k++)
-            if (k < crows) {
-              if constexpr (OM == OUT_ISING)
-                put4<OM, G::WB>(d, nullptr, edst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
-              else
-                st_chunk<OM, G::WB>(dst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
-            }
-        } else {   // a batched request's or a jump fill's last rows: up to the limit
-          for (int k = 0; k < crows; k++) {
-            const uint64_t e = edst + k * cstep;
-            const uint4 v = *reinterpret_cast<const uint4*>(src + k * RS * K);
-            if (e + 4 <= d.limit) {
-              st_chunk<OM, G::WB>(dst + k * cstep, v);
-            } else if constexpr (OM != OUT_F64) {   // doubles have no limit
-              if (e < d.limit) st_out(dst + k * cstep, v.x);
-              if (e + 1 < d.limit) st_out(dst + k * cstep + 1, v.y);
-              if (e + 2 < d.limit) st_out(dst + k * cstep + 2, v.z);
-            }
-          }
+      for (int k = 0; k < CH; k++)
+        if (k < crows) {
+          if constexpr (OM == OUT_ISING)
+            put4<OM, G::WB>(d, nullptr, edst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
+          else
+            st_chunk<OM, G::WB>(dst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
         }
-      }
     } else {
-      // Columns that are no whole 16-byte chunks, or unaligned output: scalar
-      // stores, warp per row, lanes on consecutive columns.
-      constexpr int NW = T / 32;
-      const int lane = tid & 31, wi = tid >> 5;
-      const int rows = d.n_rows - row0 < (uint64_t)T ? (int)(d.n_rows - row0) : T;
-#pragma unroll 4
-      for (int r = wi; r < rows; r += NW) {
-        const uint64_t base = (row0 + r) * d.pitch + c0;
-        if constexpr (OM == OUT_F64) {   // w, base and the limit are even
-          for (int c = 2 * lane; c < w; c += 64)
-            if (base + c < d.limit)
-              st_pair<G::WB>(out + base + c, t[r * K + 4 * ((c >> 2) ^ (r & 7)) + (c & 3)],
-                             t[r * K + 4 * ((c >> 2) ^ (r & 7)) + (c & 3) + 1]);
-        } else {
-          for (int c = lane; c < w; c += 32)
-            if (base + c < d.limit)
-              put1<OM>(d, out + base + c, base + c, t[r * K + 4 * ((c >> 2) ^ (r & 7)) + (c & 3)]);
-        }
-      }
+      odd_tile<G, T, K, OM>(d, t, row0, c0, w);
     }
     if constexpr (S == 1) __syncthreads();
     else buf ^= 1;

@@ -121,6 +121,7 @@ extern "C" int prng_batch_fill_noalloc(const prng_fill_req* reqs, uint32_t n_req
     q.d.limit = (r.n_valid == 0 || r.n_valid > full) ? full : r.n_valid;
     q.d.pos = r.reseed ? initial_pos(st->gen) : st->pos;
     q.d.p = st->p;
+    q.d.x0 = fill_multiplier(st->gen, r.n_per_stream);
     q.d.mode = r.f32 ? OUT_F32 : OUT_U32;
     q.seed = r.seed;
     q.gen = st->gen;
