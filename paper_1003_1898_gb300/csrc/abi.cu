@@ -203,7 +203,7 @@ int prng_create(prng_state** out, prng_gen_t gen, uint64_t seed, uint32_t n_stre
     if (p < 0) return PRNG_ELUXURY;
   }
   if (n_streams == 0) return PRNG_ESIZE;
-  if (g == RANLUX && lux_tables_init() != cudaSuccess) {
+  if ((g == RANLUX && lux_tables_init() != cudaSuccess) || (g == XOR128 && xor128_tables_init() != cudaSuccess)) {
     cudaGetLastError();
     return PRNG_ECUDA;
   }

@@ -139,6 +139,12 @@ cudaError_t launch_jump_mt(uint64_t x0, uint64_t first, uint64_t n, uint32_t n_c
 
 // XOR128 jump-ahead over GF(2): prng_skip of k steps on a handle's state
 // (struct-of-arrays [4][n]), and the single-sequence chunked fill.
+// Start states of a fill's segments: starts[seg][word][stream] = T^(seg 2^lg)
+// applied to stream's state ([4][n]).  The powers' device table is filled by
+// xor128_tables_init, called when an XOR128 handle is created.
+cudaError_t launch_xor128_starts(const uint32_t* state, uint32_t* starts, uint64_t n, uint32_t segs, int lg,
+                                 cudaStream_t s);
+cudaError_t xor128_tables_init();
 cudaError_t launch_skip_xor128(uint32_t* state, uint64_t n, uint64_t k, cudaStream_t s);
 cudaError_t launch_jump_xor128(uint64_t x0, uint64_t first, uint64_t n, uint32_t n_chunks,
                                void* d_out, int f32, cudaStream_t s);

@@ -1367,7 +1367,7 @@ cudaError_t launch_fill_ranlux_tc(const FillDesc& d, bool segments, cudaStream_t
   if (level < 0) return cudaErrorInvalidValue;
   if (segments && d.out != nullptr && d.mode != OUT_ISING) {
     const LuxSplit sp = lux_split((d.n_rows + 31) / 32 * (d.n_per / 24), d.n_per / 24);
-    if (sp.cut) {
+    if (sp.cut && !capturing(s)) {
       const cudaError_t e = launch_segments(d, sp, s);
       if (e != cudaErrorMemoryAllocation) return e;
       cudaGetLastError();

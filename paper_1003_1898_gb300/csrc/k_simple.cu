@@ -13,7 +13,10 @@
 // tiles one barrier per tile suffices; S = 1 halves the shared memory per
 // stream (two barriers per tile) so that every stream of a large handle can
 // be resident at once instead of running a partial second wave.
+#include <algorithm>
+
 #include "batch.cuh"
+#include "scratch.cuh"
 
 namespace prng {
 
@@ -174,9 +177,11 @@ __device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint
 }
 
 // Streams [row0, row0 + T) of a fill, one per thread; smem holds S tiles of
-// T * K words.
+// T * K words.  The n draws go to columns col0 .. col0 + n - 1; the states are
+// read from d.state and left in `store_to` (nullptr: nowhere).
 template <class G, int T, int K, int S, int OM>
-__device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, uint32_t* smem) {
+__device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, uint32_t* smem, uint64_t col0,
+                                            uint64_t n, uint32_t* store_to) {
   static_assert(K % 32 == 0, "tile rows hold whole 8-chunk swizzle groups");
   constexpr int CH = K / 4;          // 16-byte chunks per row
   constexpr int RS = T / CH;         // rows one copy-out pass of the CTA covers
@@ -200,14 +205,13 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
   // Copy-out role of this thread: chunk `cch` of rows cr0 + RS k, k < CH.
   const int cch = tid % CH, cr0 = tid / CH;
   const int cslot = swz<K>(cr0, cch);           // (cr0 + RS k) & 7 == cr0 & 7
-  uint32_t* cg = out + (row0 + cr0) * d.pitch + 4 * cch;
+  uint32_t* cg = out + (row0 + cr0) * d.pitch + col0 + 4 * cch;
   const uint64_t cstep = (uint64_t)RS * d.pitch;
   const uint64_t left = d.n_rows > row0 + cr0 ? d.n_rows - (row0 + cr0) : 0;
   const int crows = left >= (uint64_t)RS * (CH - 1) + 1 ? CH : (int)((left + RS - 1) / RS);
   const uint64_t last_row = (row0 + T < d.n_rows ? row0 + T : d.n_rows) - 1;
   const int sw = tid & 7;
 
-  const uint64_t n = d.n_per;
   int buf = 0;
   for (uint64_t c0 = 0; c0 < n; c0 += K) {
     const int w = (n - c0 < (uint64_t)K) ? (int)(n - c0) : K;
@@ -227,10 +231,10 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
       for (int c = 0; c < w; c++) my[4 * ((c >> 2) ^ sw) + (c & 3)] = conv<G, OM>(g.next());
     }
     __syncthreads();
-    if (w == K && (vec_ok || OM == OUT_ISING) && last_row * d.pitch + c0 + K <= d.limit) {
+    if (w == K && (vec_ok || OM == OUT_ISING) && last_row * d.pitch + col0 + c0 + K <= d.limit) {
       const uint32_t* src = t + cr0 * K + 4 * cslot;
       uint32_t* dst = cg + c0;
-      const uint64_t edst = (row0 + cr0) * d.pitch + 4 * cch + c0;
+      const uint64_t edst = (row0 + cr0) * d.pitch + 4 * cch + col0 + c0;
 #pragma unroll
       for (int k = 0; k < CH; k++)
         if (k < crows) {
@@ -240,18 +244,31 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
             st_chunk<OM, G::WB>(dst + k * cstep, *reinterpret_cast<const uint4*>(src + k * RS * K));
         }
     } else {
-      odd_tile<G, T, K, OM>(d, t, row0, c0, w);
+      odd_tile<G, T, K, OM>(d, t, row0, col0 + c0, w);
     }
     if constexpr (S == 1) __syncthreads();
     else buf ^= 1;
   }
-  if (active && !d.jump) g.store(d.state, d.n_rows, row);
+  if (active && store_to != nullptr) g.store(store_to, d.n_rows, row);
 }
 
 template <class G, int T, int K, int S, int OM>
 __global__ void __launch_bounds__(T) k_fill_simple(const FillDesc d) {
   extern __shared__ __align__(16) uint32_t smem[];
-  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem);
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, 0, d.n_per, d.jump ? nullptr : d.state);
+}
+
+// Segment blockIdx.y of every stream: draws [seg L, seg L + L) of the call, from
+// the states that `starts` holds for it ([segment][word][stream]); the last
+// segment leaves the handle's states.
+template <class G, int T, int K, int S, int OM>
+__global__ void __launch_bounds__(T) k_fill_segments(FillDesc d, uint32_t* starts, uint64_t L) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  uint32_t* const state = d.state;
+  const uint64_t seg = blockIdx.y, col0 = seg * L;
+  const uint64_t n = d.n_per - col0 < L ? d.n_per - col0 : L;
+  d.state = starts + seg * 4 * d.n_rows;
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, col0, n, seg + 1 == gridDim.y ? state : nullptr);
 }
 
 // Batched XOR128 fills: a block pops an item (T streams of one request).
@@ -266,7 +283,7 @@ __global__ void __launch_bounds__(T) k_batch_xor128(const BatchQueue q) {
     __shared__ FillDesc sd;
     load_desc(&sd, q.reqs[si.req].d, threadIdx.x, T);
     __syncthreads();
-    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem);
+    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem, 0, sd.n_per, sd.state);
   }
 }
 
@@ -341,6 +358,43 @@ static cudaError_t launch_g(const FillDesc& d, Tile t, cudaStream_t s) {
   return launch_tk<G, 128, 32, 1>(d, s);
 }
 
+// A plain XOR128 fill of few streams as segments of L = 2^k draws, each a thread
+// of its own, whose starts T^(seg L) s come from xor128_starts first.  A thread
+// makes a draw in about 17 ns whatever the number of streams while those leave
+// the GPU idle, so a stream is cut until there are some 65,536 threads, into at
+// most 64 segments of at least 64 draws.  The starts cost a second kernel (about
+// the time of 800 draws) and, at 65,536 threads, that of some 460 more.  us, whole
+// / cut: 256 x 4,096 u32 74 / 28, f64 (as many draws) 165 / 29; 256 x 8,192 135 /
+// 28; 4,096 x 4,096 73 / 38; 1,000 x 4,095 (unaligned) 427 / 41; 16,384 x 4,096
+// 73 / 71, f64 168 / 84; 4,096 x 1,024 26 / 33, which stays whole.
+static cudaError_t launch_xor128_segments(const FillDesc& d, bool& done, cudaStream_t s) {
+  done = false;
+  if (d.n_rows >= 32768 || d.n_per < 900) return cudaSuccess;
+  const uint64_t want = std::min<uint64_t>(64, 65536 / d.n_rows);
+  int lg = 6;
+  while (lg < 57 && ((d.n_per - 1) >> lg) + 1 > want) lg++;
+  const uint64_t L = 1ull << lg, segs = ((d.n_per - 1) >> lg) + 1;
+  if (lg > 56 || L >= d.n_per || d.n_per - L < 800 + 460 * d.n_rows * segs / 65536) return cudaSuccess;
+  if (capturing(s)) return cudaSuccess;
+  uint32_t* starts = nullptr;
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&starts), segs * 4 * d.n_rows * sizeof(uint32_t), s);
+  if (e != cudaSuccess) {   // no room: whole streams
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  done = true;
+  e = launch_xor128_starts(d.state, starts, d.n_rows, (uint32_t)segs, lg, s);
+  if (e == cudaSuccess)
+    e = with_mode(d.mode, [&](auto m) {
+      constexpr int T = 64, K = 32;
+      const dim3 grid((unsigned)((d.n_rows + T - 1) / T), (unsigned)segs);
+      k_fill_segments<Xor128Gen, T, K, 1, decltype(m)::value><<<grid, T, T * K * sizeof(uint32_t), s>>>(d, starts, L);
+      return cudaGetLastError();
+    });
+  const cudaError_t ef = scratch_free(starts, s);
+  return e != cudaSuccess ? e : ef;
+}
+
 cudaError_t launch_fill_simple(int gen, const FillDesc& d, Tile t, cudaStream_t s) {
   if (d.n_rows == 0 || d.n_per == 0) return cudaSuccess;
   if (d.out == nullptr) {  // skip: plain stepping (the MLCG generators jump instead)
@@ -350,7 +404,14 @@ cudaError_t launch_fill_simple(int gen, const FillDesc& d, Tile t, cudaStream_t 
   }
   switch (gen) {
     case GGL: return launch_g<GglGen>(d, t, s);
-    case XOR128: return launch_g<Xor128Gen>(d, t, s);
+    case XOR128: {
+      if (!tile_chosen(XOR128, 0) && !d.jump) {
+        bool done = false;
+        const cudaError_t e = launch_xor128_segments(d, done, s);
+        if (done || e != cudaSuccess) return e;
+      }
+      return launch_g<Xor128Gen>(d, t, s);
+    }
     case RANECU: return launch_g<RanecuGen>(d, t, s);
     default: return cudaErrorInvalidValue;
   }

@@ -26,7 +26,7 @@
 
 namespace prng {
 
-struct Gf2x128 {
+struct alignas(16) Gf2x128 {
   uint32_t col[128][4];   // col[j] = T e_j
 };
 
@@ -170,6 +170,67 @@ __global__ void __launch_bounds__(256) k_xor128_apply3(const __grid_constant__ G
   if (j & 1) gf2_apply_dev(P.m[0], x);
 #pragma unroll
   for (int i = 0; i < 4; i++) state[i * pitch + r] = x[i];
+}
+
+// T^(2^i), i < 64, on the device (128 KB; filled on a device's first XOR128 handle).
+__device__ Gf2x128 g_pow[64];
+
+cudaError_t xor128_tables_init() {
+  static std::mutex lock;
+  static bool done[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> guard(lock);
+  if (done[dev]) return cudaSuccess;
+  e = cudaMemcpyToSymbol(g_pow, pow2_table(), 64 * sizeof(Gf2x128));
+  if (e == cudaSuccess) done[dev] = true;
+  return e;
+}
+
+// Segment blockIdx.y of every stream: a thread applies the powers T^(2^(lg + i))
+// for the bits i of its segment's number, columns from shared memory (every
+// thread reads the same one).
+__global__ void __launch_bounds__(128) k_xor128_starts(const uint32_t* state, uint32_t* starts, uint64_t n, int lg) {
+  __shared__ uint4 col[128];
+  const uint64_t row = (uint64_t)blockIdx.x * 128 + threadIdx.x;
+  const uint32_t seg = blockIdx.y;
+  uint32_t x[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) x[i] = row < n ? state[i * n + row] : 0u;
+  for (int i = 0; seg >> i; i++) {
+    if (!((seg >> i) & 1u)) continue;
+    __syncthreads();
+    col[threadIdx.x] = reinterpret_cast<const uint4*>(&g_pow[lg + i])[threadIdx.x];
+    __syncthreads();
+    uint4 o[2] = {};   // two chains
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+#pragma unroll 8
+      for (int b = 0; b < 32; b++) {
+        const uint32_t m = (uint32_t)((int32_t)(x[w] << (31 - b)) >> 31);
+        const uint4 c = col[32 * w + b];
+        o[b & 1].x ^= c.x & m;
+        o[b & 1].y ^= c.y & m;
+        o[b & 1].z ^= c.z & m;
+        o[b & 1].w ^= c.w & m;
+      }
+    }
+    x[0] = o[0].x ^ o[1].x;
+    x[1] = o[0].y ^ o[1].y;
+    x[2] = o[0].z ^ o[1].z;
+    x[3] = o[0].w ^ o[1].w;
+  }
+  if (row < n)
+#pragma unroll
+    for (int i = 0; i < 4; i++) starts[((uint64_t)seg * 4 + i) * n + row] = x[i];
+}
+
+cudaError_t launch_xor128_starts(const uint32_t* state, uint32_t* starts, uint64_t n, uint32_t segs, int lg,
+                                 cudaStream_t s) {
+  k_xor128_starts<<<dim3((unsigned)((n + 127) / 128), segs), 128, 0, s>>>(state, starts, n, lg);
+  return cudaGetLastError();
 }
 
 __global__ void k_xor128_set_row(uint32_t* state, uint64_t pitch, uint64_t row, uint32_t x,
