@@ -22,9 +22,32 @@ namespace {
 constexpr uint32_t kBlobMagic = 0x50524E47u;  // "PRNG"
 constexpr uint32_t kBlobVersion = 1u;
 
-// The launch tile of a plain fill: the caller's, or by the fill's shape.
+// The launch tile of a plain fill: the caller's, or by the fill's shape.  In us,
+// u32 (f32 alike unless said), the handle's default tile / the one chosen here:
+//   XOR128, 64 staged columns instead of 32: 131,072 x 8,192 763 / 666, x 1,024
+//   111 / 94; 65,536 x 4,096 210 / 202, f64 257 / 249; not for short rows that
+//   leave a tile part empty (fused half-sweeps take such a tile site by site).
+//   RANMAR, four warps per CTA instead of eight, once rows and streams are many:
+//   131,072 x 8,192 677 / 662; 131,072 x 500 71 / 77, which keeps eight.
+//   MT19937, two streams per warp once there are enough to fill the GPU so (f64
+//   keeps a warp per stream, 1,035 / 1,056): in CTAs of a warp for short rows,
+//   8,192 x 64 24 / 17, x 1,000 30 / 22, 6,000 x 5,000 41 / 35; of two for long
+//   ones, 8,192 x 131,072 728 / 678 (one warp 685); 1,024 x 20,000 36 / 37.
 Tile fill_tile(const prng_state* st, const FillDesc& d) {
-  if (!tile_chosen(st->gen, st->p) && st->gen == RANLUX) return ranlux_auto_tile(d);
+  if (!tile_chosen(st->gen, st->p)) switch (st->gen) {
+    case RANLUX: return ranlux_auto_tile(d);
+    case XOR128:
+      if (d.n_per % 64 == 0 || (d.n_per >= 256 && d.mode != OUT_ISING)) return Tile{128, 64, 1};
+      break;
+    case RANMAR:
+      if (d.n_rows >= 32768 && d.n_per >= 4096) return Tile{128, 128, 1};
+      break;
+    case MT19937:
+      if (d.n_rows >= 2048 && (d.mode == OUT_U32 || d.mode == OUT_F32))
+        return d.n_per < 20000 ? Tile{32, 624, 2} : Tile{64, 624, 2};
+      break;
+    default: break;
+  }
   return default_tile(st->gen, st->p);
 }
 

@@ -106,10 +106,18 @@ constexpr uint32_t const_powmod(uint64_t a, uint64_t e, uint64_t m) {
 }
 
 // FillDesc::x0 of a fill of n draws per stream (0 for generators without one).
+template <uint32_t A, uint32_t M>   // a constant modulus: no division per step
+inline uint64_t pow_fixed(uint64_t e) {
+  uint64_t r = 1, a = A;
+  for (; e; e >>= 1) {
+    if (e & 1) r = r * a % M;
+    a = a * a % M;
+  }
+  return r;
+}
 inline uint64_t fill_multiplier(int gen, uint64_t n) {
-  if (gen == GGL) return const_powmod(16807, n, 2147483647ull);
-  if (gen == RANECU)
-    return const_powmod(40014, n, 2147483563ull) | (uint64_t)const_powmod(40692, n, 2147483399ull) << 32;
+  if (gen == GGL) return pow_fixed<16807u, 2147483647u>(n);
+  if (gen == RANECU) return pow_fixed<40014u, 2147483563u>(n) | pow_fixed<40692u, 2147483399u>(n) << 32;
   return 0;
 }
 
