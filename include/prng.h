@@ -146,13 +146,11 @@ int prng_set_state(prng_state *st, const void *h_buf, size_t bytes);
  * sequence into more, shorter chunks than asked (at least 131072 when n
  * allows 64 draws each; the output is the same), and takes a
  * stream-ordered scratch array of 16 bytes per chunk (PRNG_EALLOC if that
- * fails).  MT19937: x0 < 2^32, the sequence of init_genrand(x0); chunk c
- * starts from its table moved c*L words on, built in log2(n_chunks)
- * doubling passes of the jump polynomial (about 6 million word XORs per
- * chunk, so a few thousand chunks is the useful range), with a scratch
- * array of 2.5 KB per chunk.  The MT19937 form merges the chunks into fewer,
- * longer ones when more are asked than one wave of warps holds (27 per SM,
- * a warp per chunk; the output is the same).  The scratch arrays come from a stream-ordered
+ * fails).  MT19937: x0 < 2^32, the sequence of init_genrand(x0); the library
+ * cuts it into chunks of a power of two of draws, as many as pay (up to 4,096),
+ * chunk c starting from its table moved c*L words on, built in log2(chunks)
+ * doubling passes of the jump polynomial (about 6 million word XORs per chunk),
+ * with a scratch array of 44 KB per chunk.  The scratch arrays come from a stream-ordered
  * memory pool that the library creates on first use on each device and
  * that keeps its memory until the process exits, so repeated jump fills do
  * not allocate afresh.  Other generators return PRNG_EUNSUPPORTED. */

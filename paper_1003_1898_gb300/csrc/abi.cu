@@ -32,7 +32,9 @@ constexpr uint32_t kBlobVersion = 1u;
 //   MT19937, two streams per warp once there are enough to fill the GPU so (f64
 //   keeps a warp per stream, 1,035 / 1,056): in CTAs of a warp for short rows,
 //   8,192 x 64 24 / 17, x 1,000 30 / 22, 6,000 x 5,000 41 / 35; of two for long
-//   ones, 8,192 x 131,072 728 / 678 (one warp 685); 1,024 x 20,000 36 / 37.
+//   ones, 8,192 x 131,072 728 / 678 (one warp 685).  A CTA per stream while they
+//   are few: 1 x 100,000 99 / 48, 456 x 65,536 71 / 49, 256 x 4,096 19 / 14, 1,024
+//   x 20,000 37 / 36.
 Tile fill_tile(const prng_state* st, const FillDesc& d) {
   if (!tile_chosen(st->gen, st->p)) switch (st->gen) {
     case RANLUX: return ranlux_auto_tile(d);
@@ -43,6 +45,7 @@ Tile fill_tile(const prng_state* st, const FillDesc& d) {
       if (d.n_rows >= 32768 && d.n_per >= 4096) return Tile{128, 128, 1};
       break;
     case MT19937:
+      if (d.n_rows <= 1024 && d.n_per >= 512 && (d.mode == OUT_U32 || d.mode == OUT_F32)) return Tile{256, 227, 1};
       if (d.n_rows >= 2048 && (d.mode == OUT_U32 || d.mode == OUT_F32))
         return d.n_per < 20000 ? Tile{32, 624, 2} : Tile{64, 624, 2};
       break;
@@ -166,14 +169,14 @@ bool tile_supported(int gen, Tile t, int p = 0) {
   static const Tile lux[] = {{64, 48, 1}, {128, 48, 1}, {256, 48, 1},
                              {64, 56, 1}, {128, 56, 1}, {256, 56, 1}};   // 56: the per-row ring
   static const Tile mar[] = {{128, 128, 1}, {256, 128, 1}};
-  static const Tile mt[] = {{64, 624, 1}, {128, 624, 1}, {256, 624, 1},
+  static const Tile mt[] = {{256, 227, 1}, {64, 624, 1}, {128, 624, 1}, {256, 624, 1},
                             {32, 624, 2}, {64, 624, 2}, {128, 624, 2}, {256, 624, 2}};
   const Tile* list = simple;
   int n = 4;
   if ((gen == GGL || gen == RANECU) && t.cols == 128) { list = mlcg; n = 2; }
   else if (gen == RANLUX) { list = lux; n = 6; }
   else if (gen == RANMAR) { list = mar; n = 2; }
-  else if (gen == MT19937) { list = mt; n = 7; }
+  else if (gen == MT19937) { list = mt; n = 8; }   // 227: a CTA per stream
   for (int i = 0; i < n; i++)
     if (list[i].threads == t.threads && list[i].cols == t.cols && list[i].stages == t.stages)
       return true;

@@ -89,6 +89,7 @@ cudaError_t launch_fill_simple(int gen, const FillDesc& d, Tile t, cudaStream_t 
 cudaError_t launch_fill_mlcg(int gen, const FillDesc& d, Tile t, cudaStream_t s);
 cudaError_t launch_fill_ranmar(const FillDesc& d, Tile t, cudaStream_t s);
 cudaError_t launch_fill_ranlux(const FillDesc& d, Tile t, cudaStream_t s);
+cudaError_t launch_fill_mt_wide(const FillDesc& d, cudaStream_t s);   // a CTA per stream; u32 or f32
 cudaError_t launch_fill_mt(const FillDesc& d, Tile t, cudaStream_t s);
 cudaError_t launch_seed(int gen, int p, uint64_t seed, uint64_t n, uint32_t* state,
                         cudaStream_t s);
@@ -139,8 +140,11 @@ __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 struct MtPoly {
   uint32_t w[624];
 };
-cudaError_t launch_mt_poly_apply(const MtPoly& g, uint32_t* state, uint64_t r0, uint64_t r1,
-                                 uint64_t src_off, cudaStream_t s);
+cudaError_t launch_mt_poly_apply(const MtPoly& g, uint32_t* state, uint64_t n, cudaStream_t s);
+constexpr uint32_t kMtSeq = 33 * 624;   // words of a table's sequence that a polynomial reaches
+cudaError_t launch_mt_sequence(const uint32_t* tables, uint32_t* seq, uint64_t r0, uint64_t rows, cudaStream_t s);
+cudaError_t launch_mt_apply_seq(const MtPoly& g, const uint32_t* seq, uint32_t* tables, uint64_t dst0,
+                                uint64_t rows, cudaStream_t s);
 cudaError_t launch_skip_mt(uint32_t* state, uint64_t n, uint64_t k, cudaStream_t s);
 cudaError_t launch_jump_mt(uint64_t x0, uint64_t first, uint64_t n, uint32_t n_chunks,
                            void* d_out, int mode, cudaStream_t s);

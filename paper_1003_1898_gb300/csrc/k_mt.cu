@@ -349,6 +349,141 @@ __device__ __forceinline__ void mt_stream(const FillDesc& d, uint64_t row, uint3
   __syncwarp();
 }
 
+// ------------------------------------------------------ a CTA per stream
+//
+// For few streams: 227 threads twist one table at once.  Thread t owns words t,
+// 227 + t and (t < 170) 454 + t, in registers from block to block.  A new word
+// needs its old self, the next old word (the neighbour thread's, by a shuffle,
+// or through shared memory at the ends of warps) and the word 227 before or 397
+// behind it: for the second and third of a thread's words that is its own word
+// before, just made.  Only the first takes its lag from other threads, through
+// 227 words of shared memory, so a block of 624 words costs one CTA barrier.
+struct MtWide {
+  uint32_t lag[2][228];   // words 397 .. 623 of the table, by buffer
+  uint32_t edge[2][3][9]; // word i of thread 32 w, and at [1][0][8] of thread 1
+};
+
+struct MtWideRegs {
+  uint32_t a[3];
+};
+
+// Share what the other threads need of the table (buffer b), then a barrier.
+__device__ __forceinline__ void mt_wide_share(MtWide& sh, const MtWideRegs& r, int t, int b) {
+  if (t < 170) sh.lag[b][57 + t] = r.a[2];
+  else if (t < 227) sh.lag[b][t - 170] = r.a[1];
+  if ((t & 31) == 0) {
+#pragma unroll
+    for (int i = 0; i < 3; i++) sh.edge[b][i][t >> 5] = r.a[i];
+  }
+  if (t == 1) sh.edge[b][0][8] = r.a[0];
+  __syncthreads();
+}
+
+// One twist, from buffer b.
+__device__ __forceinline__ void mt_wide_twist(const MtWide& sh, MtWideRegs& r, int t, int b) {
+  const int lane = t & 31, w = t >> 5;
+  uint32_t n[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    n[i] = __shfl_down_sync(0xFFFFFFFFu, r.a[i], 1);
+    if (lane == 31) n[i] = sh.edge[b][i][w < 7 ? w + 1 : 7];
+  }
+  if (t == 226) {   // the next word belongs to thread 0
+    n[0] = sh.edge[b][1][0];
+    n[1] = sh.edge[b][2][0];
+  }
+  if (t == 169) n[2] = mt_mix(sh.edge[b][0][0], sh.edge[b][0][8], sh.lag[b][0]);   // X_624: the new X_0
+  r.a[0] = mt_mix(r.a[0], n[0], sh.lag[b][t < 227 ? t : 0]);
+  r.a[1] = mt_mix(r.a[1], n[1], r.a[0]);
+  r.a[2] = mt_mix(r.a[2], n[2], r.a[1]);
+}
+
+template <int OM>
+__global__ void __launch_bounds__(256) k_fill_mt_wide(const FillDesc d) {
+  __shared__ MtWide sh;
+  const int t = threadIdx.x;
+  const uint64_t row = blockIdx.x;
+  uint32_t* gs = d.state + row * 624;
+  const bool own = t < 227;
+  const int cnt = t < 170 ? 3 : own ? 2 : 0;   // words this thread owns
+  MtWideRegs r;
+#pragma unroll
+  for (int i = 0; i < 3; i++) r.a[i] = i < cnt ? gs[227 * i + t] : 0u;
+  uint32_t* out = static_cast<uint32_t*>(d.out);
+  uint32_t* orow = out != nullptr ? out + row * d.pitch : nullptr;
+  const uint64_t n = d.n_per;
+  uint64_t nv = n;   // words of the row that are written
+  if (d.limit - row * d.pitch < nv) nv = d.limit - row * d.pitch;
+  const uint32_t mti = d.pos;
+  uint64_t j = 0;
+  if (mti < 624) {   // rest of the current table
+    j = 624 - mti < n ? 624 - mti : n;
+    if (orow != nullptr)
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const uint32_t k = 227 * i + t;
+        if (i < cnt && k >= mti && k - mti < j && k - mti < nv) st_out(orow + (k - mti), mt_conv<OM>(mt_temper(r.a[i])));
+      }
+  }
+  int b = 0;
+  mt_wide_share(sh, r, t, b);
+  // Whole blocks.
+  uint64_t nb = orow != nullptr ? (nv > j ? (nv - j) / 624 : 0) : 0;
+  uint32_t* o = orow != nullptr ? orow + j + t : nullptr;
+  j += nb * 624;
+  for (; nb > 0; nb--) {
+    mt_wide_twist(sh, r, t, b);
+    b ^= 1;
+    mt_wide_share(sh, r, t, b);
+    if (own) {
+      st_out(o, mt_conv<OM>(mt_temper(r.a[0])));
+      st_out(o + 227, mt_conv<OM>(mt_temper(r.a[1])));
+    }
+    if (t < 170) st_out(o + 454, mt_conv<OM>(mt_temper(r.a[2])));
+    o += 624;
+  }
+  // What is left: blocks that are cut, or a skip's.
+  while (j < n) {
+    mt_wide_twist(sh, r, t, b);
+    b ^= 1;
+    mt_wide_share(sh, r, t, b);
+    if (orow != nullptr)
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const uint64_t k = 227 * i + t;
+        if (i < cnt && j + k < nv) st_out(orow + j + k, mt_conv<OM>(mt_temper(r.a[i])));
+      }
+    j += 624;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+    if (i < cnt) gs[227 * i + t] = r.a[i];
+}
+
+// The word sequences that tables [r0, r0 + gridDim.x) start, kMtSeq words each
+// (33 tables: all that a polynomial of degree 19,936 reaches), into seq[r].
+__global__ void __launch_bounds__(256) k_mt_sequence(const uint32_t* tables, uint32_t* seq, uint64_t r0) {
+  __shared__ MtWide sh;
+  const int t = threadIdx.x;
+  const uint64_t row = r0 + blockIdx.x;
+  const uint32_t* gs = tables + row * 624;
+  uint32_t* o = seq + row * kMtSeq;
+  const int cnt = t < 170 ? 3 : t < 227 ? 2 : 0;
+  MtWideRegs r;
+#pragma unroll
+  for (int i = 0; i < 3; i++) r.a[i] = i < cnt ? gs[227 * i + t] : 0u;
+  int b = 0;
+  for (int k = 0;; k++) {
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+      if (i < cnt) o[624 * k + 227 * i + t] = r.a[i];
+    if (k == 32) break;
+    mt_wide_share(sh, r, t, b);
+    mt_wide_twist(sh, r, t, b);
+    b ^= 1;
+  }
+}
+
 // SPW streams per warp (1: a warp per stream; 2: a half-warp each, which
 // halves the warps of a fill so that every stream of a large handle is
 // resident in one wave).
@@ -384,28 +519,17 @@ __global__ void __launch_bounds__(WPB * 32) k_batch_mt(const BatchQueue q) {
   }
 }
 
-// Jump-ahead (see k_mt_jump.cu): rows [r0, r1) of a table array become
-// g(T) applied to row r - src_off and moved one more word on, where T moves
-// a table one word along the sequence of Appendix A, "Mersenne twister".
-// Word j of the result is the XOR, over the coefficients g_i = 1, of word
-// 1 + i + j of the word sequence that the source table starts.  A warp
-// walks that sequence 624 words at a time: the current table and the next
-// (twisted from a copy) sit side by side in shared memory, so the words
-// 1 + i + j of a block of 624 values of i are one contiguous window.  Lane l
-// owns result words 20 l .. 20 l + 19 in registers and takes sixteen
+// Jump-ahead (see k_mt_jump.cu): a table becomes g(T) applied to it and moved one
+// more word on, where T moves a table one word along the sequence of Appendix A,
+// "Mersenne twister".  Word j of the result is the XOR, over the coefficients g_i
+// = 1, of word 1 + i + j of the word sequence that the source table starts.  Lane
+// l owns result words 20 l .. 20 l + 19 in registers and takes sixteen
 // coefficients at a time: the 35 words they need start one word past a
 // 16-byte boundary (i is a multiple of 16 and 1 + i + 20 l = 1 mod 4), so
 // they are ten aligned 16-byte shared loads (lanes 80 bytes apart hit eight
 // different bank quads), shared by the sixteen coefficients.  Each nibble
 // of set coefficients (BITS, a compile-time variant) is folded with
 // three-input XORs.
-//
-// The 19937 coefficients are 32 blocks of 624.  A table's blocks can be
-// split over S warps (segments of ceil(32 / S) blocks): segment s first
-// twists its copy of the source table forward by its first block, then
-// accumulates its blocks and XORs its partial result into the (zeroed)
-// destination row with atomics.  S = 1 stores the result directly and may
-// run in place (destination row = source row).
 template <int OFF, int BITS>
 __device__ __forceinline__ void mt_poly_nib(uint32_t (&acc)[20], const uint32_t (&win)[40]) {
 #pragma unroll
@@ -432,34 +556,101 @@ __device__ __forceinline__ void mt_poly_nib_any(uint32_t bits4, uint32_t (&acc)[
   }
 }
 
+// The polynomial product from sequences made beforehand (k_mt_sequence):
+// table dst0 + r becomes g(T) applied to table r and moved one word more, for r <
+// rows.  A warp takes `per` coefficients (a multiple of 16) of one table, whose
+// window of the sequence it stages in shared memory, and XORs its part of the
+// result into the (zeroed) destination.  The few tables of the first doubling
+// passes are spread over as many warps as there are segments of 160 coefficients,
+// each of which starts at once, where a warp that walks the sequence itself has to
+// twist its way to its first block: a pass of one table takes 9 us instead
+// of 30, one of 256 tables 79 instead of 142.
+constexpr int kMtPerMax = 800;   // coefficients a warp takes at most
+
+__global__ void __launch_bounds__(32) k_mt_apply_seq(const __grid_constant__ MtPoly g, const uint32_t* seq,
+                                                     uint32_t* tables, uint64_t dst0, int per) {
+  constexpr int D = 19937;
+  __shared__ __align__(16) uint32_t B[kMtPerMax + 624 + 32];
+  const int lane = threadIdx.x;
+  const uint64_t r = blockIdx.y;
+  const int i0 = blockIdx.x * per, i1 = i0 + per < D ? i0 + per : D;
+  const uint32_t* w = seq + r * kMtSeq + i0;       // 16-byte aligned: i0 and kMtSeq are multiples of 16 words
+  // Words i0 .. i0 + per + 655 (lane 31's words past 623 are computed and
+  // dropped); the sequence's end is never needed, zeros stand for it.
+  for (int k = 4 * lane; k < per + 656; k += 128)
+    *reinterpret_cast<uint4*>(B + k) = i0 + k + 3 < (int)kMtSeq ? *reinterpret_cast<const uint4*>(w + k) : uint4{};
+  __syncwarp();
+  uint32_t acc[20];
+#pragma unroll
+  for (int t = 0; t < 20; t++) acc[t] = 0;
+  for (int i = i0; i < i1; i += 16) {
+    uint32_t bits = (g.w[i >> 5] >> (i & 31)) & 0xFFFFu;
+    if (i1 - i < 16) bits &= (1u << (i1 - i)) - 1u;
+    if (!bits) continue;
+    const int a = (i - i0) + 20 * lane;
+    uint32_t win[40];
+#pragma unroll
+    for (int q = 0; q < 10; q++) {
+      const uint4 v = *reinterpret_cast<const uint4*>(B + a + 4 * q);
+      win[4 * q] = v.x; win[4 * q + 1] = v.y; win[4 * q + 2] = v.z; win[4 * q + 3] = v.w;
+    }
+    mt_poly_nib_any<0>(bits & 0xFu, acc, win);
+    mt_poly_nib_any<4>((bits >> 4) & 0xFu, acc, win);
+    mt_poly_nib_any<8>((bits >> 8) & 0xFu, acc, win);
+    mt_poly_nib_any<12>(bits >> 12, acc, win);
+  }
+  // Through shared memory, so that a warp's atomics cover whole sectors.
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 5; q++)
+    *reinterpret_cast<uint4*>(B + 20 * lane + 4 * q) =
+        make_uint4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+  __syncwarp();
+  uint32_t* dst = tables + (dst0 + r) * 624;
+#pragma unroll
+  for (int k = lane; k < 624; k += 32) atomicXor(dst + k, B[k]);
+}
+
+cudaError_t launch_mt_sequence(const uint32_t* tables, uint32_t* seq, uint64_t r0, uint64_t rows, cudaStream_t s) {
+  if (rows == 0) return cudaSuccess;
+  k_mt_sequence<<<(unsigned)rows, 256, 0, s>>>(tables, seq, r0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mt_apply_seq(const MtPoly& g, const uint32_t* seq, uint32_t* tables, uint64_t dst0,
+                                uint64_t rows, cudaStream_t s) {
+  if (rows == 0) return cudaSuccess;
+  if (rows > 65535) return cudaErrorInvalidValue;
+  // As many warps as run at once, eight per scheduler, of at least 160 coefficients
+  // (and no more than leaves room for their windows in shared memory).
+  int per = 160;
+  while (per < kMtPerMax && rows * ((19937 + per - 1) / per) > 32 * (uint64_t)sm_count()) per += 160;
+  k_mt_apply_seq<<<dim3((19937 + per - 1) / per, (unsigned)rows), 32, 0, s>>>(g, seq, tables, dst0, per);
+  return cudaGetLastError();
+}
+
+// In place on n tables (a handle's skip), a warp each: it walks the sequence 624
+// words at a time, the current table and the next (twisted from a copy) side by
+// side in shared memory, so the words 1 + i + j of a block of 624 values of i are
+// one contiguous window.
 template <int WPB>
-__global__ void __launch_bounds__(WPB * 32) k_mt_poly_apply(const __grid_constant__ MtPoly g,
-                                                            uint32_t* state, uint64_t r0,
-                                                            uint64_t r1, uint64_t src_off,
-                                                            uint32_t S) {
-  constexpr int D = 19937, NB = (D + 623) / 624;
+__global__ void __launch_bounds__(WPB * 32) k_mt_poly_apply(const __grid_constant__ MtPoly g, uint32_t* state,
+                                                            uint64_t n) {
+  constexpr int D = 19937;
   // current table | next table | room for lane 31's over-reach (its words
   // past 623 are computed and dropped; its last window ends at word 1267)
   __shared__ __align__(16) uint32_t buf[WPB][1280];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const uint64_t w = (uint64_t)blockIdx.x * WPB + wi;
-  const uint64_t r = r0 + w / S;
-  if (r >= r1) return;  // whole warp; no CTA-wide barriers below
-  const int per = (NB + (int)S - 1) / (int)S;
-  const int b0 = (int)(w % S) * per, b1 = b0 + per < NB ? b0 + per : NB;
-  if (b0 >= b1) return;
+  const uint64_t r = (uint64_t)blockIdx.x * WPB + wi;
+  if (r >= n) return;  // whole warp; no CTA-wide barriers below
   uint32_t* B = buf[wi];
-  const uint32_t* src = state + (r - src_off) * 624;
-  for (int k = lane; k < 624; k += 32) B[k] = src[k];
+  uint32_t* const table = state + r * 624;
+  for (int k = lane; k < 624; k += 32) B[k] = table[k];
   for (int k = 1248 + lane; k < 1280; k += 32) B[k] = 0;
-  for (int b = 0; b < b0; b++) {   // to the segment's first block
-    __syncwarp();
-    mt_twist<OUT_U32, false>(B, lane, nullptr, 624, false);
-  }
   uint32_t acc[20];
 #pragma unroll
   for (int t = 0; t < 20; t++) acc[t] = 0;
-  for (int i0 = b0 * 624; i0 < b1 * 624 && i0 < D; i0 += 624) {
+  for (int i0 = 0; i0 < D; i0 += 624) {
     __syncwarp();
     for (int k = lane; k < 624; k += 32) B[624 + k] = B[k];
     __syncwarp();
@@ -484,36 +675,17 @@ __global__ void __launch_bounds__(WPB * 32) k_mt_poly_apply(const __grid_constan
     __syncwarp();
     for (int k = lane; k < 624; k += 32) B[k] = B[624 + k];
   }
-  uint32_t* dst = state + r * 624;
-  if (S == 1) {
 #pragma unroll
-    for (int t = 0; t < 20; t++)
-      if (20 * lane + t < 624) dst[20 * lane + t] = acc[t];
-  } else {
-#pragma unroll
-    for (int t = 0; t < 20; t++)
-      if (20 * lane + t < 624) atomicXor(dst + 20 * lane + t, acc[t]);
-  }
+  for (int t = 0; t < 20; t++)
+    if (20 * lane + t < 624) table[20 * lane + t] = acc[t];
 }
 
-cudaError_t launch_mt_poly_apply(const MtPoly& g, uint32_t* state, uint64_t r0, uint64_t r1,
-                                 uint64_t src_off, cudaStream_t s) {
-  if (r1 <= r0) return cudaSuccess;
+cudaError_t launch_mt_poly_apply(const MtPoly& g, uint32_t* state, uint64_t n, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
   constexpr int WPB = 4;
-  // Few tables: split each table's coefficient blocks over up to 32 warps
-  // (destination rows zeroed first), so that a pass keeps about 4096 warps
-  // busy.  In place (src_off = 0) needs the unsplit form.
-  const uint64_t tables = r1 - r0;
-  uint32_t S = 1;
-  if (src_off != 0)
-    while (S < 32 && tables * S < 4096) S *= 2;
-  if (S > 1) {
-    const cudaError_t e = cudaMemsetAsync(state + r0 * 624, 0, tables * 624 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-  }
-  const uint64_t blocks = (tables * S + WPB - 1) / WPB;
+  const uint64_t blocks = (n + WPB - 1) / WPB;
   if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-  k_mt_poly_apply<WPB><<<(unsigned)blocks, WPB * 32, 0, s>>>(g, state, r0, r1, src_off, S);
+  k_mt_poly_apply<WPB><<<(unsigned)blocks, WPB * 32, 0, s>>>(g, state, n);
   return cudaGetLastError();
 }
 
@@ -535,11 +707,20 @@ static cudaError_t launch_mt(const FillDesc& d, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_fill_mt_wide(const FillDesc& d, cudaStream_t s) {
+  if (d.n_rows == 0 || d.n_per == 0) return cudaSuccess;
+  if (d.n_rows > 0x7FFFFFFFull) return cudaErrorInvalidValue;
+  if (d.mode == OUT_F32) k_fill_mt_wide<OUT_F32><<<(unsigned)d.n_rows, 256, 0, s>>>(d);
+  else k_fill_mt_wide<OUT_U32><<<(unsigned)d.n_rows, 256, 0, s>>>(d);
+  return cudaGetLastError();
+}
+
 // Tile: threads per CTA (64, 128, 256; 32 with two streams per warp, so that
 // the CTAs of a large fill spread evenly over the SMs) and, in `stages`,
 // streams per warp.
 cudaError_t launch_fill_mt(const FillDesc& d, Tile t, cudaStream_t s) {
   if (d.n_rows == 0 || d.n_per == 0) return cudaSuccess;
+  if (t.threads == 256 && t.cols == 227 && (d.mode == OUT_U32 || d.mode == OUT_F32)) return launch_fill_mt_wide(d, s);
   return with_mode(d.mode, [&](auto m) {
     constexpr int OM = decltype(m)::value;
     if (t.stages == 2) {

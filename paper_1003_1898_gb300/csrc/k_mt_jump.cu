@@ -9,8 +9,7 @@
 // degree 19937.  On the state, T^k acts as g(T) for g = t^k mod phi; T drops
 // the low 31 bits of the window's oldest word (not part of the state), so
 // the jump applies g = t^(k-1) mod phi and then one more step, which makes
-// every word of the new table exact (the device kernel, k_mt_poly_apply,
-// does both at once).
+// every word of the new table exact (the device kernels do both at once).
 //
 //  * phi is found once per process by the Berlekamp-Massey algorithm on
 //    2 x 19937 output bits of a host MT19937, with bit-packed polynomials.
@@ -19,8 +18,8 @@
 //    terms (its second-highest exponent is 623 below the top, so a 64-bit
 //    chunk of high coefficients never lands in itself).
 //  * The single-sequence fill from init_genrand(x0): chunk starts by
-//    log2(C) doubling passes of the polynomial for (L 2^i), then the
-//    ordinary MT19937 fill kernel with one chunk per warp.
+//    log2(C) doubling passes of the polynomial for (L 2^i), each from the word
+//    sequences of the known starts, then the MT19937 fill with a CTA per chunk.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -206,36 +205,79 @@ MtPoly jump_poly(uint64_t k) {
 
 cudaError_t launch_skip_mt(uint32_t* state, uint64_t n, uint64_t k, cudaStream_t s) {
   if (n == 0 || k == 0) return cudaSuccess;
-  return launch_mt_poly_apply(jump_poly(k), state, 0, n, 0, s);
+  return launch_mt_poly_apply(jump_poly(k), state, n, s);
+}
+
+// Draws per chunk of a jump fill of n draws, a power of two (so that the jump
+// polynomials, t^(L 2^i - 1) with a squaring each, are the same few whatever n
+// is), from the measured costs in ns: a doubling pass about 17,000, a chunk's
+// start 250, a block of 624 draws 280 and 30 more for every chunk on the SM, or
+// 120 a chunk once they fill it.  n draws in us, a warp per chunk and up to 4,104
+// of them -> this: 10^5 194 -> 65, 5 10^5 533 -> 98, 1.8 10^7 1,648 -> 223, 2^28
+// 2,248 -> 673, 2^30 2,902 -> 1,676.
+static int jump_log2(uint64_t n) {
+  const uint64_t sms = (uint64_t)sm_count();
+  int best = 63;
+  uint64_t cost = ~0ull;
+  for (int lg = 10; lg < 63; lg++) {
+    const uint64_t C = ((n - 1) >> lg) + 1;
+    if (C > 4096) continue;
+    uint64_t passes = 0;
+    while ((1ull << passes) < C) passes++;
+    const uint64_t c = (C + sms - 1) / sms;
+    const uint64_t blocks = (C == 1 ? n : 1ull << lg) / 624 + 1;
+    const uint64_t ns = passes * 17000 + C * 250 + blocks * std::max(280 + 30 * c, 120 * c);
+    if (ns < cost) {
+      cost = ns;
+      best = lg;
+    }
+    if (C == 1) break;
+  }
+  return best;
 }
 
 cudaError_t launch_jump_mt(uint64_t x0, uint64_t first, uint64_t n, uint32_t n_chunks,
                            void* d_out, int mode, cudaStream_t s) {
-  // Every chunk costs one application of a jump polynomial, the bulk of the
-  // call.  A warp per chunk (the fill's full-warp tile) keeps the GPU as busy
-  // as two chunks per warp do, so more chunks than that many warps (27 per
-  // SM, one wave) are merged into longer ones: any contiguous cut of the one
-  // sequence gives the same output.
-  const uint32_t wave = 27u * (uint32_t)sm_count();
-  Tile tile = default_tile(MT19937, 0);
-  if (n_chunks > wave) {
-    n_chunks = wave;
-    tile = Tile{64, 624, 1};
-  }
-  const uint64_t L = (n + n_chunks - 1) / n_chunks;   // draws per chunk
-  const uint64_t C = (n + L - 1) / L;                 // chunks, none empty
+  // The chunks are the library's choice (any contiguous cut of the one sequence
+  // gives the same output): every chunk's start costs a polynomial product, and a
+  // CTA per chunk keeps the GPU busy with a few hundred of them.
+  (void)n_chunks;
+  const int lg = jump_log2(n);
+  uint64_t L = 1ull << lg;                            // draws per chunk
+  uint64_t C = ((n - 1) >> lg) + 1;                   // chunks, none empty
+  if (C == 1) L = n;
+  // Tables of the chunks and one more, then the sequences of those that others
+  // start from; without room for them, one chunk.
   HostMt mt;
   mt.init((uint32_t)x0);
   uint32_t* S = nullptr;
-  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&S), C * 624 * sizeof(uint32_t), s);
+  cudaError_t e;
+  for (;;) {
+    const uint64_t seqs = std::max<uint64_t>(C > 1 ? (C + 1) / 2 : 0, first > 0 ? 1 : 0);
+    e = scratch_alloc(reinterpret_cast<void**>(&S), ((C + 1) * 624 + 64 + seqs * kMtSeq) * sizeof(uint32_t), s);
+    if (e != cudaErrorMemoryAllocation || C == 1) break;
+    cudaGetLastError();
+    C = 1;
+    L = n;
+  }
   if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(S, mt.mt, sizeof(mt.mt), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && first > 0)   // the start table moved `first` words on, in place
-    e = launch_mt_poly_apply(jump_poly(first), S, 0, 1, 0, s);
+  uint32_t* const seq = S + ((C + 1) * 624 + 63) / 64 * 64;
+  e = cudaMemsetAsync(S, 0, (C + 1) * 624 * sizeof(uint32_t), s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(first > 0 ? S + C * 624 : S, mt.mt, sizeof(mt.mt), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && first > 0) {   // the start table moved `first` words on
+    e = launch_mt_sequence(S + C * 624, seq, 0, 1, s);
+    if (e == cudaSuccess) e = launch_mt_apply_seq(jump_poly(first), seq, S, 0, 1, s);
+  }
   // Pass i: chunks [2^i, 2^(i+1)) from chunks [0, 2^i), L 2^i outputs on.
+  uint64_t made = 0;                     // sequences
   int i = 0;
-  for (uint64_t half = 1; e == cudaSuccess && half < C; half <<= 1, i++)
-    e = launch_mt_poly_apply(jump_poly(L << i), S, half, std::min(2 * half, C), half, s);
+  for (uint64_t half = 1; e == cudaSuccess && half < C; half <<= 1, i++) {
+    const uint64_t rows = std::min(2 * half, C) - half;
+    e = launch_mt_sequence(S, seq, made, rows > made ? rows - made : 0, s);
+    made = std::max(made, rows);
+    if (e == cudaSuccess) e = launch_mt_apply_seq(jump_poly(L << i), seq, S, half, rows, s);
+  }
   if (e == cudaSuccess) {
     FillDesc d{};
     d.state = S;
@@ -246,7 +288,7 @@ cudaError_t launch_jump_mt(uint64_t x0, uint64_t first, uint64_t n, uint32_t n_c
     d.limit = n;
     d.pos = 624;          // fresh tables: the next output twists
     d.mode = mode;
-    e = launch_fill_mt(d, tile, s);
+    e = launch_fill_mt_wide(d, s);
   }
   const cudaError_t ef = scratch_free(S, s);
   return e != cudaSuccess ? e : ef;

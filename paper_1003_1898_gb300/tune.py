@@ -32,7 +32,7 @@ TILES = {
                     (128, 24, 1)],               # one tensor-core product per luxury cycle
     "ranmar": [(128, 128, 1), (256, 128, 1)],
     "mt19937": [(64, 624, 1), (128, 624, 1), (256, 624, 1), (32, 624, 2), (64, 624, 2),
-                (128, 624, 2), (256, 624, 2)],
+                (128, 624, 2), (256, 624, 2), (256, 227, 1)],   # 227: a CTA per stream
 }
 
 # Workload shapes the tiles are tuned for: the roofline bulk fill, and for
