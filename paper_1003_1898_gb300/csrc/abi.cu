@@ -320,6 +320,11 @@ int prng_ising_fused(prng_state* st, int8_t* d_spins, uint32_t L, uint32_t colou
   q.shift = kFloatShift[st->gen];
   q.t4 = t4;
   q.t8 = t8;
+  const uint64_t w4 = (uint64_t)t4 << q.shift, w8 = (uint64_t)t8 << q.shift;
+  q.below4 = (uint32_t)w4;
+  q.below8 = (uint32_t)w8;
+  q.always4 = w4 >> 32 ? 0xFEFEFEFEu : 0u;
+  q.always8 = w8 >> 32 ? 0xFEFEFEFEu : 0u;
   q.vec4 = (L % 8 == 0 && (reinterpret_cast<uintptr_t>(d_spins) & 7) == 0) ? 1u : 0u;
   const Tile t = fill_tile(st, d);
   const cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -58,6 +58,8 @@ struct IsingSink {
   uint32_t colour;     // sites with (x + y) % 2 == colour
   uint32_t shift;      // 24-bit acceptance value = draw >> shift
   uint32_t t4, t8;     // integer thresholds for dE = 4 and dE = 8
+  uint32_t below4, below8;     // the same on the whole draw: threshold << shift, 32 bits of it,
+  uint32_t always4, always8;   // and 0xFEFEFEFE where it is past them
   uint32_t vec4;       // L % 8 == 0 and spins 8-byte aligned: 4 aligned ranks as one 8-byte chunk
 };
 
@@ -295,6 +297,37 @@ __device__ __forceinline__ void ising_site(const IsingSink& q, uint32_t k, uint3
   if (dE <= 0 || (dE == 4 ? r < q.t4 : r < q.t8)) row[x] = (int8_t)(-s);
 }
 
+// m |= bit when d < t.
+__device__ __forceinline__ void or_if_below(uint32_t& m, uint32_t d, uint32_t t, uint32_t bit) {
+  asm("{\n\t"
+      ".reg .pred p;\n\t"
+      "setp.lt.u32 p, %1, %2;\n\t"
+      "@p or.b32 %0, %0, %3;\n\t"
+      "}"
+      : "+r"(m)
+      : "r"(d), "r"(t), "r"(bit));
+}
+
+// 0xFE in the bytes of the four sites c that flip, given their neighbours above
+// (u), below (n) and on either side (l, r) and their draws.
+__device__ __forceinline__ uint32_t ising_flips4(uint32_t c, uint32_t u, uint32_t n, uint32_t l, uint32_t r,
+                                                 uint4 d, uint32_t t4, uint32_t t8, uint32_t always4,
+                                                 uint32_t always8) {
+  uint32_t m4 = always4, m8 = always8;
+  or_if_below(m4, d.x, t4, 0x000000FEu);
+  or_if_below(m4, d.y, t4, 0x0000FE00u);
+  or_if_below(m4, d.z, t4, 0x00FE0000u);
+  or_if_below(m4, d.w, t4, 0xFE000000u);
+  or_if_below(m8, d.x, t8, 0x000000FEu);
+  or_if_below(m8, d.y, t8, 0x0000FE00u);
+  or_if_below(m8, d.z, t8, 0x00FE0000u);
+  or_if_below(m8, d.w, t8, 0xFE000000u);
+  const uint32_t any_v = (u ^ c) | (n ^ c), both_v = (u ^ c) & (n ^ c);
+  const uint32_t any_h = (l ^ c) | (r ^ c), both_h = (l ^ c) & (r ^ c);
+  const uint32_t any = any_v | any_h;
+  return both_v | both_h | (any_v & any_h) | (any & m4) | (~any & m8);
+}
+
 // The same update of the four sites of colour ranks k .. k+3, k % 4 == 0,
 // with L % 8 == 0: they lie in one row at bytes xb .. xb+7 (xb = 2 (k - y L/2),
 // a multiple of 8), every other byte, so the row chunk and the chunks above
@@ -309,29 +342,19 @@ __device__ __forceinline__ void ising_site4(const IsingSink& q, uint32_t k, uint
   const uint32_t par = (y + q.colour) & 1u;
   const uint32_t yu = y == 0 ? L - 1 : y - 1, yd = y + 1 == L ? 0 : y + 1;
   int8_t* row = q.spins + (uint64_t)y * L;
-  union B8 { uint2 v; int8_t c[8]; };
-  B8 C, U, D;
-  C.v = *reinterpret_cast<const uint2*>(row + xb);
-  U.v = *reinterpret_cast<const uint2*>(q.spins + (uint64_t)yu * L + xb);
-  D.v = *reinterpret_cast<const uint2*>(q.spins + (uint64_t)yd * L + xb);
-  const int side = par ? row[xb + 8 == L ? 0 : xb + 8] : row[xb == 0 ? L - 1 : xb - 1];
-  const uint32_t dr[4] = {v.x, v.y, v.z, v.w};
-  B8 O = C;
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-#pragma unroll
-    for (int p = 0; p < 2; p++) {
-      if ((uint32_t)p != par) continue;
-      const int bi = 2 * i + p;
-      const int s = C.c[bi];
-      const int l = bi == 0 ? side : C.c[bi - 1];
-      const int r = bi == 7 ? side : C.c[bi + 1];
-      const int dE = 2 * s * (U.c[bi] + D.c[bi] + l + r);
-      const uint32_t a = dr[i] >> q.shift;
-      if (dE <= 0 || (dE == 4 ? a < q.t4 : a < q.t8)) O.c[bi] = (int8_t)(-s);
-    }
-  }
-  *reinterpret_cast<uint2*>(row + xb) = O.v;
+  const uint2 C = *reinterpret_cast<const uint2*>(row + xb);
+  const uint2 U = *reinterpret_cast<const uint2*>(q.spins + (uint64_t)yu * L + xb);
+  const uint2 D = *reinterpret_cast<const uint2*>(q.spins + (uint64_t)yd * L + xb);
+  const uint32_t side = (uint8_t)(par ? row[xb + 8 == L ? 0 : xb + 8] : row[xb == 0 ? L - 1 : xb - 1]);
+  // Bytes of the colour (and, in the row itself, of the other one), in order; the
+  // other neighbour in the row one place before (even sites) or behind (odd ones).
+  const uint32_t mine = par ? 0x7531u : 0x6420u, other = par ? 0x6420u : 0x7531u;
+  const uint32_t c = __byte_perm(C.x, C.y, mine), o = __byte_perm(C.x, C.y, other);
+  const uint32_t s = __byte_perm(o, side, par ? 0x4321u : 0x2104u);
+  const uint32_t f = ising_flips4(c, __byte_perm(U.x, U.y, mine), __byte_perm(D.x, D.y, mine), o, s, v, q.below4,
+                                  q.below8, q.always4, q.always8);
+  *reinterpret_cast<uint2*>(row + xb) = make_uint2(C.x ^ __byte_perm(f, 0, par ? 0x1404u : 0x4140u),
+                                                   C.y ^ __byte_perm(f, 0, par ? 0x3424u : 0x4342u));
 }
 
 // Output of four consecutive draws (element index e of the first, at p) or

@@ -108,37 +108,6 @@ __device__ __forceinline__ uint32_t div_pow2(uint32_t a, uint32_t b) {
   return (b & (b - 1)) == 0 ? a >> (31 - __clz(b)) : a / b;
 }
 
-// m |= bit when d < t.
-__device__ __forceinline__ void or_if_below(uint32_t& m, uint32_t d, uint32_t t, uint32_t bit) {
-  asm("{\n\t"
-      ".reg .pred p;\n\t"
-      "setp.lt.u32 p, %1, %2;\n\t"
-      "@p or.b32 %0, %0, %3;\n\t"
-      "}"
-      : "+r"(m)
-      : "r"(d), "r"(t), "r"(bit));
-}
-
-// 0xFE in the bytes of the four sites c that flip, given their neighbours above
-// (u), below (n) and on either side (l, r) and their draws.
-__device__ __forceinline__ uint32_t ising_flips4(uint32_t c, uint32_t u, uint32_t n, uint32_t l, uint32_t r,
-                                                 uint4 d, uint32_t t4, uint32_t t8, uint32_t always4,
-                                                 uint32_t always8) {
-  uint32_t m4 = always4, m8 = always8;
-  or_if_below(m4, d.x, t4, 0x000000FEu);
-  or_if_below(m4, d.y, t4, 0x0000FE00u);
-  or_if_below(m4, d.z, t4, 0x00FE0000u);
-  or_if_below(m4, d.w, t4, 0xFE000000u);
-  or_if_below(m8, d.x, t8, 0x000000FEu);
-  or_if_below(m8, d.y, t8, 0x0000FE00u);
-  or_if_below(m8, d.z, t8, 0x00FE0000u);
-  or_if_below(m8, d.w, t8, 0xFE000000u);
-  const uint32_t any_v = (u ^ c) | (n ^ c), both_v = (u ^ c) & (n ^ c);
-  const uint32_t any_h = (l ^ c) | (r ^ c), both_h = (l ^ c) & (r ^ c);
-  const uint32_t any = any_v | any_h;
-  return both_v | both_h | (any_v & any_h) | (any & m4) | (~any & m8);
-}
-
 __global__ void __launch_bounds__(kIsingVecThreads) k_ising_half_sweep_v(const __grid_constant__ IsingLaunch b) {
   const uint32_t lo = ising_lattice_of(b);
   const prng_ising_req& q = b.r[lo];

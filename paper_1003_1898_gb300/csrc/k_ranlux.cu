@@ -34,7 +34,14 @@ PRNG_RANLUX_DECLARE(408)
 // whose short rows pay off later (4096^2 over 65,536 streams, 128 draws each, p =
 // 223: 50 / 55; over 4,096, 2,048 draws each, p = 389: 550 / 470).
 Tile ranlux_auto_tile(const FillDesc& d) {
+  // The borrow chain's own tile: the ring, but for short rows of many streams
+  // (131,072 x 64 at p = 24 27 / 23 us without it, x 248 41 / 37); in wide CTAs
+  // for long rows at p = 48 (131,072 x 8,192 781 / 714, 4,096 x 4,096 70 / 95).
   Tile t = ranlux_ring_ok(d) || d.p < 97 ? Tile{64, 56, 1} : Tile{64, 96, 1};
+  if (d.p < 97 && d.n_rows >= 32768) {
+    if (d.n_per < 320) t = Tile{64, 48, 1};
+    else if (d.p == 48 && d.n_rows >= 65536 && d.n_per >= 1024) t = Tile{256, 56, 1};
+  }
   if (d.p < kLuxTcMinP || d.n_per < 24) return t;
   const uint64_t nb = d.n_per / 24, p = (uint64_t)d.p, sms = (uint64_t)sm_count();
   auto product = [&](uint64_t tiles) {   // cycles of a product with `tiles` tiles to run

@@ -49,7 +49,7 @@ constexpr int kRanmarRing = 132;
 // sector).
 template <int NW, int OM, bool LIMITED>
 __device__ __forceinline__ void ranmar_warps(const FillDesc& d, uint64_t row0, int rows,
-                                             uint32_t* smem) {
+                                             uint32_t* smem, uint32_t* stage = nullptr) {
   constexpr int RS = kRanmarRing;
   const uint64_t nr = d.n_rows;
   for (int e = threadIdx.x; e < 98 * NW; e += NW * 32) {
@@ -108,6 +108,8 @@ __device__ __forceinline__ void ranmar_warps(const FillDesc& d, uint64_t row0, i
       const uint32_t b1 = __shfl_sync(0xFFFFFFFFu, vb, src + 1);
       st_pair<24>(orow + col0 + 2 * l, l < 16 ? a0 : a1, l < 16 ? b0 : b1);
     };
+    const bool quads = OM == OUT_ISING && d.ising.vec4 && (rbase & 3) == 0;
+    uint32_t* const mine = stage + 128 * w;
     uint64_t g = 0;
     for (; g + 128 <= n; g += 128) {
       uint32_t v[4];
@@ -118,7 +120,18 @@ __device__ __forceinline__ void ranmar_warps(const FillDesc& d, uint64_t row0, i
         __syncwarp();
         v[s] = out_word(y, s);
         if constexpr (OM != OUT_F64 || LIMITED)
-          if (store) emit(g + 32 * s, v[s], true);
+          if (store && !quads) emit(g + 32 * s, v[s], true);
+      }
+      if constexpr (OM == OUT_ISING) {
+        // Four consecutive sites per lane (their chunk of a lattice row updates as
+        // one), exchanged through the warp's 128 words of shared memory.
+        if (quads) {
+#pragma unroll
+          for (int s = 0; s < 4; s++) mine[32 * s + l] = v[s];
+          __syncwarp();
+          put4<OM, 24>(d, nullptr, rbase + g + 4 * l, *reinterpret_cast<const uint4*>(mine + 4 * l));
+          __syncwarp();
+        }
       }
       if constexpr (OM == OUT_F64 && !LIMITED) {
         if (store) {
@@ -164,9 +177,10 @@ __device__ __forceinline__ void ranmar_warps(const FillDesc& d, uint64_t row0, i
 template <int T, int OM>
 __global__ void __launch_bounds__(T) k_fill_ranmar(const FillDesc d) {
   __shared__ uint32_t smem[(T / 32) * kRanmarRing];
+  __shared__ __align__(16) uint32_t stage[OM == OUT_ISING ? (T / 32) * 128 : 4];
   const uint64_t row0 = (uint64_t)blockIdx.x * (T / 32);
   const uint64_t left = d.n_rows - row0;
-  ranmar_warps<T / 32, OM, false>(d, row0, left < (uint64_t)(T / 32) ? (int)left : T / 32, smem);
+  ranmar_warps<T / 32, OM, false>(d, row0, left < (uint64_t)(T / 32) ? (int)left : T / 32, smem, stage);
 }
 
 // Batched RANMAR fills: one block per item (up to T / 32 streams of one
