@@ -358,6 +358,32 @@ static cudaError_t launch_g(const FillDesc& d, Tile t, cudaStream_t s) {
   return launch_tk<G, 128, 32, 1>(d, s);
 }
 
+// Whether a plain XOR128 fill of these many streams and draws is faster cut into
+// segments of 64-column tiles, by the time a draw of every stream takes (ps).
+// Whole, a scheduler's warps decide: one per 19,456 streams, and the fullest
+// schedulers set the pace while others idle.  Cut to 131,072 threads and more the
+// schedulers are even and the stores run at their rate.  The starts and the
+// second launch cost about 16 us.  us, whole / cut, u32 and f64 (as many draws):
+// 32,768 x 4,096 97 / 108 and 184 / 124; 40,000 x 8,192 260 / 225 and 398 / 272;
+// 50,000 x 2,048 79 / 89 and 110 / 115; 65,536 x 4,096 203 / 188 and 250 / 223;
+// 65,536 x 16,384 759 / 662 and 956 / 818; 80,000 x 8,192 494 / 401 and 586 / 509;
+// 40,000 x 8,190 (unaligned) 612 / 424 and 928 / 557.
+static bool xor128_cut_pays(const FillDesc& d) {
+  const uint64_t w = (d.n_rows + 19455) / 19456;
+  uint64_t whole, cut;
+  if (d.mode == OUT_F64) {
+    whole = std::max<uint64_t>(41600, 14400 * w);
+    cut = 760 * d.n_rows / 1000;
+  } else if (d.mode == OUT_F32) {
+    whole = 3600 + 11000 * w;
+    cut = 630 * d.n_rows / 1000;
+  } else {
+    whole = 11400 * w;
+    cut = 620 * d.n_rows / 1000;
+  }
+  return whole > cut && d.n_per >= 16000000 / (whole - cut);
+}
+
 // A plain XOR128 fill of few streams as segments of L = 2^k draws, each a thread
 // of its own, whose starts T^(seg L) s come from xor128_starts first.  A thread
 // makes a draw in about 17 ns whatever the number of streams while those leave
@@ -367,14 +393,25 @@ static cudaError_t launch_g(const FillDesc& d, Tile t, cudaStream_t s) {
 // / cut: 256 x 4,096 u32 74 / 28, f64 (as many draws) 165 / 29; 256 x 8,192 135 /
 // 28; 4,096 x 4,096 73 / 38; 1,000 x 4,095 (unaligned) 427 / 41; 16,384 x 4,096
 // 73 / 71, f64 168 / 84; 4,096 x 1,024 26 / 33, which stays whole.
+// From 120 M draws on the stores bound it, and it takes 64-column tiles, whose
+// 256-byte row runs they like better, and up to 200,704 threads, as streams too
+// many for the first form do where xor128_cut_pays.  us, 65,536 threads of 32
+// columns / this: 4,096 x 65,536 u32 221 / 197, f64 271 / 238; 16,384 x 16,384
+// 214 / 191, 265 / 230; 30,000 x 4,096 113 / 102; 25,000 x 4,096 90 / 92 and
+// 12,000 x 8,192 89 / 104, below the line.
 static cudaError_t launch_xor128_segments(const FillDesc& d, bool& done, cudaStream_t s) {
   done = false;
-  if (d.n_rows >= 32768 || d.n_per < 900) return cudaSuccess;
-  const uint64_t want = std::min<uint64_t>(64, 65536 / d.n_rows);
+  if (d.n_rows >= 100352 || d.n_per < 900) return cudaSuccess;
+  const bool few = d.n_rows < 32768;
+  const bool wide = d.mode != OUT_ISING &&
+                    (few ? d.n_rows >= 2048 && d.n_per >= 120000000 / d.n_rows : xor128_cut_pays(d));
+  if (!few && !wide) return cudaSuccess;
+  const uint64_t want = std::min<uint64_t>(64, (wide ? 200704 : 65536) / d.n_rows);
   int lg = 6;
   while (lg < 57 && ((d.n_per - 1) >> lg) + 1 > want) lg++;
   const uint64_t L = 1ull << lg, segs = ((d.n_per - 1) >> lg) + 1;
-  if (lg > 56 || L >= d.n_per || d.n_per - L < 800 + 460 * d.n_rows * segs / 65536) return cudaSuccess;
+  if (lg > 56 || L >= d.n_per) return cudaSuccess;
+  if (!wide && d.n_per - L < 800 + 460 * d.n_rows * segs / 65536) return cudaSuccess;
   if (capturing(s)) return cudaSuccess;
   uint32_t* starts = nullptr;
   cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&starts), segs * 4 * d.n_rows * sizeof(uint32_t), s);
@@ -386,9 +423,15 @@ static cudaError_t launch_xor128_segments(const FillDesc& d, bool& done, cudaStr
   e = launch_xor128_starts(d.state, starts, d.n_rows, (uint32_t)segs, lg, s);
   if (e == cudaSuccess)
     e = with_mode(d.mode, [&](auto m) {
-      constexpr int T = 64, K = 32;
+      constexpr int OM = decltype(m)::value, T = 64, K = 32;
+      if constexpr (OM != OUT_ISING)
+        if (wide) {
+          const dim3 grid((unsigned)((d.n_rows + 2 * T - 1) / (2 * T)), (unsigned)segs);
+          k_fill_segments<Xor128Gen, 2 * T, 2 * K, 1, OM><<<grid, 2 * T, 4 * T * K * sizeof(uint32_t), s>>>(d, starts, L);
+          return cudaGetLastError();
+        }
       const dim3 grid((unsigned)((d.n_rows + T - 1) / T), (unsigned)segs);
-      k_fill_segments<Xor128Gen, T, K, 1, decltype(m)::value><<<grid, T, T * K * sizeof(uint32_t), s>>>(d, starts, L);
+      k_fill_segments<Xor128Gen, T, K, 1, OM><<<grid, T, T * K * sizeof(uint32_t), s>>>(d, starts, L);
       return cudaGetLastError();
     });
   const cudaError_t ef = scratch_free(starts, s);

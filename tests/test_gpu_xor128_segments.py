@@ -70,3 +70,44 @@ def test_segments():
     r = subprocess.run([sys.executable, "-c", CHILD.format(root=root)], capture_output=True, text=True, timeout=300,
                        cwd=root)
     assert r.returncode == 0 and "segments ok" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
+
+
+WIDE = '''
+import sys; sys.path.insert(0, {root!r})
+import numpy as np, torch, oracle
+import paper_1003_1898_gb300 as P
+# enough draws for the wide segments: streams x draws, then a short call from the states left
+for ns, n, kind in ((2048, 65000, "u32"), (32767, 4099, "f32"), (33001, 5000, "f32"), (40000, 6001, "u32"),
+                    (65537, 4500, "u32"), (32768, 4096, "f64"), (98304, 3072, "f64"), (100351, 2100, "f64")):
+    h = P.prng_create("xor128", 84, ns, 0)
+    f64 = kind == "f64"
+    ty = dict(u32=torch.int32, f32=torch.float32, f64=torch.float64)[kind]
+    fill = dict(u32=P.prng_fill_u32, f32=P.prng_fill_f32, f64=P.prng_fill_f64)[kind]
+    per = n // 2 if f64 else n
+    out = torch.full((ns * per + 8,), -7, dtype=ty, device="cuda")
+    fill(h, out, per)
+    tail = torch.empty((ns, 8), dtype=torch.int32, device="cuda")
+    P.prng_fill_u32(h, tail, 8)
+    assert torch.all(out[ns * per:] == -7)
+    got = out[:ns * per].view(ns, per)
+    for r0 in (0, ns // 2 - 65, ns - 130):
+        ref = oracle.fill("xor128", 84 + r0, 130, n + 8)
+        if f64:
+            want = oracle.fill_f64("xor128", 84 + r0, 130, per)
+        else:
+            want = oracle.to_f32("xor128", ref[:, :n]) if kind == "f32" else ref[:, :n].view(np.int32)
+        np.testing.assert_array_equal(got[r0:r0 + 130].cpu().numpy(), want)
+        np.testing.assert_array_equal(tail[r0:r0 + 130].cpu().numpy().view(np.uint32), ref[:, n:])
+    P.prng_destroy(h)
+print("wide ok")
+'''
+
+
+def test_wide_segments():
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", WIDE.format(root=root)], capture_output=True, text=True, timeout=300,
+                       cwd=root)
+    assert r.returncode == 0 and "wide ok" in r.stdout, r.stdout[-2000:] + r.stderr[-4000:]
