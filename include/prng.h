@@ -303,7 +303,7 @@ int prng_float_shift(prng_gen_t gen, uint32_t *shift);
  * what prng_batch_create + one prng_batch_launch + prng_batch_destroy do
  * for the same requests -- the same draws, the same handle advance -- but
  * its descriptors, work items and work counters live in one fixed device
- * array inside the library (about 2.4 MB, held on every device that loads
+ * array inside the library (about 2.7 MB, held on every device that loads
  * the library until the process exits), staged through a fixed host
  * buffer, and its kernels run one after the other on `stream`.
  *   - At most PRNG_NOALLOC_MAX_REQUESTS requests and PRNG_NOALLOC_MAX_ITEMS
