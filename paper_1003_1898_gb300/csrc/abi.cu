@@ -32,9 +32,13 @@ constexpr uint32_t kBlobVersion = 1u;
 //   MT19937, two streams per warp once there are enough to fill the GPU so (f64
 //   keeps a warp per stream, 1,035 / 1,056): in CTAs of a warp for short rows,
 //   8,192 x 64 24 / 17, x 1,000 30 / 22, 6,000 x 5,000 41 / 35; of two for long
-//   ones, 8,192 x 131,072 728 / 678 (one warp 685).  A CTA per stream while they
+//   ones, 8,192 x 131,072 728 / 678 (one warp 685).  But a scheduler holds whole
+//   warps, and an odd number of streams each leaves half a warp idle in the
+//   paired form: long rows then keep a warp per stream (that / paired, x 60,000:
+//   2,729 142 / 154, 4,096 186 / 194, 3,648 (even) 164 / 150), until from 14 on the
+//   half warp is lost among them (9,000 366 / 360).  A CTA per stream while they
 //   are few: 1 x 100,000 99 / 48, 456 x 65,536 71 / 49, 256 x 4,096 19 / 14, 1,024
-//   x 20,000 37 / 36.
+//   x 20,000 37 / 36, but 1,024 x 60,000 76 / 82 (800 77 / 73).
 Tile fill_tile(const prng_state* st, const FillDesc& d) {
   if (!tile_chosen(st->gen, st->p)) switch (st->gen) {
     case RANLUX: return ranlux_auto_tile(d);
@@ -45,9 +49,13 @@ Tile fill_tile(const prng_state* st, const FillDesc& d) {
       if (d.n_rows >= 32768 && d.n_per >= 4096) return Tile{128, 128, 1};
       break;
     case MT19937:
-      if (d.n_rows <= 1024 && d.n_per >= 512 && (d.mode == OUT_U32 || d.mode == OUT_F32)) return Tile{256, 227, 1};
-      if (d.n_rows >= 2048 && (d.mode == OUT_U32 || d.mode == OUT_F32))
+      if (d.mode != OUT_U32 && d.mode != OUT_F32) break;
+      if (d.n_per >= 512 && d.n_rows <= (d.n_per < 30000 ? 1024 : 912)) return Tile{256, 227, 1};
+      if (d.n_rows >= 2048) {
+        const uint64_t scheds = 4 * (uint64_t)sm_count(), w = (d.n_rows + scheds - 1) / scheds;
+        if (d.n_per >= 10000 && w < 14 && w % 2 == 1) return Tile{64, 624, 1};
         return d.n_per < 20000 ? Tile{32, 624, 2} : Tile{64, 624, 2};
+      }
       break;
     default: break;
   }
