@@ -11,8 +11,24 @@
 
 namespace prng {
 
+// Whether a batch's requests of a RANLUX family are faster on the tensor cores, in
+// cycles: the chain by its longest stream or by its warps' throughput, as for a
+// plain fill (ranlux_auto_tile), against two launches, the starts and the
+// products.  us, tensor cores / chain, in back-to-back serving ticks of 4,096 streams
+// a client: 1 client 25 / 19, 4 83 / 70, 12 109 / 95; 6, one of them
+// with a long fill, 180 / 487.
+inline bool lux_tensor_pays(int p, const LuxSplit& sp, uint64_t warp_blocks, uint64_t longest) {
+  const uint64_t sms = (uint64_t)sm_count();
+  const uint64_t chain = std::max<uint64_t>(longest * ((49 * p + 5900) / 10),
+                                            warp_blocks * ((17 * p + 1120) / 4) / (4 * sms));
+  const uint64_t len = sp.cut ? std::min<uint64_t>(longest, 1ull << sp.lgb) : longest;
+  const uint64_t product = std::max<uint64_t>(len * 1712, warp_blocks * 2873 / (16 * sms));
+  return chain > 30000 + product;
+}
+
 struct ItemPlan {
   bool tensor = true;            // false: RANLUX on the borrow chain (no room for the segments' starts)
+  bool lux_pays[FAM_COUNT];      // RANLUX families worth the tensor cores
   Tile tile[FAM_COUNT];
   LuxSplit split[FAM_COUNT];     // tensor-core families
   uint32_t max_seg[FAM_COUNT] = {};
@@ -20,11 +36,14 @@ struct ItemPlan {
   uint32_t ranmar_seed_rows = 256;
 
   ItemPlan() {
-    for (int f = 0; f < FAM_COUNT; f++) tile[f] = tile_of(f);
+    for (int f = 0; f < FAM_COUNT; f++) {
+      tile[f] = tile_of(f);
+      lux_pays[f] = true;
+    }
   }
   // RANLUX families whose fills run on the tensor cores.
   bool is_lux_tc(int f) const {
-    return tensor && kind_of(f) >= FAM_LUX24 && kind_of(f) < FAM_KINDS && lux_p_of(f) >= kLuxTcMinP;
+    return tensor && lux_pays[f] && kind_of(f) >= FAM_LUX24 && kind_of(f) < FAM_KINDS && lux_p_of(f) >= kLuxTcMinP;
   }
   // The segment length of every tensor-core family, from all its requests;
   // without `cut` each stream is one segment and MT19937 items are coarser.
@@ -33,6 +52,7 @@ struct ItemPlan {
     const bool fine = cut && !tile_chosen(XOR128, 0);
     tile[FAM_XOR128] = tile[FAM_XOR128 + FAM_F32] = fine ? Tile{64, 32, 1} : tile_of(FAM_XOR128);
     ranmar_seed_rows = cut ? 16 : 256;
+    for (int f = 0; f < FAM_COUNT; f++) lux_pays[f] = true;
     uint64_t wb[FAM_COUNT] = {}, longest[FAM_COUNT] = {};
     for (uint32_t i = 0; i < n; i++) {
       if (reqs[i].n_per_stream == 0) continue;
@@ -47,6 +67,11 @@ struct ItemPlan {
       max_seg[f] = 0;
       if (cut && longest[f] > 0) split[f] = lux_split(wb[f], longest[f]);
       if (split[f].cut) max_seg[f] = (uint32_t)(segments(f, 24 * longest[f]) - 1);
+      if (is_lux_tc(f) && !lux_tensor_pays(lux_p_of(f), split[f], wb[f], longest[f])) {
+        lux_pays[f] = false;
+        split[f] = LuxSplit{};
+        max_seg[f] = 0;
+      }
     }
   }
   // Segments of a request of n draws per stream.  (A start inside a block can

@@ -178,3 +178,22 @@ def test_batches_of_segments(lux):
         (P.prng_batcher_destroy if batcher else P.prng_batch_destroy)(b)
         for h in hs:
             P.prng_destroy(h)
+
+
+@pytest.mark.parametrize("per", [20, 24 * 8, 24 * 24 + 5, 24 * 40])
+def test_batch_on_either_side_of_the_line(per):
+    # Short requests stay on the borrow chain, long ones take the products.
+    ns = 33
+    ref = oracle.fill("ranlux", 91, ns, 3 * per, luxury=223)
+    h = P.prng_create("ranlux", 91, ns, 223)
+    out = torch.empty(ns * per, dtype=torch.int32, device="cuda")
+    reqs = [{"st": h, "d_out": out, "n_per_stream": per, "n_valid": 0, "f32": False}]
+    batch, batcher = P.prng_batch_create(reqs), P.prng_batcher_create(1, 64)
+    for k in range(3):
+        P.prng_batch_launch(batch) if k != 1 else P.prng_batcher_launch(batcher, reqs)
+        got = out.cpu().numpy().view(np.uint32).reshape(ns, per)
+        np.testing.assert_array_equal(got, ref[:, k * per:(k + 1) * per])
+    torch.cuda.synchronize()
+    P.prng_batch_destroy(batch)
+    P.prng_batcher_destroy(batcher)
+    P.prng_destroy(h)
