@@ -637,16 +637,8 @@ __device__ __forceinline__ void lux_head(uint32_t (&V)[24], uint32_t& c, int h, 
   for (int j = 0; j < 24; j++) V[j] = scratch[j + ph < 24 ? j + ph : j + ph - 24];
 }
 
-struct LuxPlan {   // a row's pieces: h draws that finish an open block, nb blocks, m < 24 more
-  uint64_t nb;
-  int h, m;
-  __device__ __forceinline__ LuxPlan(const FillDesc& d) {
-    const uint64_t n = d.n_per;
-    const uint64_t left = d.pos < 24 ? 24 - d.pos : 0;
-    h = (int)(left < n ? left : n);
-    nb = (n - h) / 24;
-    m = (int)(n - h - 24 * nb);
-  }
+struct LuxPlan : LuxPieces {
+  __device__ __forceinline__ explicit LuxPlan(const FillDesc& d) : LuxPieces(d.n_per, d.pos) {}
 };
 
 // State of row `row` at a block's end, R and its carry, and what of it a tail of
@@ -947,9 +939,6 @@ constexpr uint32_t kHeadWords = sizeof(LuxHead) / 4, kHeadPitch = 64;
 static_assert(sizeof(LuxHead) % 4 == 0 && kHeadWords <= kHeadPitch, "copied as words by two lanes' turns");
 constexpr uint32_t kStartWords = kHeadPitch + 19 * 32;
 
-constexpr int kLgGroup = 4, kGroup = (int)kLuxGroup;
-static_assert(kGroup == 1 << kLgGroup, "");
-
 // Head of item `it`, by its warp.
 __device__ __forceinline__ void lux_head_of(const LuxJob& job, uint32_t it, LuxHead* h) {
   const int lane = threadIdx.x & 31;
@@ -986,7 +975,7 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
   const uint32_t it = !have                 ? 0
                       : job.firsts != nullptr ? job.firsts[g]
                       : job.reqs != nullptr   ? g
-                                              : g / job.warps * kGroup * job.warps + g % job.warps;
+                                              : lux_first_item(g, job.warps);
   lux_setup(sh);
 
   uint32_t N[18];
@@ -999,8 +988,8 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
     const bool active = row < d.n_rows;
     seg = heads[wi].seg;
     const LuxPlan plan(d);
-    const uint64_t segs = job.max_seg > 0 ? ((d.n_per / 24 + (1ull << job.lgb) - 1) >> job.lgb) : 1;
-    cnt = segs > seg + kGroup ? kGroup : segs > seg ? (uint32_t)(segs - seg) : 1u;
+    // As many as the host counted when it sized the items: from the same function.
+    cnt = lux_group_size(job.max_seg > 0 ? lux_segments(d.n_per, job.lgb) : 1, seg);
     warps = (uint32_t)((d.n_rows + 31) / 32);
     uint32_t V[24], c;
     lux_state(d, row, active, V, c);
@@ -1028,11 +1017,11 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
   bool ok = true;
   uint32_t products = 0;
   // To the group's first segment, by the bits of its number.
-  const uint32_t group = have ? seg / kGroup : 0;
+  const uint32_t group = have ? seg / kLuxGroup : 0;
   for (int i = 0; __syncthreads_or((group >> i) != 0); i++) {
     const bool take = (group >> i) & 1u;
     if (!__syncthreads_or(take)) continue;          // also: the operand is not in use any more
-    lux_operand(sh, level, job.lgb + kLgGroup + i);
+    lux_operand(sh, level, job.lgb + kLgLuxGroup + i);
     if (!lux_issue(sh, tm, N, !ok)) break;
     uint32_t T[18];
     ok = lux_take(sh, tm, products & 1u, T) && ok;
@@ -1045,7 +1034,7 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
   // Segment after segment.
   if (__syncthreads_or(cnt > 1)) lux_operand(sh, level, job.lgb);
   for (uint32_t j = 0;; j++) {
-    if (j < cnt) {
+    if (j < cnt && it + j * warps < job.n_items) {
       uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords;
       if (lane == 0) heads[wi].seg = seg + j;
       __syncwarp();
@@ -1321,7 +1310,7 @@ LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest) {
   LuxSplit sp;
   while (sp.lgb < 40 && (1ull << sp.lgb) < want) sp.lgb++;
   // Group g starts by powers lgb + 4 .. lgb + 4 + log2(g).
-  while ((longest >> sp.lgb >> kLgGroup >> std::max(0, kPowers - kLgGroup - sp.lgb)) != 0) sp.lgb++;
+  while ((longest >> sp.lgb >> kLgLuxGroup >> std::max(0, kPowers - kLgLuxGroup - sp.lgb)) != 0) sp.lgb++;
   sp.cut = longest > 1ull << sp.lgb;
   return sp;
 }
@@ -1345,15 +1334,14 @@ cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s) {
 // A plain fill cut into segments (scratch for their starts from the retained pool).
 static cudaError_t launch_segments(const FillDesc& d, const LuxSplit& sp, cudaStream_t s) {
   LuxJob job{};
-  const uint64_t nb = (d.n_per - std::min<uint64_t>(d.n_per, d.pos < 24 ? 24 - d.pos : 0)) / 24;
-  const uint64_t warps = (d.n_rows + 31) / 32, segs = std::max<uint64_t>(1, (nb + (1ull << sp.lgb) - 1) >> sp.lgb);
+  const uint64_t warps = (d.n_rows + 31) / 32, segs = lux_segments(d.n_per, sp.lgb);
   if (warps * segs > 0x7FFFFFFFull) return cudaErrorInvalidValue;
   job.one = d;
   job.warps = (uint32_t)warps;
   job.n_items = (uint32_t)(warps * segs);
   job.lgb = sp.lgb;
   job.max_seg = (uint32_t)segs - 1;
-  job.n_groups = (uint32_t)(warps * ((segs + kGroup - 1) / kGroup));
+  job.n_groups = (uint32_t)lux_groups(segs, warps);
   job.tiles = lux_out_map(d.out, d.pitch, d.n_rows, &job.map) ? 1 : 0;
   cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&job.starts), lux_start_bytes(job.n_items), s);
   if (e != cudaSuccess) return e;

@@ -74,13 +74,8 @@ struct ItemPlan {
       }
     }
   }
-  // Segments of a request of n draws per stream.  (A start inside a block can
-  // leave one block fewer than n / 24; a segment past the last block is skipped.)
-  uint64_t segments(int f, uint64_t n) const {
-    if (!split[f].cut) return 1;
-    const uint64_t B = 1ull << split[f].lgb;
-    return std::max<uint64_t>(1, (n / 24 + B - 1) / B);
-  }
+  // Segments of a request of n draws per stream.
+  uint64_t segments(int f, uint64_t n) const { return split[f].cut ? lux_segments(n, split[f].lgb) : 1; }
   // Streams per re-seeding item.
   uint32_t seed_rows(const prng_state* st) const { return st->gen == RANMAR ? ranmar_seed_rows : 256u; }
   uint32_t rows(int f) const { return kind_of(f) == FAM_MT ? mt_rows : rows_per_item(f, tile[f]); }

@@ -3,6 +3,7 @@
 
 #include <cuda.h>
 
+#include "lux_plan.cuh"
 #include "ranlux.cuh"
 
 namespace prng {
@@ -40,9 +41,6 @@ struct LuxJob {
   uint32_t n_items, n_groups, warps, max_seg, tiles;
   int lgb;                  // segments of 2^lgb blocks; all of a stream when max_seg = 0
 };
-// Segments whose starts one row walks after one another.
-constexpr uint32_t kLuxGroup = 16;
-
 cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s);
 uint64_t lux_start_bytes(uint64_t items);
 

@@ -1,0 +1,33 @@
+"""RANLUX fills at the edges of their division into segments and tiles."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1003_1898_gb300 as P  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1003_1898_gb300 import build
+    build.build()
+    P.lib()
+
+
+@pytest.mark.parametrize("ns,per", [(256, 984), (4096, 984), (33, 24 * 8 * 5 + 24), (1, 24 * 8 * 17 + 12)])
+def test_fresh_rows_one_block_past_whole_segments(ns, per):
+    # An open block of a whole 24 draws leaves one block fewer to cut.
+    ref = oracle.fill("ranlux", 5, ns, 2 * per, luxury=223)
+    h = P.prng_create("ranlux", 5, ns, 223)
+    try:
+        for k in range(2):
+            out = torch.empty((ns, per), dtype=torch.int32, device="cuda")
+            P.prng_fill_u32(h, out, per)
+            np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), ref[:, k * per:(k + 1) * per])
+    finally:
+        P.prng_destroy(h)
