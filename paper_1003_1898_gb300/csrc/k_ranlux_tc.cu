@@ -42,10 +42,8 @@ namespace {
 
 constexpr int kLevels = 6;   // p >= kLuxTcMinP
 constexpr int kLevelP[kLevels] = {97, 223, 389, 120, 240, 408};
-// Operands per level: 2^i luxury cycles, i < kPowers (0: the fill's own; the
+// Operands per level: 2^i luxury cycles, i < kLuxPowers (0: the fill's own; the
 // others move a segment's start along its stream).
-constexpr int kPowers = 24;
-
 constexpr int kNK = 80;                       // K and N of the product: 72 bytes, constants, padding
 constexpr int kTabBytes = kNK * kNK * 2;      // the f16 operand, in core-matrix order
 constexpr uint32_t kKStep = (kNK / 8) * 128;  // bytes between core matrices along K
@@ -54,8 +52,8 @@ constexpr uint32_t kMagic = 0x3F000000u;      // pattern of 2^23 x 2^-24
 
 constexpr int kTmemCols = 128, kColD = 0, kColA = 80;
 
-// Filled on a device's first RANLUX handle (1.8 MB).
-__device__ uint4 g_tab[kLevels][kPowers][kTabBytes / 16];
+// Filled on a device's first RANLUX handle (2.4 MB).
+__device__ uint4 g_tab[kLevels][kLuxPowers][kTabBytes / 16];
 // Set when a kernel gave up waiting for the tensor core (never seen).
 __device__ uint32_t g_stuck;
 
@@ -186,17 +184,10 @@ void build_tab(const Big& a, uint16_t* tab) {
 
 }  // namespace
 
-// Fill the current device's operands once (bounded: one static array).
-cudaError_t lux_tables_init() {
-  static std::mutex lock;
-  static bool done[64] = {};
+// The operands of every level and power (bounded: one array, built once per
+// process; the caller holds the lock of lux_tables_init).
+const std::vector<uint16_t>& lux_host_tables() {
   static std::vector<uint16_t> host;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> guard(lock);
-  if (done[dev]) return cudaSuccess;
   if (host.empty()) {
     // (m - 1) / b = b^23 - b^9, so b (b^23 - b^9) = -1 and b^{-1} = m - b^23 + b^9 (mod m).
     Big one{};
@@ -211,19 +202,34 @@ cudaError_t lux_tables_init() {
       c >>= 32;
     }
     const Big binv = mod_m(v);
-    host.resize((size_t)kLevels * kPowers * kTabBytes / 2);
+    std::vector<uint16_t> t((size_t)kLevels * kLuxPowers * kTabBytes / 2);
     for (int l = 0; l < kLevels; l++) {
       Big a = one, s = binv;
       for (int k = kLevelP[l]; k; k >>= 1) {
         if (k & 1) a = mul_m(a, s);
         s = mul_m(s, s);
       }
-      for (int i = 0; i < kPowers; i++) {
-        build_tab(a, host.data() + (size_t)(l * kPowers + i) * kTabBytes / 2);
+      for (int i = 0; i < kLuxPowers; i++) {
+        build_tab(a, t.data() + (size_t)(l * kLuxPowers + i) * kTabBytes / 2);
         a = mul_m(a, a);
       }
     }
+    host.swap(t);
   }
+  return host;
+}
+
+// Fill the current device's operands once.
+cudaError_t lux_tables_init() {
+  static std::mutex lock;
+  static bool done[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> guard(lock);
+  if (done[dev]) return cudaSuccess;
+  const std::vector<uint16_t>& host = lux_host_tables();
   e = cudaMemcpyToSymbol(g_tab, host.data(), host.size() * 2);
   if (e == cudaSuccess) done[dev] = true;
   return e;
@@ -1302,17 +1308,7 @@ bool lux_out_map(void* out, uint64_t pitch, uint64_t rows, CUtensorMap* map) {
 uint64_t lux_start_bytes(uint64_t items) { return items * kStartWords * sizeof(uint32_t); }
 
 LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest) {
-  // Four CTAs per SM of four warps each.  Few blocks: a segment for each of those
-  // warps, of 8 blocks at least (a segment's start costs about three).  Many: three
-  // or four segments per warp, which even out the last wave.
-  const uint64_t slots = 16 * (uint64_t)sm_count(), share = warp_blocks / slots;
-  const uint64_t want = share < 24 ? std::max<uint64_t>(8, share + 1) : std::max<uint64_t>(16, share / 4);
-  LuxSplit sp;
-  while (sp.lgb < 40 && (1ull << sp.lgb) < want) sp.lgb++;
-  // Group g starts by powers lgb + 4 .. lgb + 4 + log2(g).
-  while ((longest >> sp.lgb >> kLgLuxGroup >> std::max(0, kPowers - kLgLuxGroup - sp.lgb)) != 0) sp.lgb++;
-  sp.cut = longest > 1ull << sp.lgb;
-  return sp;
+  return lux_split(warp_blocks, longest, (uint64_t)sm_count());
 }
 
 cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s) {

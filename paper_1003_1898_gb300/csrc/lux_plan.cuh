@@ -14,6 +14,9 @@
 
 namespace prng {
 
+// Multiplier operands per level: one for 2^i luxury cycles each, i < kLuxPowers.
+constexpr int kLuxPowers = 32;
+
 // Segments whose starts one row walks after one another.
 constexpr int kLgLuxGroup = 4;
 constexpr uint32_t kLuxGroup = 1u << kLgLuxGroup;
@@ -30,6 +33,29 @@ struct LuxPieces {
     m = (int)(n - h - 24 * nb);
   }
 };
+
+// How long the segments are of fills that have warp_blocks blocks in all (per 32
+// streams) and `longest` blocks in the longest stream, on `sms` SMs; cut: whether
+// any stream is.
+struct LuxSplit {
+  int lgb = 0;
+  bool cut = false;
+};
+PRNG_HD LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest, uint64_t sms) {
+  // Four CTAs per SM of four warps each.  Few blocks: a segment for each of those
+  // warps, of 8 blocks at least (a segment's start costs about three).  Many: three
+  // or four segments per warp, which even out the last wave.
+  const uint64_t slots = 16 * sms, share = warp_blocks / slots;
+  const uint64_t want = share < 24 ? (share + 1 > 8 ? share + 1 : 8) : (share / 4 > 16 ? share / 4 : 16);
+  LuxSplit sp;
+  while (sp.lgb < 40 && (1ull << sp.lgb) < want) sp.lgb++;
+  // A segment's start is lgb cycles' power after the one before, group g's first
+  // start the powers lgb + 4 .. lgb + 4 + log2(g): all below kLuxPowers while the
+  // stream has fewer than 2^kLuxPowers blocks.  Longer ones (10^11 draws a stream
+  // and up) stay whole.
+  sp.cut = longest > 1ull << sp.lgb && longest >> kLuxPowers == 0;
+  return sp;
+}
 
 // Segments of 2^lgb blocks that a row of n draws is cut into, wherever its first
 // block starts: an open block can leave one block fewer than n / 24, and a last

@@ -44,12 +44,7 @@ struct LuxJob {
 cudaError_t launch_lux_job(const LuxJob& job, int p, int mode, cudaStream_t s);
 uint64_t lux_start_bytes(uint64_t items);
 
-// How long the segments are of fills that have warp_blocks blocks in all (per 32
-// streams) and `longest` blocks in the longest stream; cut: whether any stream is.
-struct LuxSplit {
-  int lgb = 0;
-  bool cut = false;
-};
+// The split on the current device.
 LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest);
 
 // The tensor map of an output as a rows x pitch array of words in tiles of 32 x

@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -39,6 +40,13 @@ extern "C" int walk(uint64_t n, uint32_t pos, uint64_t rows, int lgb) {
   if (p.h + 24 * p.nb + p.m != n || p.m >= 24) return 6;
   return segs << lgb >= p.nb ? 0 : 7;
 }
+
+// log2 of the segments' blocks on 152 SMs, or -1 when the streams stay whole.
+extern "C" int split(uint64_t warp_blocks, uint64_t longest) {
+  const LuxSplit s = lux_split(warp_blocks, longest, 152);
+  return s.cut ? s.lgb : -1;
+}
+extern "C" int powers() { return kLuxPowers; }
 """
 
 
@@ -52,6 +60,7 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_1003_1898_gb300", "csrc"), str(src), "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.walk.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int]
+    L.split.argtypes = [ctypes.c_uint64, ctypes.c_uint64]
     return L
 
 
@@ -71,3 +80,51 @@ def test_segment_starts_stay_in_their_scratch(lib, pos):
 @pytest.mark.parametrize("rows,n,lgb", [(256, 984, 3), (4096, 984, 3), (1, 24, 3), (1, 1, 3)])
 def test_fresh_handles(lib, rows, n, lgb):
     assert lib.walk(n, 0, rows, lgb) == 0
+
+
+@pytest.mark.parametrize("warps", [1, 8, 4096, 2**27])
+def test_every_power_of_a_cut_fill_has_an_operand(lib, warps):
+    # A segment's start takes the power lgb, group g's first one lgb + 4 + (the bits of g).
+    powers = lib.powers()
+    for e in range(3, 64):
+        for longest in (2**e - 1, 2**e, 2**e + 1, 3 * 2**e // 2):
+            if longest * warps >= 2**64:
+                continue
+            lgb = lib.split(warps * longest, longest)
+            if lgb < 0:
+                continue
+            segs = -(-longest // 2**lgb)
+            used = [lgb] + [lgb + 4 + i for i in range(((segs - 1) >> 4).bit_length())]
+            assert max(used) < powers, (longest, lgb)
+            assert segs * warps < 2**31
+
+
+def test_long_streams_are_cut_as_finely_as_shorter_ones(lib):
+    # One stream: from 2^20 blocks on (a share of more than 24 per warp) at least a
+    # segment for each of the GPU's 16 x 152 warps.
+    for e in range(20, 32):
+        lgb = lib.split(2**e, 2**e)
+        assert lgb >= 0 and 2**e >> lgb >= 2432, e
+
+
+def test_operands_are_the_powers_of_the_luxury_cycle():
+    """Column k < 72 of power i at level p: the bytes of 256^k b^(-p 2^i) mod m."""
+    from paper_1003_1898_gb300 import build
+    L = ctypes.CDLL(build.build())
+    f = L._ZN4prng15lux_host_tablesEv
+    f.restype = ctypes.POINTER(ctypes.c_void_p * 2)              # a vector: begin, end
+    begin, end = f().contents
+    tab = np.ctypeslib.as_array(ctypes.cast(begin, ctypes.POINTER(ctypes.c_uint16)), ((end - begin) // 2,))
+    levels, K = (97, 223, 389, 120, 240, 408), 80
+    tab = tab.reshape(len(levels), -1, K // 8, K // 8, 8, 8)      # level, power, k / 8, n / 8, n % 8, k % 8
+    assert tab.shape[1] == 32
+    b = 2**24
+    m = b**24 - b**10 + 1
+    for l, p in enumerate(levels):
+        a = pow(b, -p, m)
+        for i in range(32):
+            got = tab[l, i].transpose(1, 2, 0, 3).reshape(K, K).view(np.float16)   # [n][k]
+            for k in (0, 1, 37, 71):
+                want = (pow(256, k, m) * a % m).to_bytes(72, "little")
+                np.testing.assert_array_equal(got[:72, k], np.frombuffer(want, np.uint8), err_msg=f"p {p} power {i}")
+            a = a * a % m
