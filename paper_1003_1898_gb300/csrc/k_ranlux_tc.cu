@@ -1287,8 +1287,8 @@ bool lux_out_map(void* out, uint64_t pitch, uint64_t rows, CUtensorMap* map) {
       f = nullptr;
     return reinterpret_cast<Encode>(f);
   }();
-  if (encode == nullptr || out == nullptr || (reinterpret_cast<uintptr_t>(out) & 15) != 0 || (pitch & 3) != 0 ||
-      pitch == 0 || rows == 0 || pitch >= 1ull << 32 || rows >= 1ull << 32)
+  if (encode == nullptr || out == nullptr || (reinterpret_cast<uintptr_t>(out) & 15) != 0 ||
+      !lux_tiles_reach(pitch, rows))
     return false;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, out) != cudaSuccess) {

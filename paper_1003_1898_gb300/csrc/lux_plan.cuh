@@ -75,4 +75,11 @@ PRNG_HD uint32_t lux_group_size(uint64_t segs, uint32_t seg) {
 PRNG_HD uint32_t lux_first_item(uint32_t g, uint32_t warps) { return g / warps * kLuxGroup * warps + g % warps; }
 PRNG_HD uint64_t lux_groups(uint64_t segs, uint64_t warps) { return (segs + kLuxGroup - 1) / kLuxGroup * warps; }
 
+// Whether the tile engine can store rows x pitch words (a multiple of 4) in tiles
+// of 32 x 32: its tile coordinates are signed 32-bit numbers.
+constexpr uint64_t kLuxTileLimit = (1ull << 31) - 32;
+PRNG_HD bool lux_tiles_reach(uint64_t pitch, uint64_t rows) {
+  return pitch > 0 && (pitch & 3) == 0 && pitch <= kLuxTileLimit && rows > 0 && rows <= kLuxTileLimit;
+}
+
 }  // namespace prng

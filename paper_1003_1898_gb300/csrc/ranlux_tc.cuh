@@ -48,8 +48,8 @@ uint64_t lux_start_bytes(uint64_t items);
 LuxSplit lux_split(uint64_t warp_blocks, uint64_t longest);
 
 // The tensor map of an output as a rows x pitch array of words in tiles of 32 x
-// 32; false when it has none (unaligned, not this device's memory, past the
-// map's limits).
+// 32; false when it has none (unaligned, not this device's memory, more than 2^31 - 32
+// words in a row or rows: lux_tiles_reach).
 bool lux_out_map(void* out, uint64_t pitch, uint64_t rows, CUtensorMap* map);
 
 }  // namespace prng

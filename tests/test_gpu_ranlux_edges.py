@@ -1,4 +1,6 @@
 """RANLUX fills at the edges of their division into segments and tiles."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -31,3 +33,17 @@ def test_fresh_rows_one_block_past_whole_segments(ns, per):
             np.testing.assert_array_equal(out.cpu().numpy().view(np.uint32), ref[:, k * per:(k + 1) * per])
     finally:
         P.prng_destroy(h)
+
+
+@pytest.mark.parametrize("pitch,has_map", [(1024, True), (2**31 - 32, True), (2**31, False), (2**31 + 32, False),
+                                           (2**32 - 4, False)])
+def test_rows_past_the_tile_engine_have_no_map(pitch, has_map):
+    # The engine's column coordinate would turn negative and its tiles be dropped;
+    # such rows are stored by the warps.  Only the map is asked for: nothing is filled.
+    f = P.lib()._ZN4prng11lux_out_mapEPvmmP14CUtensorMap_st
+    f.restype = ctypes.c_bool
+    f.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_void_p]
+    out = torch.empty(1024, dtype=torch.int32, device="cuda")
+    room = ctypes.create_string_buffer(128 + 64)
+    at = (ctypes.addressof(room) + 63) // 64 * 64
+    assert f(out.data_ptr(), pitch, 1, at) == has_map

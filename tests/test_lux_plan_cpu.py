@@ -47,6 +47,7 @@ extern "C" int split(uint64_t warp_blocks, uint64_t longest) {
   return s.cut ? s.lgb : -1;
 }
 extern "C" int powers() { return kLuxPowers; }
+extern "C" int tiles_reach(uint64_t pitch, uint64_t rows) { return lux_tiles_reach(pitch, rows); }
 """
 
 
@@ -60,7 +61,7 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_1003_1898_gb300", "csrc"), str(src), "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.walk.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int]
-    L.split.argtypes = [ctypes.c_uint64, ctypes.c_uint64]
+    L.split.argtypes = L.tiles_reach.argtypes = [ctypes.c_uint64, ctypes.c_uint64]
     return L
 
 
@@ -128,3 +129,15 @@ def test_operands_are_the_powers_of_the_luxury_cycle():
                 want = (pow(256, k, m) * a % m).to_bytes(72, "little")
                 np.testing.assert_array_equal(got[:72, k], np.frombuffer(want, np.uint8), err_msg=f"p {p} power {i}")
             a = a * a % m
+
+
+@pytest.mark.parametrize("pitch", [4, 32, 36, 2**30, 2**31 - 64, 2**31 - 32, 2**31 - 4, 2**31, 2**31 + 32, 2**32 - 4,
+                                   2**32, 2**40])
+def test_tile_coordinates_are_signed_32_bit(lib, pitch):
+    # The last tile of a row starts at column (pitch - 1) / 32 * 32, and a full one ends 32 on.
+    last = (pitch - 1) // 32 * 32
+    for p, r in ((pitch, 1), (4, pitch)):
+        if lib.tiles_reach(p, r):
+            assert last + 32 <= 2**31 - 1
+        else:
+            assert pitch > 2**31 - 32
