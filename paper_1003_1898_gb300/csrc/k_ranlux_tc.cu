@@ -1220,6 +1220,9 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
       so.done = so.pos >> 5;
       so.lo = (uint32_t)(so.pos & 31);
       so.map = so.off != 0 ? nullptr : job.reqs != nullptr ? heads[wi].map : job.tiles ? &job.map : nullptr;
+      // A batch's maps are in memory that the host rewrites between launches; a
+      // single fill's is a kernel parameter.  The lane that stores the tiles waits.
+      if (so.map != nullptr && job.reqs != nullptr && lane == 0) tc::map_acquire(so.map);
       so.whole = d.limit / d.pitch;
       have = true;
     }

@@ -110,6 +110,12 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// Before this thread's first use of a tensor map in global memory that a copy may
+// have rewritten since: descriptors are cached apart from data.
+__device__ __forceinline__ void map_acquire(const void* map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
+
 // One 2-D tile of shared memory to the tensor map's array at element column x,
 // row y (what lies past the array is not written), as a bulk group of its own.
 __device__ __forceinline__ void tile_store(const void* map, uint32_t smem, uint32_t x, uint32_t y) {

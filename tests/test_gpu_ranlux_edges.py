@@ -47,3 +47,35 @@ def test_rows_past_the_tile_engine_have_no_map(pitch, has_map):
     room = ctypes.create_string_buffer(128 + 64)
     at = (ctypes.addressof(room) + 63) // 64 * 64
     assert f(out.data_ptr(), pitch, 1, at) == has_map
+
+
+@pytest.mark.parametrize("lux", [223, 389])
+def test_batcher_outputs_that_move_between_launches(lux):
+    # Every launch rewrites a slot's tensor maps at the same addresses: other
+    # outputs, pitches and limits each time, over more launches than slots, with
+    # nothing between them.
+    ns, n = 96, 11
+    hs = [P.prng_create("ranlux", 700 + i, ns, lux) for i in range(2)]
+    b = P.prng_batcher_create(2, 4096)
+    rng = np.random.default_rng(lux)
+    drawn, launched = [0, 0], []
+    for k in range(n):
+        reqs = []
+        for i, h in enumerate(hs):
+            per = 4 * int(rng.integers(100, 700))
+            valid = int(rng.integers(1, ns * per)) if k % 3 == 1 else 0
+            out = torch.full((ns * per + 64,), -7, dtype=torch.int32, device="cuda")
+            reqs.append({"st": h, "d_out": out, "n_per_stream": per, "n_valid": valid})
+            launched.append((i, drawn[i], per, valid, out))
+            drawn[i] += per
+        P.prng_batcher_launch(b, reqs)
+    torch.cuda.synchronize()
+    refs = [oracle.fill("ranlux", 700 + i, ns, drawn[i], luxury=lux) for i in range(2)]
+    for i, at, per, valid, out in launched:
+        got = out.cpu().numpy()
+        want = refs[i][:, at:at + per].reshape(-1)[:valid or None]
+        np.testing.assert_array_equal(got[:want.size].view(np.uint32), want)
+        assert np.all(got[want.size:] == -7)
+    P.prng_batcher_destroy(b)
+    for h in hs:
+        P.prng_destroy(h)
