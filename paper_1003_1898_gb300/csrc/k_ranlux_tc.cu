@@ -1039,14 +1039,18 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
   }
   // Segment after segment.
   if (__syncthreads_or(cnt > 1)) lux_operand(sh, level, job.lgb);
+  // The head of segment seg + j, by its warp; its item's start, or nullptr past the items.
+  auto head = [&](uint32_t j) -> uint32_t* {
+    if (j >= cnt || it + j * warps >= job.n_items) return nullptr;
+    uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords;
+    if (lane == 0) heads[wi].seg = seg + j;
+    __syncwarp();
+    const uint32_t* h = reinterpret_cast<const uint32_t*>(&heads[wi]);
+    for (uint32_t k = lane; k < kHeadWords; k += 32) st[k] = h[k];
+    return st + kHeadPitch + lane;
+  };
   for (uint32_t j = 0;; j++) {
-    if (j < cnt && it + j * warps < job.n_items) {
-      uint32_t* st = job.starts + (uint64_t)(it + j * warps) * kStartWords;
-      if (lane == 0) heads[wi].seg = seg + j;
-      __syncwarp();
-      const uint32_t* h = reinterpret_cast<const uint32_t*>(&heads[wi]);
-      for (uint32_t k = lane; k < kHeadWords; k += 32) st[k] = h[k];
-      st += kHeadPitch + lane;
+    if (uint32_t* st = head(j)) {
 #pragma unroll
       for (int k = 0; k < 18; k++) st[32 * k] = N[k];
       st[32 * 18] = zero ? 1u : 0u;
@@ -1054,6 +1058,12 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
     if (!__syncthreads_or(j + 1 < cnt) || !lux_issue(sh, tm, N, !ok)) break;
     ok = lux_take(sh, tm, products & 1u, N) && ok;
     products++;
+  }
+  // A CTA that gave up leaves heads without draws, so that the items' kernel skips
+  // its segments instead of reading starts that were never written.
+  if (__syncthreads_or(!ok)) {
+    if (lane == 0) heads[wi].d.n_per = 0;
+    for (uint32_t j = 0; j < cnt; j++) head(j);
   }
   if (!ok) atomicExch(&g_stuck, 1u);
   lux_teardown(tm);
@@ -1203,7 +1213,7 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
       __syncwarp();
       const LuxPlan plan(d);
       const uint64_t b0 = (uint64_t)heads[wi].seg << job.lgb;
-      if (b0 > 0 && plan.nb <= b0) continue;
+      if (b0 > 0 && plan.nb <= b0) continue;   // an empty last segment, or a start that was given up
       uint64_t nb = plan.nb - b0;
       last = true;
       if (job.max_seg > 0 && nb > 1ull << job.lgb) {

@@ -46,6 +46,10 @@ extern "C" int split(uint64_t warp_blocks, uint64_t longest) {
   const LuxSplit s = lux_split(warp_blocks, longest, 152);
   return s.cut ? s.lgb : -1;
 }
+extern "C" uint64_t pieces(uint64_t n, uint32_t pos) {
+  const LuxPieces p(n, pos);
+  return p.nb + p.h + p.m;
+}
 extern "C" int powers() { return kLuxPowers; }
 extern "C" int tiles_reach(uint64_t pitch, uint64_t rows) { return lux_tiles_reach(pitch, rows); }
 """
@@ -61,6 +65,7 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_1003_1898_gb300", "csrc"), str(src), "-o", str(so)], check=True)
     L = ctypes.CDLL(str(so))
     L.walk.argtypes = [ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint64, ctypes.c_int]
+    L.pieces.argtypes = [ctypes.c_uint64, ctypes.c_uint32]
     L.split.argtypes = L.tiles_reach.argtypes = [ctypes.c_uint64, ctypes.c_uint64]
     return L
 
@@ -141,3 +146,10 @@ def test_tile_coordinates_are_signed_32_bit(lib, pitch):
             assert last + 32 <= 2**31 - 1
         else:
             assert pitch > 2**31 - 32
+
+
+@pytest.mark.parametrize("pos", [0, 1, 23, 24])
+def test_a_head_without_draws_asks_for_nothing(lib, pos):
+    # What the segments' kernel is left when a start was given up: no block, no
+    # head and no tail, whatever the segment.
+    assert lib.pieces(0, pos) == 0
