@@ -17,6 +17,10 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *     stream).  Fills are asynchronous on that stream; the caller orders
  *     work on one handle (a handle is not thread-safe).
+ *   - RANLUX kernels wait for their tensor core with a limit of some seconds.
+ *     One that gave up leaves its fill and handle undone; from then on every
+ *     fill, skip, batch and prng_get_state of a RANLUX handle of that device
+ *     returns PRNG_ECUDA.
  *   - Outputs are stream-major: element (i, j) of a fill, the j-th new draw
  *     of stream i, is at d_out[i * n_per_stream + j].
  *   - u32 outputs: GGL x_n in [1, 2^31-2]; XOR128 the new word; RANECU the

@@ -77,6 +77,7 @@ int fill_impl(prng_state* st, void* d_out, uint64_t n_per, int mode, cudaStream_
     n_per *= 2;
   }
   if (st->n_streams > UINT64_MAX / n_per) return PRNG_ESIZE;
+  if (handle_failed(st)) return PRNG_ECUDA;
   FillDesc d{};
   d.state = st->d_state;
   d.n_rows = st->n_streams;
@@ -304,6 +305,7 @@ int prng_ising_fused(prng_state* st, int8_t* d_spins, uint32_t L, uint32_t colou
   if (L < 2 || (L & 1) != 0 || L > 65534 || colour > 1) return PRNG_ESIZE;
   const uint64_t sites = (uint64_t)L * (L / 2);
   if (sites % st->n_streams != 0) return PRNG_ESIZE;
+  if (handle_failed(st)) return PRNG_ECUDA;
   FillDesc d{};
   d.state = st->d_state;
   d.n_rows = st->n_streams;
@@ -360,6 +362,7 @@ constexpr uint64_t kMtPolySkip = 1ull << 20;
 int prng_skip(prng_state* st, uint64_t k, void* stream) {
   if (st == nullptr) return PRNG_ENULL;
   if (k == 0) return PRNG_OK;
+  if (handle_failed(st)) return PRNG_ECUDA;
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   if (st->gen == GGL || st->gen == RANECU) {
@@ -406,8 +409,7 @@ int prng_get_state(prng_state* st, void* h_buf, size_t* bytes) {
     return PRNG_ESIZE;
   }
   std::vector<uint32_t> dev((size_t)n * W);
-  if (st->gen == RANLUX && lux_tc_stuck()) return PRNG_ECUDA;
-  if (cudaDeviceSynchronize() != cudaSuccess ||
+  if (cudaDeviceSynchronize() != cudaSuccess || handle_failed(st) ||
       cudaMemcpy(dev.data(), st->d_state, dev.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
     return PRNG_ECUDA;
   uint32_t* b = static_cast<uint32_t*>(h_buf);

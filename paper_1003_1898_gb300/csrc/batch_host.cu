@@ -252,6 +252,8 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
 
 int prng_batch_launch(prng_batch* b, void* stream) {
   if (b == nullptr) return PRNG_ENULL;
+  for (const prng_fill_req& r : b->reqs)
+    if (handle_failed(r.st)) return PRNG_ECUDA;
   Buffers& u = b->buf[b->next];
   if (u.pending) {  // the pinned buffer may still be in flight from two launches ago
     if (cudaEventSynchronize(u.done) != cudaSuccess) return PRNG_ECUDA;

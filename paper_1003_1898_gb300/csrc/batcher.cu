@@ -123,6 +123,7 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
     if (r.n_per_stream > 0 && r.d_out == nullptr) return PRNG_ENULL;
     if ((reinterpret_cast<uintptr_t>(r.d_out) & 3) != 0) return PRNG_ESIZE;
     if (r.n_per_stream > 0 && r.st->n_streams > UINT64_MAX / r.n_per_stream) return PRNG_ESIZE;
+    if (handle_failed(r.st)) return PRNG_ECUDA;
   }
   // Items per family: RANLUX streams cut into segments where the slot has room
   // for them, whole otherwise.

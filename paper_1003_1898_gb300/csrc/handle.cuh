@@ -17,6 +17,11 @@ struct prng_state {
 
 namespace prng {
 
+// A RANLUX handle of a device on which a RANLUX kernel gave up waiting for its
+// tensor core (k_ranlux_tc.cu).
+bool lux_tc_failed(int dev);
+inline bool handle_failed(const prng_state* st) { return st->gen == RANLUX && lux_tc_failed(st->device); }
+
 // Luxury level or p -> p: levels 0..4 are the standard p = 24, 48, 97, 223,
 // 389 (Appendix A, "RANLUX"); p itself is accepted, and so are the planar
 // scheme's p = 120, 240, 408 (Section 3.6: 96, 216, 384 discarded after each

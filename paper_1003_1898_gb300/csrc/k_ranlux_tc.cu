@@ -54,8 +54,16 @@ constexpr int kTmemCols = 128, kColD = 0, kColA = 80;
 
 // Filled on a device's first RANLUX handle (2.4 MB).
 __device__ uint4 g_tab[kLevels][kLuxPowers][kTabBytes / 16];
-// Set when a kernel gave up waiting for the tensor core (never seen).
-__device__ uint32_t g_stuck;
+// The device's word that a kernel sets when it gave up waiting for the tensor core
+// (never seen): in mapped host memory, so that a later call sees it without a copy.
+__device__ uint32_t* g_failed;
+constexpr int kMaxDevices = 64;
+uint32_t* g_failed_host[kMaxDevices] = {};
+
+__device__ __forceinline__ void lux_give_up() {
+  *static_cast<volatile uint32_t*>(g_failed) = 1u;
+  __threadfence_system();
+}
 
 // ---------------------------------------------------------- host: the operands
 
@@ -222,22 +230,34 @@ const std::vector<uint16_t>& lux_host_tables() {
 // Fill the current device's operands once.
 cudaError_t lux_tables_init() {
   static std::mutex lock;
-  static bool done[64] = {};
+  static bool done[kMaxDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> guard(lock);
   if (done[dev]) return cudaSuccess;
+  uint32_t *word = g_failed_host[dev], *at = nullptr;
+  if (word == nullptr) {
+    e = cudaHostAlloc(reinterpret_cast<void**>(&word), sizeof(*word), cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    *word = 0;
+    g_failed_host[dev] = word;
+  }
+  e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&at), word, 0);
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_failed, &at, sizeof(at));
+  if (e != cudaSuccess) return e;
   const std::vector<uint16_t>& host = lux_host_tables();
   e = cudaMemcpyToSymbol(g_tab, host.data(), host.size() * 2);
   if (e == cudaSuccess) done[dev] = true;
   return e;
 }
 
-bool lux_tc_stuck() {
-  uint32_t v = 0;
-  return cudaMemcpyFromSymbol(&v, g_stuck, sizeof(v)) != cudaSuccess || v != 0;
+uint32_t* lux_failed_word(int dev) { return dev >= 0 && dev < kMaxDevices ? g_failed_host[dev] : nullptr; }
+
+bool lux_tc_failed(int dev) {
+  const volatile uint32_t* w = lux_failed_word(dev);
+  return w != nullptr && *w != 0;
 }
 
 // --------------------------------------------------------------------- device
@@ -745,7 +765,7 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tiles(const FillDesc d, 
   }
   ok = !__syncthreads_or(!ok);                    // also: no product reads the table any more
   if (!ok) {
-    if (tid == 0) atomicExch(&g_stuck, 1u);
+    if (tid == 0) lux_give_up();
   } else {
     if (products > 0) {
       if (plan.m == 0) {
@@ -895,7 +915,7 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int
   }
   ok = !__syncthreads_or(!ok);                    // also: no product reads the table any more
   if (!ok) {
-    if (tid == 0) atomicExch(&g_stuck, 1u);
+    if (tid == 0) lux_give_up();
   } else if (products > 0) {
     if (plan.m == 0) {
       deliver();
@@ -1065,7 +1085,7 @@ __global__ void __launch_bounds__(128, 4) k_lux_starts(const __grid_constant__ L
     if (lane == 0) heads[wi].d.n_per = 0;
     for (uint32_t j = 0; j < cnt; j++) head(j);
   }
-  if (!ok) atomicExch(&g_stuck, 1u);
+  if (!ok) lux_give_up();
   lux_teardown(tm);
 }
 
@@ -1275,7 +1295,7 @@ __global__ void __launch_bounds__(128, 4) k_lux_items(const __grid_constant__ Lu
     }
     have = false;
   }
-  if (!ok && lane == 0) atomicExch(&g_stuck, 1u);
+  if (!ok && lane == 0) lux_give_up();
   if (lane == 0) tc::tile_store_wait_read();
   lux_teardown(tm);
 }

@@ -67,6 +67,7 @@ extern "C" int prng_batch_fill_noalloc(const prng_fill_req* reqs, uint32_t n_req
     if (r.n_per_stream > 0 && r.d_out == nullptr) return PRNG_ENULL;
     if ((reinterpret_cast<uintptr_t>(r.d_out) & 3) != 0) return PRNG_ESIZE;
     if (r.n_per_stream > 0 && r.st->n_streams > UINT64_MAX / r.n_per_stream) return PRNG_ESIZE;
+    if (handle_failed(r.st)) return PRNG_ECUDA;
     g_sorted[i] = r.st;
     if (r.reseed) fam_n[FAM_SEED] += (r.st->n_streams + 255) / 256;
     if (r.n_per_stream > 0) {

@@ -17,9 +17,12 @@ constexpr int kLuxTcMinP = 97;
 // RANLUX handle is created, before any of its fills).
 cudaError_t lux_tables_init();
 
-// Whether a kernel on the current device ever gave up waiting for its tensor
-// core (its handle's state is then not the one after the fill).  Synchronises.
-bool lux_tc_stuck();
+// Whether a kernel on device `dev` has given up waiting for its tensor core: its
+// fill's output and handle are then not the ones asked for, and every later call
+// on a RANLUX handle of the device says so.  Reads a word of host memory
+// (lux_failed_word, nullptr before the device's first RANLUX handle).
+bool lux_tc_failed(int dev);
+uint32_t* lux_failed_word(int dev);
 
 // The launch tile of a plain fill that leaves it to the library.
 Tile ranlux_auto_tile(const FillDesc& d);

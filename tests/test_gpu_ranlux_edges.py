@@ -79,3 +79,40 @@ def test_batcher_outputs_that_move_between_launches(lux):
     P.prng_batcher_destroy(b)
     for h in hs:
         P.prng_destroy(h)
+
+
+def test_a_given_up_wait_reaches_every_later_call():
+    # The word that a kernel sets when it gives up (here the test sets it): every
+    # call that would draw from a RANLUX handle of the device, or read its state,
+    # reports it before it launches anything.
+    h = P.prng_create("ranlux", 3, 64, 223)
+    g = P.prng_create("ggl", 3, 64)
+    out = torch.empty((64, 64), dtype=torch.int32, device="cuda")
+    spins = torch.ones((16, 16), dtype=torch.int8, device="cuda")
+    req = [{"st": h, "d_out": out, "n_per_stream": 24}]
+    batch, batcher = P.prng_batch_create(req), P.prng_batcher_create(1, 64)
+    f = P.lib()._ZN4prng15lux_failed_wordEi
+    f.restype = ctypes.POINTER(ctypes.c_uint32)
+    word = f(torch.cuda.current_device())
+    blob = P.prng_get_state(h)
+    calls = [lambda: P.prng_fill_u32(h, out, 24), lambda: P.prng_fill_f64(h, out, 24), lambda: P.prng_skip(h, 24),
+             lambda: P.prng_ising_fused(h, spins, 16, 0, 1, 1), lambda: P.prng_batch_launch(batch),
+             lambda: P.prng_batcher_launch(batcher, req), lambda: P.prng_batch_fill_noalloc(req),
+             lambda: P.prng_get_state(h)]
+    word[0] = 1
+    try:
+        for i, call in enumerate(calls):
+            with pytest.raises(P.PrngError) as e:
+                call()
+            assert e.value.code == -6, i
+        P.prng_fill_u32(g, out, 24)             # other generators do not use it
+    finally:
+        word[0] = 0
+    assert P.prng_get_state(h) == blob
+    for call in calls:
+        call()
+    torch.cuda.synchronize()
+    P.prng_batch_destroy(batch)
+    P.prng_batcher_destroy(batcher)
+    P.prng_destroy(h)
+    P.prng_destroy(g)
