@@ -350,12 +350,14 @@ int prng_calib_swb(uint32_t chains, uint32_t warps_per_sm, uint32_t iters, uint3
 /* Launch tile used by fills of generator `gen` (for RANLUX: of luxury p)
  * on this process: threads per CTA, staged draws per thread per tile
  * (RANMAR: 97, MT19937: 624) and staging buffers (1 or 2; for MT19937 the
- * streams per warp: 1, or 2 on half a warp each).  Set by the
- * autotuner; only the combinations compiled into the library are accepted
- * (PRNG_EUNSUPPORTED otherwise).  RANLUX at p >= 97 also takes 128, 24, 1 (the
- * tensor-core form) and 128, 24, 2 (the same, long streams cut into parts, whose
- * start states come from the library's stream-ordered pool); until a tile is
- * set, RANLUX fills choose theirs by shape.  Not thread-safe against concurrent fills. */
+ * streams per warp: 1, or 2 on half a warp each).  Until one is fixed here,
+ * and again once 0, 0, 0 is given, every fill's tile is chosen by its shape;
+ * prng_get_tile then returns 0, 0, 0, so that setting what it returned puts a
+ * generator back as it was.  Only the combinations compiled into the library
+ * are accepted (PRNG_EUNSUPPORTED otherwise).  RANLUX at p >= 97 also takes
+ * 128, 24, 1 (the tensor-core form) and 128, 24, 2 (the same, long streams cut
+ * into parts, whose start states come from the library's stream-ordered pool).
+ * Not thread-safe against concurrent fills. */
 int prng_set_tile(prng_gen_t gen, uint32_t luxury, uint32_t threads, uint32_t cols,
                   uint32_t stages);
 int prng_get_tile(prng_gen_t gen, uint32_t luxury, uint32_t *threads, uint32_t *cols,

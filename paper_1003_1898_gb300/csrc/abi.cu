@@ -202,11 +202,13 @@ int lux_index(int p) {
 }
 
 // Per generator (RANLUX: per p) launch tiles; slot 5 + i is RANLUX p index i >= 1.
-Tile g_tiles[13] = {{128, 128, 1}, {128, 32, 1}, {128, 128, 1}, {256, 128, 1}, {128, 48, 1},
-                    {128, 624, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1},
-                    {128, 48, 1}, {128, 48, 1}, {128, 48, 1}};
-// Slots whose tile the caller chose; the others' plain fills choose by shape.
-bool g_tile_chosen[13] = {};
+constexpr int kSlots = 13;
+constexpr Tile kDefaultTile[kSlots] = {{128, 128, 1}, {128, 32, 1}, {128, 128, 1}, {256, 128, 1}, {128, 48, 1},
+                                       {128, 624, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1}, {128, 48, 1},
+                                       {128, 48, 1}, {128, 48, 1}, {128, 48, 1}};
+// Tiles that the caller fixed (threads = 0: none; the slot's plain fills choose by
+// shape, and what else asks for its tile gets the default).
+Tile g_tiles[kSlots] = {};
 
 int tile_slot(int gen, int p) {
   if (gen != RANLUX) return gen;
@@ -218,9 +220,12 @@ int tile_slot(int gen, int p) {
 
 namespace prng {
 
-Tile default_tile(int gen, int p) { return g_tiles[tile_slot(gen, p)]; }
+Tile default_tile(int gen, int p) {
+  const int i = tile_slot(gen, p);
+  return g_tiles[i].threads != 0 ? g_tiles[i] : kDefaultTile[i];
+}
 
-bool tile_chosen(int gen, int p) { return g_tile_chosen[tile_slot(gen, p)]; }
+bool tile_chosen(int gen, int p) { return g_tiles[tile_slot(gen, p)].threads != 0; }
 
 }  // namespace prng
 
@@ -483,9 +488,9 @@ int prng_set_tile(prng_gen_t gen, uint32_t luxury, uint32_t threads, uint32_t co
     if (p < 0) return PRNG_ELUXURY;
   }
   const Tile t{(int)threads, (int)cols, (int)stages};
-  if (!tile_supported(g, t, p)) return PRNG_EUNSUPPORTED;
+  const bool by_shape = threads == 0 && cols == 0 && stages == 0;
+  if (!by_shape && !tile_supported(g, t, p)) return PRNG_EUNSUPPORTED;
   g_tiles[tile_slot(g, p)] = t;
-  g_tile_chosen[tile_slot(g, p)] = true;
   return PRNG_OK;
 }
 

@@ -69,11 +69,14 @@ inline int lux_p_of(int fam) { return kLuxFamilyP[kind_of(fam) - FAM_LUX24]; }
 // bulk-fill tile: a work item is one CTA's rows of one request, and most
 // requests of a batch have few streams, so 32-row items waste fewer threads
 // (measured: 0.75 against 0.50 numbers/ns with 64-row items on the mixed
-// 20,000-request batch).  The others use the generator's default tile.
+// 20,000-request batch).  XOR128 stages 64 columns unless a tile was fixed (40
+// fills of 4,096 x 4,096 in one prng_batch_fill_noalloc 495 / 476 us, 20 of 1,024
+// x 20,000 583 / 425).  The others use the generator's default tile.
 inline Tile tile_of(int fam) {
   const int k = kind_of(fam);
   if (k == FAM_SEED) return Tile{256, 0, 1};
   if (k >= FAM_LUX24) return Tile{32, 48, 1};
+  if (k == FAM_XOR128 && !tile_chosen(XOR128, 0)) return Tile{128, 64, 1};
   const int gen = k == FAM_MLCG ? GGL : k == FAM_XOR128 ? XOR128 : k == FAM_RANMAR ? RANMAR : MT19937;
   return default_tile(gen, 0);
 }

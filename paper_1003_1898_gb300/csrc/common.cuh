@@ -124,8 +124,8 @@ inline uint64_t fill_multiplier(int gen, uint64_t n) {
   return 0;
 }
 
-Tile default_tile(int gen, int p);
-bool tile_chosen(int gen, int p);   // by prng_set_tile
+Tile default_tile(int gen, int p);  // the fixed tile, or the generator's own
+bool tile_chosen(int gen, int p);   // a tile was fixed by prng_set_tile
 
 // SplitMix64 (Steele, Lea, Flood 2014): gamma increment, then mix64.
 __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {

@@ -36,11 +36,16 @@ PRNG_RANLUX_DECLARE(408)
 Tile ranlux_auto_tile(const FillDesc& d) {
   // The borrow chain's own tile: the ring, but for short rows of many streams
   // (131,072 x 64 at p = 24 27 / 23 us without it, x 248 41 / 37); in wide CTAs
-  // for long rows at p = 48 (131,072 x 8,192 781 / 714, 4,096 x 4,096 70 / 95).
+  // for long rows at p = 48 (131,072 x 8,192 781 / 714, 4,096 x 4,096 70 / 95), in
+  // CTAs of 128 for long rows of about 100,000 streams at p = 24 (98,304 x 8,192 596 /
+  // 538, 131,072 x 8,192 781 / 766, x 4,096 388 / 382; 200,000 x 4,096 549 / 549;
+  // 65,536 x 4,096 205 / 213; doubles no faster).
   Tile t = ranlux_ring_ok(d) || d.p < 97 ? Tile{64, 56, 1} : Tile{64, 96, 1};
   if (d.p < 97 && d.n_rows >= 32768) {
     if (d.n_per < 320) t = Tile{64, 48, 1};
     else if (d.p == 48 && d.n_rows >= 65536 && d.n_per >= 1024) t = Tile{256, 56, 1};
+    else if (d.p == 24 && d.mode != OUT_F64 && d.n_rows >= 98304 && d.n_rows <= 131072 && d.n_per >= 4096)
+      t = Tile{128, 56, 1};
   }
   if (d.p < kLuxTcMinP || d.n_per < 24) return t;
   const uint64_t nb = d.n_per / 24, p = (uint64_t)d.p, sms = (uint64_t)sm_count();

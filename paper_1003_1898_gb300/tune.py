@@ -4,10 +4,13 @@ For each generator (RANLUX: each luxury p) it times one fill of a given
 workload shape with every tile compiled into the library (threads per CTA,
 staged draws per thread, staging buffers), keeps the fastest, and can save
 the choice as JSON so later processes apply it with ``apply()`` before
-filling.  Timing uses CUDA events on the current stream after a warm-up
+filling.  A fixed tile holds for every shape: XOR128, RANMAR, RANLUX and
+MT19937, whose fills choose their tile by shape (and XOR128 and RANLUX cut few
+long streams into segments) as long as none is fixed, are timed that way too and
+keep it unless ``fixed`` asks for the one best tile.  Timing uses CUDA events on the current stream after a warm-up
 fill; outputs larger than L2 are used so no flush is needed.
 
-  python -m paper_1003_1898_gb300.tune [--out tuned_tiles.json]
+  python -m paper_1003_1898_gb300.tune [--out tuned_tiles.json] [--fixed]
 """
 from __future__ import annotations
 
@@ -35,6 +38,9 @@ TILES = {
                 (128, 624, 2), (256, 624, 2), (256, 227, 1)],   # 227: a CTA per stream
 }
 
+BY_SHAPE = (0, 0, 0)     # no fixed tile
+SHAPE_RULES = ("xor128", "ranmar", "ranlux", "mt19937")
+
 # Workload shapes the tiles are tuned for: the roofline bulk fill, and for
 # RANLUX at p >= 97 (not part of that fill) the luxury sweep.
 SHAPES = {"mt19937": (8192, 131072)}
@@ -55,7 +61,7 @@ def key(gen: str, luxury: int = 0) -> str:
 
 def time_fill(gen: str, tile, n_streams: int, n_per: int, luxury: int = 0, dtype: str = "u32",
               reps: int = 5) -> float:
-    """Median milliseconds of one fill with the given tile."""
+    """Median milliseconds of one fill with the given tile (which stays set)."""
     import torch
     prng_set_tile(gen, luxury, *tile)
     h = prng_create(gen, 0x5EED, n_streams, luxury)
@@ -81,9 +87,11 @@ def time_fill(gen: str, tile, n_streams: int, n_per: int, luxury: int = 0, dtype
     return ts[len(ts) // 2]
 
 
-def tune(gens=GEN_NAMES, luxuries=LUXURY_P + PLANAR_P[1:], reps: int = 5, verbose: bool = True) -> dict:
+def tune(gens=GEN_NAMES, luxuries=LUXURY_P + PLANAR_P[1:], reps: int = 5, verbose: bool = True,
+         fixed: bool = False) -> dict:
     """Time every compiled tile and return {key: {"tile": [...], "ms": {...}}};
-    a tile's ms is the sum of one u32 and one f32 fill of the shape."""
+    a tile's ms is the sum of one u32 and one f32 fill of the shape.  The tile
+    of a generator with shape rules is BY_SHAPE unless `fixed`."""
     result = {}
     jobs = []
     for g in gens:
@@ -95,10 +103,11 @@ def tune(gens=GEN_NAMES, luxuries=LUXURY_P + PLANAR_P[1:], reps: int = 5, verbos
         ns, nper = LUXURY_SHAPE if (g == "ranlux" and lux >= 97) else SHAPES.get(g, DEFAULT_SHAPE)
         before = prng_get_tile(g, lux)
         ms = {}
-        for t in tiles_for(g, lux):   # a u32 fill plus an f32 fill, as the benchmark step does
+        rules = g in SHAPE_RULES
+        for t in tiles_for(g, lux) + [BY_SHAPE] * rules:   # a u32 plus an f32 fill, as the benchmark step does
             ms[",".join(map(str, t))] = (time_fill(g, t, ns, nper, lux, "u32", reps=reps) +
                                          time_fill(g, t, ns, nper, lux, "f32", reps=reps))
-        best = min(ms, key=ms.get)
+        best = ",".join(map(str, BY_SHAPE)) if rules and not fixed else min(ms, key=ms.get)
         tile = [int(x) for x in best.split(",")]
         prng_set_tile(g, lux, *tile)
         result[key(g, lux)] = {"tile": tile, "ms": ms, "shape": [ns, nper],
@@ -136,10 +145,11 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--out", default=DEFAULT_CACHE)
     ap.add_argument("--reps", type=int, default=5)
+    ap.add_argument("--fixed", action="store_true", help="the one best tile for generators with shape rules too")
     args = ap.parse_args()
     from . import build
     build.build()
-    res = tune(reps=args.reps)
+    res = tune(reps=args.reps, fixed=args.fixed)
     with open(args.out, "w") as f:
         json.dump(res, f, indent=1, sort_keys=True)
     print(args.out)
