@@ -55,7 +55,8 @@ namespace {
 void destroy_batcher(prng_batcher* b) {
   if (b == nullptr) return;
   for (auto& u : b->slot) {
-    if (u.pending && u.done) cudaEventSynchronize(u.done);
+    // The event of a captured launch cannot be waited for; the error stays here.
+    if (u.pending && u.done && cudaEventSynchronize(u.done) != cudaSuccess) cudaGetLastError();
     if (u.done) cudaEventDestroy(u.done);
     if (u.h_reqs) cudaFreeHost(u.h_reqs);
     if (u.h_items) cudaFreeHost(u.h_items);
@@ -166,11 +167,14 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
   uint64_t lux_items = 0;
   for (int f = 0; f < FAM_COUNT; f++)
     if (plan.is_lux_tc(f)) lux_items += fam_n[f];
+  // A captured launch takes no scratch, as captured fills: an allocation would
+  // become a node of the graph, which could then be instantiated once only.
   if (lux_items > 0 &&
-      scratch_alloc(reinterpret_cast<void**>(&starts), lux_start_bytes(lux_items), s) != cudaSuccess) {
+      (capturing(s) ||
+       scratch_alloc(reinterpret_cast<void**>(&starts), lux_start_bytes(lux_items), s) != cudaSuccess)) {
     cudaGetLastError();
     starts = nullptr;
-    plan.tensor = false;        // no room: the borrow chain, with no more items than uncut streams
+    plan.tensor = false;        // the borrow chain, with no more items than uncut streams
     count(false);
   }
   bool maps = false;
