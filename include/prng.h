@@ -156,8 +156,9 @@ int prng_set_state(prng_state *st, const void *h_buf, size_t bytes);
  * doubling passes of the jump polynomial (about 6 million word XORs per chunk),
  * with a scratch array of 44 KB per chunk.  The scratch arrays come from a stream-ordered
  * memory pool that the library creates on first use on each device and
- * that keeps its memory until the process exits, so repeated jump fills do
- * not allocate afresh.  Other generators return PRNG_EUNSUPPORTED. */
+ * that keeps up to 1 GiB of it until the process exits, so repeated jump fills do
+ * not allocate afresh; what it held beyond that goes back to the device at the
+ * next synchronisation.  Other generators return PRNG_EUNSUPPORTED. */
 int prng_fill_jump_u32(prng_gen_t gen, uint64_t x0, uint64_t n, uint32_t n_chunks,
                        uint32_t *d_out, void *stream);
 int prng_fill_jump_f32(prng_gen_t gen, uint64_t x0, uint64_t n, uint32_t n_chunks,

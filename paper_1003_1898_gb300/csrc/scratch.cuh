@@ -1,7 +1,8 @@
-// scratch.cuh -- stream-ordered scratch for the jump fills' chunk-start
-// tables, from a memory pool the library creates once per device and that
-// keeps its memory for reuse (the device's default pool would hand freed
-// memory back at every synchronisation, so that each call allocated afresh).
+// scratch.cuh -- stream-ordered scratch (the jump fills' chunk starts, the
+// segments' starts of XOR128 and RANLUX fills), from a memory pool the library
+// creates once per device and that keeps up to 1 GiB for reuse (the device's
+// default pool would hand freed memory back at every synchronisation, so that
+// each call allocated afresh).
 #pragma once
 
 #include <cstddef>
