@@ -243,9 +243,10 @@ int prng_create(prng_state** out, prng_gen_t gen, uint64_t seed, uint32_t n_stre
     if (p < 0) return PRNG_ELUXURY;
   }
   if (n_streams == 0) return PRNG_ESIZE;
-  if ((g == RANLUX && lux_tables_init() != cudaSuccess) || (g == XOR128 && xor128_tables_init() != cudaSuccess)) {
+  const cudaError_t e = g == RANLUX ? lux_tables_init() : g == XOR128 ? xor128_tables_init() : cudaSuccess;
+  if (e != cudaSuccess) {
     cudaGetLastError();
-    return PRNG_ECUDA;
+    return e == cudaErrorMemoryAllocation ? PRNG_EALLOC : PRNG_ECUDA;
   }
   prng_state* st = new (std::nothrow) prng_state;
   if (st == nullptr) return PRNG_EALLOC;

@@ -111,13 +111,8 @@ cudaError_t capture(prng_batch* b, Buffers& u) {
   return e;
 }
 
-}  // namespace
-
-extern "C" {
-
-int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_reqs) {
-  if (out == nullptr) return PRNG_ENULL;
-  *out = nullptr;
+// prng_batch_create; b is the caller's to release if an allocation throws.
+int create_batch(prng_batch** out, prng_batch*& b, const prng_fill_req* reqs, uint32_t n_reqs) {
   if (n_reqs == 0) return PRNG_ESIZE;
   if (reqs == nullptr) return PRNG_ENULL;
   std::vector<const prng_state*> seen;
@@ -133,7 +128,7 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
   std::sort(seen.begin(), seen.end());
   if (std::adjacent_find(seen.begin(), seen.end()) != seen.end()) return PRNG_EBLOB;
 
-  prng_batch* b = new (std::nothrow) prng_batch;
+  b = new (std::nothrow) prng_batch;
   if (b == nullptr) return PRNG_EALLOC;
   b->reqs.assign(reqs, reqs + n_reqs);
   cudaGetDevice(&b->device);
@@ -248,6 +243,22 @@ int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_re
   }
   *out = b;
   return PRNG_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int prng_batch_create(prng_batch** out, const prng_fill_req* reqs, uint32_t n_reqs) {
+  if (out == nullptr) return PRNG_ENULL;
+  *out = nullptr;
+  prng_batch* b = nullptr;
+  try {
+    return create_batch(out, b, reqs, n_reqs);
+  } catch (const std::bad_alloc&) {   // no exception leaves a C entry point
+    destroy_batch(b);
+    return PRNG_EALLOC;
+  }
 }
 
 int prng_batch_launch(prng_batch* b, void* stream) {

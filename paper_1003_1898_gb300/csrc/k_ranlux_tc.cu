@@ -29,6 +29,7 @@
 // same per-row ring and warp-level 128-byte copy-outs as k_fill_ranlux_ring.
 #include <algorithm>
 #include <mutex>
+#include <new>
 #include <utility>
 #include <vector>
 
@@ -231,11 +232,17 @@ const std::vector<uint16_t>& lux_host_tables() {
 cudaError_t lux_tables_init() {
   static std::mutex lock;
   static bool done[kMaxDevices] = {};
+  std::lock_guard<std::mutex> guard(lock);
+  const std::vector<uint16_t>* host;
+  try {
+    host = &lux_host_tables();
+  } catch (const std::bad_alloc&) {   // no exception leaves a C entry point
+    return cudaErrorMemoryAllocation;
+  }
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> guard(lock);
   if (done[dev]) return cudaSuccess;
   uint32_t *word = g_failed_host[dev], *at = nullptr;
   if (word == nullptr) {
@@ -247,8 +254,7 @@ cudaError_t lux_tables_init() {
   e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&at), word, 0);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_failed, &at, sizeof(at));
   if (e != cudaSuccess) return e;
-  const std::vector<uint16_t>& host = lux_host_tables();
-  e = cudaMemcpyToSymbol(g_tab, host.data(), host.size() * 2);
+  e = cudaMemcpyToSymbol(g_tab, host->data(), host->size() * 2);
   if (e == cudaSuccess) done[dev] = true;
   return e;
 }
