@@ -389,7 +389,7 @@ int prng_skip(prng_state* st, uint64_t k, void* stream) {
     d.limit = 0;
     d.pos = st->pos;
     d.p = st->p;
-    const Tile t = default_tile(st->gen, st->p);
+    const Tile t = st->gen == RANLUX ? fill_tile(st, d) : default_tile(st->gen, st->p);
     switch (st->gen) {
       case RANMAR: e = launch_fill_ranmar(d, t, s); break;
       case RANLUX: e = launch_fill_ranlux(d, t, s); break;

@@ -40,8 +40,12 @@ Tile ranlux_auto_tile(const FillDesc& d) {
   // CTAs of 128 for long rows of about 100,000 streams at p = 24 (98,304 x 8,192 596 /
   // 538, 131,072 x 8,192 781 / 766, x 4,096 388 / 382; 200,000 x 4,096 549 / 549;
   // 65,536 x 4,096 205 / 213; doubles no faster).
-  Tile t = ranlux_ring_ok(d) || d.p < 97 ? Tile{64, 56, 1} : Tile{64, 96, 1};
-  if (d.p < 97 && d.n_rows >= 32768) {
+  // A skip, which writes nothing, is faster without the ring (65,536 x 2,400 at p = 24
+  // 48 / 37; at p = 223 203, the product 114).
+  Tile t = d.out == nullptr                   ? Tile{128, 48, 1}
+           : ranlux_ring_ok(d) || d.p < 97    ? Tile{64, 56, 1}
+                                              : Tile{64, 96, 1};
+  if (d.out != nullptr && d.p < 97 && d.n_rows >= 32768) {
     if (d.n_per < 320) t = Tile{64, 48, 1};
     else if (d.p == 48 && d.n_rows >= 65536 && d.n_per >= 1024) t = Tile{256, 56, 1};
     else if (d.p == 24 && d.mode != OUT_F64 && d.n_rows >= 98304 && d.n_rows <= 131072 && d.n_per >= 4096)
@@ -64,7 +68,7 @@ Tile ranlux_auto_tile(const FillDesc& d) {
   };
   offer((d.mode == OUT_ISING ? 40000 : 6500) + nb * product(tiles), Tile{128, 24, 1});
   const LuxSplit sp = lux_split(warps * nb, nb);
-  if (sp.cut && d.mode != OUT_ISING && nb < 1ull << 40) {
+  if (sp.cut && d.mode != OUT_ISING && d.out != nullptr && nb < 1ull << 40) {   // a skip has no segments
     const uint64_t B = 1ull << sp.lgb, segs = (nb + B - 1) / B, slots = 16 * sms;
     const uint64_t rounds = (warps * segs + slots - 1) / slots;
     offer(30000 + std::min<uint64_t>(segs, 16) * product(std::min<uint64_t>(tiles, 4 * sms)) +
