@@ -116,6 +116,7 @@ __device__ __forceinline__ int swz(int row, int ch) { return ch ^ (row & 7); }
 template <class G, int T, int K, int OM>
 __device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint64_t row0, uint64_t c0, int w) {
   constexpr int CH = K / 4, RS = T / CH, NW = T / 32;
+  __builtin_assume(__isShared(t));
   const int tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
   const uint64_t pitch = d.pitch, limit = d.limit;
   const int rows = d.n_rows - row0 < (uint64_t)T ? (int)(d.n_rows - row0) : T;
@@ -155,11 +156,29 @@ __device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint
     }
     return;
   }
-  // Word by word: a warp per row, lanes on consecutive columns.
-  if (OM != OUT_F64 && w == K && rows == T && !cut) {   // eight rows in flight
-    uint32_t* p = out + (row0 + wi) * pitch + c0 + lane;
-    const uint64_t step = NW * pitch;
-    for (int r0 = wi; r0 < T; r0 += 8 * NW) {
+  // Word by word (or double by double), lanes on consecutive columns, eight rows of
+  // a lane in flight.  (A row at a time, from a pointer not known to be in shared
+  // memory, each cost about 1 us a tile: 256 x 61 doubles 23 us inside the column
+  // loop as it once stood, 27 that way, here 10.)
+  if constexpr (OM == OUT_F64) {   // w, the row starts and the limit are even
+    constexpr int PR = K / 2, RW = 32 / PR;   // pairs per row, rows per warp and step
+    const int c = 2 * (lane % PR), sub = lane / PR;
+    for (int q0 = wi; q0 * RW < rows; q0 += 8 * NW) {
+      uint2 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int r = (q0 + i * NW) * RW + sub;
+        v[i] = *reinterpret_cast<const uint2*>(t + r * K + 4 * swz<K>(r, c >> 2) + (c & 3));
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int r = (q0 + i * NW) * RW + sub;
+        const uint64_t e = (row0 + r) * pitch + c0 + c;
+        if (r < rows && c < w && (!cut || e < limit)) st_pair<G::WB>(out + e, v[i].x, v[i].y);
+      }
+    }
+  } else {
+    for (int r0 = wi; r0 < rows; r0 += 8 * NW) {
       uint32_t v[8][K / 32];
 #pragma unroll
       for (int i = 0; i < 8; i++)
@@ -168,36 +187,25 @@ __device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint
           const int r = r0 + i * NW, c = lane + 32 * j;
           v[i][j] = t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)];
         }
+      uint64_t e = (row0 + r0) * pitch + c0 + lane;
 #pragma unroll
       for (int i = 0; i < 8; i++) {
 #pragma unroll
-        for (int j = 0; j < K / 32; j++) st_out(p + 32 * j, v[i][j]);
-        p += step;
+        for (int j = 0; j < K / 32; j++)
+          if (r0 + i * NW < rows && lane + 32 * j < w && (!cut || e + 32 * j < limit))
+            st_out(out + e + 32 * j, v[i][j]);
+        e += NW * pitch;
       }
-    }
-    return;
-  }
-  for (int r = wi; r < rows; r += NW) {
-    const uint64_t base = (row0 + r) * pitch + c0;
-    if constexpr (OM == OUT_F64) {   // w, base and the limit are even
-      for (int c = 2 * lane; c < w; c += 64)
-        if (base + c < limit)
-          st_pair<G::WB>(out + base + c, t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)],
-                         t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3) + 1]);
-    } else {
-      for (int c = lane; c < w; c += 32)
-        if (base + c < limit)
-          st_out(out + base + c, t[r * K + 4 * swz<K>(r, c >> 2) + (c & 3)]);
     }
   }
 }
 
 // Streams [row0, row0 + T) of a fill, one per thread; smem holds S tiles of
 // T * K words.  The n draws go to columns col0 .. col0 + n - 1; the states are
-// read from d.state and left in `store_to` (nullptr: nowhere).
+// read from `from` and left in `store_to` (nullptr: nowhere).
 template <class G, int T, int K, int S, int OM>
 __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, uint32_t* smem, uint64_t col0,
-                                            uint64_t n, uint32_t* store_to) {
+                                            uint64_t n, const uint32_t* from, uint32_t* store_to) {
   static_assert(K % 32 == 0, "tile rows hold whole 8-chunk swizzle groups");
   constexpr int CH = K / 4;          // 16-byte chunks per row
   constexpr int RS = T / CH;         // rows one copy-out pass of the CTA covers
@@ -211,9 +219,9 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
     g.zero();
   } else if constexpr (G::JUMPS) {
     if (d.jump) g.jump_start(d.x0, row * d.pitch);   // chunk `row` of one sequence
-    else g.load(d.state, d.n_rows, row);
+    else g.load(from, d.n_rows, row);
   } else {
-    g.load(d.state, d.n_rows, row);
+    g.load(from, d.n_rows, row);
   }
 
   uint32_t* out = static_cast<uint32_t*>(d.out);
@@ -268,23 +276,25 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
   if (active && store_to != nullptr) g.store(store_to, d.n_rows, row);
 }
 
+// (The descriptor stays in the parameter space: a plain parameter whose address
+// odd_tile takes would be copied to every thread's stack first.)
 template <class G, int T, int K, int S, int OM>
-__global__ void __launch_bounds__(T) k_fill_simple(const FillDesc d) {
+__global__ void __launch_bounds__(T) k_fill_simple(const __grid_constant__ FillDesc d) {
   extern __shared__ __align__(16) uint32_t smem[];
-  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, 0, d.n_per, d.jump ? nullptr : d.state);
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, 0, d.n_per, d.state, d.jump ? nullptr : d.state);
 }
 
 // Segment blockIdx.y of every stream: draws [seg L, seg L + L) of the call, from
 // the states that `starts` holds for it ([segment][word][stream]); the last
 // segment leaves the handle's states.
 template <class G, int T, int K, int S, int OM>
-__global__ void __launch_bounds__(T) k_fill_segments(FillDesc d, uint32_t* starts, uint64_t L) {
+__global__ void __launch_bounds__(T) k_fill_segments(const __grid_constant__ FillDesc d, const uint32_t* starts,
+                                                      uint64_t L) {
   extern __shared__ __align__(16) uint32_t smem[];
-  uint32_t* const state = d.state;
   const uint64_t seg = blockIdx.y, col0 = seg * L;
   const uint64_t n = d.n_per - col0 < L ? d.n_per - col0 : L;
-  d.state = starts + seg * 4 * d.n_rows;
-  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, col0, n, seg + 1 == gridDim.y ? state : nullptr);
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, col0, n, starts + seg * 4 * d.n_rows,
+                              seg + 1 == gridDim.y ? d.state : nullptr);
 }
 
 // Batched XOR128 fills: a block pops an item (T streams of one request).
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(T) k_batch_xor128(const BatchQueue q) {
     __shared__ FillDesc sd;
     load_desc(&sd, q.reqs[si.req].d, threadIdx.x, T);
     __syncthreads();
-    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem, 0, sd.n_per, sd.state);
+    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem, 0, sd.n_per, sd.state, sd.state);
   }
 }
 
