@@ -35,7 +35,9 @@ PRNG_RANLUX_DECLARE(408)
 // 223: 50 / 55; over 4,096, 2,048 draws each, p = 389: 550 / 470).
 Tile ranlux_auto_tile(const FillDesc& d) {
   // The borrow chain's own tile: the ring, but for short rows of many streams
-  // (131,072 x 64 at p = 24 27 / 23 us without it, x 248 41 / 37); in wide CTAs
+  // (131,072 x 64 at p = 24 27 / 23 us without it, x 248 41 / 37), at p >= 97 of
+  // unaligned rows too (96 columns / 48: 131,072 x 13 at p = 223 16 / 14, x 61 27.6 /
+  // 25.8; 30,320 x 127 15.3 / 14.4, 4,096 x 127 10.3 / 11.9); in wide CTAs
   // for long rows at p = 48 (131,072 x 8,192 781 / 714, 4,096 x 4,096 70 / 95), in
   // CTAs of 128 for long rows of about 100,000 streams at p = 24 (98,304 x 8,192 596 /
   // 538, 131,072 x 8,192 781 / 766, x 4,096 388 / 382; 200,000 x 4,096 549 / 549;
@@ -44,7 +46,8 @@ Tile ranlux_auto_tile(const FillDesc& d) {
   // 48 / 37; at p = 223 203, the product 114).
   Tile t = d.out == nullptr                   ? Tile{128, 48, 1}
            : ranlux_ring_ok(d) || d.p < 97    ? Tile{64, 56, 1}
-                                              : Tile{64, 96, 1};
+           : d.n_rows >= 30000 && d.n_per < 192 ? Tile{64, 48, 1}
+                                                : Tile{64, 96, 1};
   if (d.out != nullptr && d.p < 97 && d.n_rows >= 32768) {
     if (d.n_per < 320) t = Tile{64, 48, 1};
     else if (d.p == 48 && d.n_rows >= 65536 && d.n_per >= 1024) t = Tile{256, 56, 1};

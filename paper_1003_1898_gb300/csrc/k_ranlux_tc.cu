@@ -797,6 +797,10 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tiles(const FillDesc d, 
 
 // The same for any output (unaligned rows, the fused half-sweep, host memory)
 // through a per-row ring of 56 words that the warp copies out 32 words at a time.
+// Unaligned rows are stored word by word (or double by double) from eight rows held
+// in registers: a row at a time, each load waiting for the one before, took 311 us for
+// 30,320 x 1,001 doubles at p = 223 and 222 for 131,072 x 1,001 words; now 147 and 219
+// (the borrow chain 192 and 310).
 template <int OM>
 __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int level, bool vec) {
   __shared__ __align__(128) TcTable sh;
@@ -869,15 +873,45 @@ __global__ void __launch_bounds__(128, 4) k_fill_ranlux_tc(const FillDesc d, int
                            *reinterpret_cast<const uint4*>(wrows + (fr + 4 * i) * kRowWords + 4 * ch));
           }
         }
-      } else if (lane < 4 * k) {
+      } else if (OM == OUT_ISING) {
         int w = 4 * fc + lane;
         if (w >= 4 * kRC) w -= 4 * kRC;
-        for (int i = 0; i < 32 && wrow0 + i < nr; i++) {
+        for (int i = 0; lane < 4 * k && i < 32 && wrow0 + i < nr; i++) {
           const uint64_t e = (wrow0 + i) * d.pitch + fpos + lane;
-          if constexpr (OM == OUT_F64) {
-            if (!(lane & 1)) st_pair<24>(out + e, wrows[i * kRowWords + w], wrows[i * kRowWords + w + 1]);
-          } else {
-            put1<OM>(d, out + e, e, wrows[i * kRowWords + w]);
+          put1<OM>(d, out + e, e, wrows[i * kRowWords + w]);
+        }
+      } else if constexpr (OM == OUT_F64) {   // a half-warp per row, eight steps in flight
+        const int c = 2 * (lane & 15), sub = lane >> 4;
+        int w = 4 * fc + c;
+        if (w >= 4 * kRC) w -= 4 * kRC;
+        for (int i0 = 0; i0 < 32; i0 += 16) {
+          uint2 v[8];
+#pragma unroll
+          for (int i = 0; i < 8; i++)
+            v[i] = *reinterpret_cast<const uint2*>(wrows + (i0 + 2 * i + sub) * kRowWords + w);
+          uint64_t rr = wrow0 + i0 + sub;
+          uint32_t* p = out + rr * d.pitch + fpos + c;
+#pragma unroll
+          for (int i = 0; i < 8; i++) {
+            if (c < 4 * k && rr < nr) st_pair<24>(p, v[i].x, v[i].y);
+            rr += 2;
+            p += 2 * d.pitch;
+          }
+        }
+      } else {   // a warp per row, eight in flight
+        int w = 4 * fc + lane;
+        if (w >= 4 * kRC) w -= 4 * kRC;
+        for (int i0 = 0; i0 < 32; i0 += 8) {
+          uint32_t v[8];
+#pragma unroll
+          for (int i = 0; i < 8; i++) v[i] = wrows[(i0 + i) * kRowWords + w];
+          uint64_t rr = wrow0 + i0;
+          uint32_t* p = out + rr * d.pitch + fpos + lane;
+#pragma unroll
+          for (int i = 0; i < 8; i++) {
+            if (lane < 4 * k && rr < nr) st_out(p, v[i]);
+            rr++;
+            p += d.pitch;
           }
         }
       }
