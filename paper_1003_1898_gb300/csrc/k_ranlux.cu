@@ -54,6 +54,15 @@ Tile ranlux_auto_tile(const FillDesc& d) {
     else if (d.p == 24 && d.mode != OUT_F64 && d.n_rows >= 98304 && d.n_rows <= 131072 && d.n_per >= 4096)
       t = Tile{128, 56, 1};
   }
+  // Long unaligned rows at p < 97 leave through the staged tile: in CTAs of 128 where
+  // the busiest SM holds no more threads that way (30,320 x 2,047 at p = 24 143 / 136,
+  // 50,000 x 4,095 503 / 485; but 25,000 x 2,047 100 / 118, 65,536 x 4,095 at p = 48
+  // 660 / 697, and below 28,000 streams, 16,384 x 2,047, 76 / 78).
+  if (d.out != nullptr && d.p < 97 && !ranlux_ring_ok(d) && (d.mode == OUT_U32 || d.mode == OUT_F32) &&
+      d.n_rows >= 28000 && d.n_rows < 65536 && d.n_per >= 1000) {
+    const uint64_t sms = (uint64_t)sm_count(), c64 = (d.n_rows + 63) / 64, c128 = (d.n_rows + 127) / 128;
+    if ((c64 + sms - 1) / sms == 2 * ((c128 + sms - 1) / sms)) t = Tile{128, 48, 1};
+  }
   if (d.p < kLuxTcMinP || d.n_per < 24) return t;
   const uint64_t nb = d.n_per / 24, p = (uint64_t)d.p, sms = (uint64_t)sm_count();
   auto product = [&](uint64_t tiles) {   // cycles of a product with `tiles` tiles to run
