@@ -47,10 +47,28 @@ struct prng_batcher {
   Slot slot[kSlots];
   int next = 0;
   std::vector<const prng_state*> handles;   // duplicate check, sized once
-  std::vector<uint32_t> order;              // requests, longest rows first
+  std::vector<uint64_t> order, sorted;      // requests, longest rows first: 2^32 - 1 - length, index
 };
 
 namespace {
+
+// Sorts keys whose low words are already in order, by their high words: byte by
+// byte, those that all keys share left out.  (Comparing the requests themselves
+// took a third of a launch of 1,000 short ones.)
+void sort_keys(std::vector<uint64_t>& keys, std::vector<uint64_t>& tmp) {
+  if (keys.size() < 2) return;
+  uint64_t differ = 0;
+  for (uint64_t k : keys) differ |= k ^ keys[0];
+  tmp.resize(keys.size());   // within its reserve
+  for (int shift = 32; shift < 64; shift += 8) {
+    if (((differ >> shift) & 255) == 0) continue;
+    uint32_t at[257] = {};
+    for (uint64_t k : keys) at[((k >> shift) & 255) + 1]++;
+    for (int i = 0; i < 256; i++) at[i + 1] += at[i];
+    for (uint64_t k : keys) tmp[at[(k >> shift) & 255]++] = k;
+    keys.swap(tmp);
+  }
+}
 
 void destroy_batcher(prng_batcher* b) {
   if (b == nullptr) return;
@@ -86,6 +104,7 @@ int prng_batcher_create(prng_batcher** out, uint32_t max_requests, uint64_t max_
   try {
     b->handles.reserve(max_requests);
     b->order.reserve(max_requests);
+    b->sorted.reserve(max_requests);
   } catch (...) {
     delete b;
     return PRNG_EALLOC;
@@ -217,11 +236,11 @@ int prng_batcher_launch(prng_batcher* b, const prng_fill_req* reqs, uint32_t n_r
   // the same but for the last, so ordering the requests orders the items).
   b->order.clear();
   for (uint32_t i = 0; i < n_reqs; i++)
-    if (reqs[i].n_per_stream > 0) b->order.push_back(i);
-  std::sort(b->order.begin(), b->order.end(), [&](uint32_t x, uint32_t y) {
-    return reqs[x].n_per_stream != reqs[y].n_per_stream ? reqs[x].n_per_stream > reqs[y].n_per_stream : x < y;
-  });
-  for (uint32_t i : b->order) {
+    if (reqs[i].n_per_stream > 0)
+      b->order.push_back((UINT32_MAX - std::min<uint64_t>(reqs[i].n_per_stream, UINT32_MAX)) << 32 | i);
+  sort_keys(b->order, b->sorted);
+  for (uint64_t key : b->order) {
+    const uint32_t i = (uint32_t)key;
     const prng_fill_req& r = reqs[i];
     const int f = fill_family(r.st->gen, r.st->p, r.f32 != 0);
     plan.items(f, i, r.st, r.n_per_stream, [&](const BatchItem& it) { u.h_items[at[f]++] = it; });

@@ -55,7 +55,7 @@ struct ItemPlan {
     for (int f = 0; f < FAM_COUNT; f++) lux_pays[f] = true;
     uint64_t wb[FAM_COUNT] = {}, longest[FAM_COUNT] = {};
     for (uint32_t i = 0; i < n; i++) {
-      if (reqs[i].n_per_stream == 0) continue;
+      if (reqs[i].st->gen != RANLUX || reqs[i].n_per_stream == 0) continue;
       const int f = fill_family(reqs[i].st->gen, reqs[i].st->p, reqs[i].f32 != 0);
       if (!is_lux_tc(f)) continue;
       const uint64_t nb = reqs[i].n_per_stream / 24;
