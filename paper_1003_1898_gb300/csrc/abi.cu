@@ -25,8 +25,10 @@ constexpr uint32_t kBlobVersion = 1u;
 // The launch tile of a plain fill: the caller's, or by the fill's shape.  In us,
 // u32 (f32 alike unless said), the handle's default tile / the one chosen here:
 //   XOR128, 64 staged columns instead of 32: 131,072 x 8,192 763 / 666, x 1,024
-//   111 / 94; 65,536 x 4,096 210 / 202, f64 257 / 249; not for short rows that
-//   leave a tile part empty (fused half-sweeps take such a tile site by site).
+//   111 / 94; 65,536 x 4,096 210 / 202, f64 257 / 249; not for rows that leave half
+//   of their last tile empty (40,000 x 864 28 / 31, 65,536 x 4,128 198 / 200), unless
+//   streams are very many (131,072 x 4,128 369 / 355) or pairs are (872 x 432 f64 36.8 / 34.3), nor for
+//   short ones.
 //   RANMAR, four warps per CTA instead of eight, once rows and streams are many:
 //   131,072 x 8,192 677 / 662; 131,072 x 500 71 / 77, which keeps eight.
 //   MT19937, two streams per warp once there are enough to fill the GPU so (f64
@@ -43,7 +45,9 @@ Tile fill_tile(const prng_state* st, const FillDesc& d) {
   if (!tile_chosen(st->gen, st->p)) switch (st->gen) {
     case RANLUX: return ranlux_auto_tile(d);
     case XOR128:
-      if (d.n_per % 64 == 0 || (d.n_per >= 256 && d.mode != OUT_ISING)) return Tile{128, 64, 1};
+      if (d.n_per % 64 == 0 || (d.n_per >= 256 && d.mode != OUT_ISING &&
+                                (d.n_per % 64 > 32 || d.mode == OUT_F64 || (d.n_rows >= 100352 && d.n_per >= 500))))
+        return Tile{128, 64, 1};
       break;
     case RANMAR:
       if (d.n_rows >= 32768 && d.n_per >= 4096) return Tile{128, 128, 1};
