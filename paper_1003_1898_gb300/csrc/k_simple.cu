@@ -202,10 +202,10 @@ __device__ __noinline__ void odd_tile(const FillDesc& d, const uint32_t* t, uint
 
 // Streams [row0, row0 + T) of a fill, one per thread; smem holds S tiles of
 // T * K words.  The n draws go to columns col0 .. col0 + n - 1; the states are
-// read from `from` and left in `store_to` (nullptr: nowhere).
+// read from d.state and left in `store_to` (nullptr: nowhere).
 template <class G, int T, int K, int S, int OM>
 __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, uint32_t* smem, uint64_t col0,
-                                            uint64_t n, const uint32_t* from, uint32_t* store_to) {
+                                            uint64_t n, uint32_t* store_to) {
   static_assert(K % 32 == 0, "tile rows hold whole 8-chunk swizzle groups");
   constexpr int CH = K / 4;          // 16-byte chunks per row
   constexpr int RS = T / CH;         // rows one copy-out pass of the CTA covers
@@ -219,9 +219,9 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
     g.zero();
   } else if constexpr (G::JUMPS) {
     if (d.jump) g.jump_start(d.x0, row * d.pitch);   // chunk `row` of one sequence
-    else g.load(from, d.n_rows, row);
+    else g.load(d.state, d.n_rows, row);
   } else {
-    g.load(from, d.n_rows, row);
+    g.load(d.state, d.n_rows, row);
   }
 
   uint32_t* out = static_cast<uint32_t*>(d.out);
@@ -281,20 +281,22 @@ __device__ __forceinline__ void simple_rows(const FillDesc& d, uint64_t row0, ui
 template <class G, int T, int K, int S, int OM>
 __global__ void __launch_bounds__(T) k_fill_simple(const __grid_constant__ FillDesc d) {
   extern __shared__ __align__(16) uint32_t smem[];
-  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, 0, d.n_per, d.state, d.jump ? nullptr : d.state);
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, 0, d.n_per, d.jump ? nullptr : d.state);
 }
 
 // Segment blockIdx.y of every stream: draws [seg L, seg L + L) of the call, from
 // the states that `starts` holds for it ([segment][word][stream]); the last
-// segment leaves the handle's states.
+// segment leaves the handle's states.  (Its descriptor is an ordinary parameter,
+// copied to the stack once: as a grid constant the compiler kept fewer of the
+// copy-out's loads in flight, 65,536 x 2,048 f64 215 -> 231 us.)
 template <class G, int T, int K, int S, int OM>
-__global__ void __launch_bounds__(T) k_fill_segments(const __grid_constant__ FillDesc d, const uint32_t* starts,
-                                                      uint64_t L) {
+__global__ void __launch_bounds__(T) k_fill_segments(FillDesc d, uint32_t* starts, uint64_t L) {
   extern __shared__ __align__(16) uint32_t smem[];
+  uint32_t* const state = d.state;
   const uint64_t seg = blockIdx.y, col0 = seg * L;
   const uint64_t n = d.n_per - col0 < L ? d.n_per - col0 : L;
-  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, col0, n, starts + seg * 4 * d.n_rows,
-                              seg + 1 == gridDim.y ? d.state : nullptr);
+  d.state = starts + seg * 4 * d.n_rows;
+  simple_rows<G, T, K, S, OM>(d, (uint64_t)blockIdx.x * T, smem, col0, n, seg + 1 == gridDim.y ? state : nullptr);
 }
 
 // Batched XOR128 fills: a block pops an item (T streams of one request).
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(T) k_batch_xor128(const BatchQueue q) {
     __shared__ FillDesc sd;
     load_desc(&sd, q.reqs[si.req].d, threadIdx.x, T);
     __syncthreads();
-    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem, 0, sd.n_per, sd.state, sd.state);
+    simple_rows<Xor128Gen, T, K, S, F32 ? OUT_F32 : OUT_U32>(sd, si.row0, smem, 0, sd.n_per, sd.state);
   }
 }
 
