@@ -27,8 +27,8 @@ constexpr uint32_t kBlobVersion = 1u;
 //   XOR128, 64 staged columns instead of 32: 131,072 x 8,192 763 / 666, x 1,024
 //   111 / 94; 65,536 x 4,096 210 / 202, f64 257 / 249; not for rows that leave half
 //   of their last tile empty (40,000 x 864 28 / 31, 65,536 x 4,128 198 / 200), unless
-//   streams are very many (131,072 x 4,128 369 / 355) or pairs are (872 x 432 f64 36.8 / 34.3), nor for
-//   short ones.
+//   streams are very many (131,072 x 4,128 369 / 355) or pairs are stored (872 x 432
+//   f64 36.8 / 34.3), nor for short ones.
 //   RANMAR, four warps per CTA instead of eight, once rows and streams are many:
 //   131,072 x 8,192 677 / 662; 131,072 x 500 71 / 77, which keeps eight.
 //   MT19937, two streams per warp once there are enough to fill the GPU so (f64
@@ -37,8 +37,13 @@ constexpr uint32_t kBlobVersion = 1u;
 //   ones, 8,192 x 131,072 728 / 678 (one warp 685).  But a scheduler holds whole
 //   warps, and an odd number of streams each leaves half a warp idle in the
 //   paired form: long rows then keep a warp per stream (that / paired, x 60,000:
-//   2,729 142 / 154, 4,096 186 / 194, 3,648 (even) 164 / 150), until from 14 on the
-//   half warp is lost among them (9,000 366 / 360).  A CTA per stream while they
+//   2,729 142 / 154, 4,096 186 / 194, 3,648 (even) 164 / 150; 2,683 x 8,840 27.3 /
+//   28.6, x 5,000 19.6 / 19.3), until from 14 on the
+//   half warp is lost among them (9,000 366 / 360).  Blocks that start off a 16-byte
+//   boundary are stored word by word, which many words bound: they too keep a warp
+//   per stream (pairs / that: 8,192 x 7,455 u32 78 / 55, 4,613 x 7,455 37.8 / 34.9,
+//   8,192 x 2,001 25.1 / 26.3, which stays paired; f32 8,192 x 6,001 56 / 50, x 3,001
+//   29.9 / 32.4, which stays).  A CTA per stream while they
 //   are few: 1 x 100,000 99 / 48, 456 x 65,536 71 / 49, 256 x 4,096 19 / 14, 1,024
 //   x 20,000 37 / 36, but 1,024 x 60,000 76 / 82 (800 77 / 73).
 Tile fill_tile(const prng_state* st, const FillDesc& d) {
@@ -55,9 +60,12 @@ Tile fill_tile(const prng_state* st, const FillDesc& d) {
     case MT19937:
       if (d.mode != OUT_U32 && d.mode != OUT_F32) break;
       if (d.n_per >= 512 && d.n_rows <= (d.n_per < 30000 ? 1024 : 912)) return Tile{256, 227, 1};
+      if (((d.pitch & 3) != 0 || (d.pos & 3) != 0 || (reinterpret_cast<uintptr_t>(d.out) & 15) != 0) &&
+          d.n_rows >= 2048 && d.n_rows * d.n_per >= (d.mode == OUT_U32 ? 22000000 : 40000000))
+        return Tile{128, 624, 1};
       if (d.n_rows >= 2048) {
         const uint64_t scheds = 4 * (uint64_t)sm_count(), w = (d.n_rows + scheds - 1) / scheds;
-        if (d.n_per >= 10000 && w < 14 && w % 2 == 1) return Tile{64, 624, 1};
+        if (d.n_per >= 8000 && w < 14 && w % 2 == 1) return Tile{64, 624, 1};
         return d.n_per < 20000 ? Tile{32, 624, 2} : Tile{64, 624, 2};
       }
       break;
