@@ -53,7 +53,7 @@ struct ItemPlan {
     for (int f = 0; f < FAM_COUNT; f++) lux_pays[f] = true;
     uint64_t wb[FAM_COUNT] = {}, longest[FAM_COUNT] = {}, xor_odd = 0;
     for (uint32_t i = 0; i < n; i++) {
-      if (reqs[i].st->gen == XOR128 && (((reinterpret_cast<uintptr_t>(reqs[i].d_out) >> 2) | reqs[i].n_per_stream) & 3))
+      if (reqs[i].st->gen == XOR128 && (((reinterpret_cast<uintptr_t>(reqs[i].d_out) >> 2) | reqs[i].n_per_stream) & 7))
         xor_odd += reqs[i].st->n_streams;
       if (reqs[i].st->gen != RANLUX || reqs[i].n_per_stream == 0) continue;
       const int f = fill_family(reqs[i].st->gen, reqs[i].st->p, reqs[i].f32 != 0);
@@ -62,10 +62,11 @@ struct ItemPlan {
       wb[f] += (reqs[i].st->n_streams + 31) / 32 * (nb + 1);
       longest[f] = std::max(longest[f], nb);
     }
-    // XOR128: items of 64 streams, whose tail is shorter, unless many streams' rows are
-    // unaligned, which 64-column tiles store faster (items of 64 / 128, us: 5,000
-    // requests, 131,646 such streams 4,759 / 4,443, 2,000 with 47,595 1,854 / 1,795, but
-    // 20,000 short ones with 10,689 1,660 / 1,839; aligned 2,000 1,322 / 1,355).
+    // XOR128: items of 64 streams, whose tail is shorter, unless many streams' rows
+    // start inside a 32-byte sector, which 64-column tiles store faster (items of 64 /
+    // 128, us: 2,000 requests, 42,141 such streams 1,544 / 1,524, 5,000 with 112,220
+    // 3,906 / 3,737, 20,000 with 386,965 15,235 / 14,695; but 500 with 8,456 409 / 435,
+    // 20,000 short ones with 10,158 1,554 / 1,732).
     const bool fine = cut && !tile_chosen(XOR128, 0) && xor_odd < 32768;
     tile[FAM_XOR128] = tile[FAM_XOR128 + FAM_F32] = fine ? Tile{64, 32, 1} : tile_of(FAM_XOR128);
     for (int f = 0; f < FAM_COUNT; f++) {
