@@ -203,7 +203,7 @@ typedef struct prng_batch prng_batch;
  * not be destroyed before the batch); allocates the work items, two
  * descriptor buffers and the work counters.  RANLUX fills at p >= 97 are cut
  * into items of 32 streams and, when they are long, of part of their draws,
- * whose start states the plan holds too (76 bytes per stream and part; without
+ * whose start states the plan holds too (84 bytes per stream and part; without
  * room for them these fills take the serial form).  PRNG_EBLOB if a handle
  * appears twice. */
 int prng_batch_create(prng_batch **out, const prng_fill_req *reqs, uint32_t n_reqs);

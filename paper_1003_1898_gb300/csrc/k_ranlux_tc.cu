@@ -7,7 +7,7 @@
 // integer R, X = R - (R >> 336) + carry satisfies b X_{n+1} = X_n + x_n m, so
 // X_{n+1} = b^{-1} X_n mod m.  A whole luxury cycle, p steps of which p - 24
 // are thrown away, is then one multiplication by the constant a = b^{-p} mod m,
-// whatever p is.  And since b^24 X_{n+24} = X_n + m R_{n+24}, the 24 words that
+// whatever p is (so skips RANLUX++ too, Sibidanov 2017).  And since b^24 X_{n+24} = X_n + m R_{n+24}, the 24 words that
 // follow X_n are R_{n+24} = -X_n m^{-1} mod 2^576 with m^{-1} = 1 + 2^240 +
 // 2^480 (mod 2^576): two shifted additions.
 //
@@ -693,14 +693,13 @@ __device__ __forceinline__ void lux_finish(const FillDesc& d, uint64_t row, bool
 // rows 16-byte aligned in device memory and a start that leaves a multiple of 4
 // draws in the open block: output by 32 x 32-word tile stores.
 //
-// What bounds it: neither DRAM (0.68 of the copy peak) nor the tensor core (its
-// pipe is busy a fifth of the time) but the integer work around the product,
-// about 350 instructions per 24 words of a stream (the SMs with four CTAs issue
-// on 2 of 3 cycles, the ALU pipe is 73 % busy there), and the grain of the
-// work: 65,536 streams are 3.4 CTAs per SM, so some SMs run four and the rest
-// three.  2^28 words over 65,536 streams, borrow chain -> here: p = 223 405 ->
-// 234 us u32, 410 -> 240 f32; p = 389 640 -> 233 and 645 -> 242; 131,072 x 2,048
-// at p = 389 547 -> 210.  The same product with the rows copied out of a ring
+// What bounds it: neither DRAM (0.73 of the copy peak) nor the tensor core (its
+// pipe is busy 31 % of the time) but the integer work around the product, about
+// 400 instructions per 24 words of a stream (ALU pipe 61 % busy, issue 61 %), and
+// the grain of the work: 65,536 streams are 3.4 CTAs per SM, so some SMs run four
+// and the rest three.  2^28 words over 65,536 streams, a u32 and an f32 fill
+// together, borrow chain -> here: p = 223 816 -> 451 us, p = 389 1,284 -> 451 (f32
+// alone 654 -> 219).  The same product with the rows copied out of a ring
 // by the warps (k_fill_ranlux_tc below) took 320 us: 100 more instructions per
 // block.  Moving the funnel shifts to the FMA pipe (multiplies by 2^16 and their
 // high halves) was slower (224 -> 238 us).

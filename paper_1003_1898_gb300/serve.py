@@ -83,7 +83,10 @@ class Server:
         is what bounds the loop at saturation, so more half-sweeps per tick
         raise throughput; with clients of 4,096 streams they lowered the
         latency at moderate load too (4 against 1: p50/p99 1.8/9.2 against
-        3.0/13.6 ms at 2,000 requests/s).  scan_limit: pending requests
+        3.0/13.6 ms at 2,000 requests/s).  mem_cap counts
+        states, lattices, draws and outputs; the library's own scratch (four
+        launches' descriptors and work items, and RANLUX segment starts from a
+        pool that keeps 1 GiB at most) lies outside it.  scan_limit: pending requests
         examined for admission per tick (in arrival order); the rest wait,
         so the host work of a tick stays bounded when the queue is long."""
         import torch
